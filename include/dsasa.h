@@ -101,8 +101,8 @@ typedef struct {
                          * update of the complex across MD steps (the paper's Conclusions).  The
                          * simplices of the complex are the same as a fresh build's, the areas
                          * and gradient equal up to the rounding of the terms.  0: off; 1
-                         * (default): for molecules of more than one wave of the fused cell
-                         * kernel (about 5,400 atoms on a GB300), where it pays; 2: always. */
+                         * (default): for molecules of more than 36 atoms per
+                         * multiprocessor (5,472 on a GB300), where it pays; 2: always. */
 } dsasa_config;
 
 /* Fills cfg with defaults: MIXED, skin 0, grow on demand, default cell cap, carry 1 (auto). */
@@ -251,9 +251,9 @@ dsasa_status dsasa_deferred_count(dsasa_ctx* ctx, int64_t* deferred);
  * to *calls_out (may be NULL), and resets the sums.  Phases: */
 #define DSASA_NPHASE 5
 #define DSASA_PHASE_CELL_LIST 0   /* cell-list build (input pass, grid, scan, scatter) */
-#define DSASA_PHASE_CELL 1        /* restricted power cell per atom (gather, sort, clipping); when
-                                     all atoms fit one wave of the GPU this kernel also classifies,
-                                     and DSASA_PHASE_CLASSIFY is (near) zero */
+#define DSASA_PHASE_CELL 1        /* restricted power cell per atom (gather, sort, clipping); on
+                                     small molecules this kernel also classifies, and
+                                     DSASA_PHASE_CLASSIFY is (near) zero */
 #define DSASA_PHASE_CLASSIFY 2    /* simplices of the cell in C (Steps 2a-2c) */
 #define DSASA_PHASE_TERMS 3       /* area terms and gradient gathers */
 #define DSASA_PHASE_LARGE 4       /* the large-capacity pass over deferred atoms */

@@ -130,7 +130,7 @@ class Context:
         cfg.skin = float(skin)
         cfg.max_atoms = int(max_atoms)
         cfg.max_cells = int(max_cells)
-        cfg.carry = int(carry)   # 0 off, 1 beyond one wave of the fused cell kernel, 2 always
+        cfg.carry = int(carry)   # 0 off, 1 beyond 36 atoms per multiprocessor, 2 always
         self.device = device
         h = _vp()
         st = _lib.dsasa_create(ctypes.byref(h), device, _vp(self._stream_handle(stream)), ctypes.byref(cfg))

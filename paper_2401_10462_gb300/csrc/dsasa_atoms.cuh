@@ -22,9 +22,9 @@
 // table) and in registers (each lane caches the homogeneous coordinates of up to NT / 32
 // cell vertices).  The fast path runs the steps as separate kernels that hand the cell over
 // through a per-atom record in HBM (PH_CELL: Step 1; PH_CLASS: Step 2; PH_TERMS: Step 3;
-// PH_VOL: the volume), so that each kernel's code fits the instruction cache.  When all atoms
-// fit in one wave, Steps 1 and 2 run as one kernel (PH_CC), so that classifications overlap
-// the slowest cells.  With carried cells, Step 1 is PH_CARRY (on calls reusing the neighbour
+// PH_VOL: the volume), so that each kernel's code fits the instruction cache.  On small
+// molecules Steps 1 and 2 run as one kernel (PH_CC, cells_fused), so that classifications
+// overlap the slowest cells.  With carried cells, Step 1 is PH_CARRY (on calls reusing the neighbour
 // lists, each atom's cell from the previous call, kept when exact predicates certify it) and
 // then PH_CELL over the atoms it could not keep.  The fused form (PH_ALL) serves the
 // large-capacity pass and the no-allocation entry point.
@@ -46,13 +46,16 @@ constexpr uint8_t NONE = 0xff;
 // and terms kernels
 constexpr int WARPS = 1, WARPS_CELL = 2, WARPS_CLASS = 2, WARPS_TERMS = 2;
 // resident blocks per SM that each kernel's register budget is sized for (one warp each)
-constexpr int MINB = 32, MINB_CELL = 18, MINB_CLASS = 18, MINB_TERMS = 18;
+// (the cell kernels: 64 registers and 32 warps an SM; 20,003-atom globule 176 us, against 186 at
+// 18 blocks of 56 registers, 182 at 14, 194 at 12 and 251 at 21)
+constexpr int MINB = 32, MINB_CELL = 16, MINB_CLASS = 18, MINB_TERMS = 18;
 
 // kernel phases: the whole computation in one kernel, or three kernels that pass the cell
 // through a global record per atom: the cell construction (gather, sort, clipping), the
 // classification (Steps 2a-2c: which simplices of the cell are in C), and the area terms and
 // gradient.  Each kernel's code then fits the instruction cache.
 enum { PH_ALL = 0, PH_CELL = 1, PH_CLASS = 2, PH_TERMS = 3, PH_VOL = 4, PH_CC = 5, PH_CARRY = 6 };
+template <int N> struct IntC { static constexpr int value = N; };
 enum { CELL_OK = 0, CELL_DONE = 1 };   // record flag: CELL_DONE = outputs already written
 
 // Per-warp cell storage.  NE plane entries (0..5 ghosts, then the candidates in sorted
@@ -63,11 +66,11 @@ template <class R, int NE, int NT> struct Smem {
     using Real = R;
     static constexpr int kNE = NE, kNT = NT;
     alignas(16) R pq[NE][4];   // plane q.x, q.y, q.z, b (relative to p_i)
-    R pB[NE];             // magnitude proxy of b for the filters
+    R pm[NE][2];          // filter magnitudes: |q|_1 rounded up (cell kernels only), and of b
     int pg[NE];           // global atom index (>= 0) or -1 - ghost id
     uint8_t start[NE];    // a vertex slot on the face of this plane
-    // boundary edges of the current cut, by number: (a, b, kept neighbour slot, new slot, edge
-    // index in the kept neighbour) packed 7/7/7/7/2 bits; the new slot by first and last plane
+    // boundary edges of the current cut, by number: planes a, b and the kept neighbour's slot,
+    // one byte each; the new vertex on the edge that ends at plane b
     unsigned bedge[NE];
     uint8_t bslot[NE], eslot[NE];
     uint8_t ord[NE];      // clipping order (entry ids)
@@ -79,10 +82,8 @@ template <class R, int NE, int NT> struct Smem {
     unsigned tf[NT];      // bit k: the triangle of edge k is in C; bit 4+k: it is processed here
     unsigned skey[NE];    // orderable sort key of each candidate
     uint16_t tl[NT * 3 / 2 + 2];   // compacted exterior triangles (slot << 2 | edge)
-    uint8_t rem[NT];
-    uint8_t rsl[NT];      // removed slots in order
-    uint8_t fs[NT];       // free slot stack
-    int hw, nfree, bad;
+    uint8_t rem[NT];      // carried cells: start slots on the way to start[]
+    int hw, bad;
 };
 
 // The cell of one atom between the two kernels (first NG + nc plane entries, first hw
@@ -203,9 +204,6 @@ template <> struct GAcc<double> {
     }
 };
 __device__ __forceinline__ uint8_t tv_get(const uchar4& v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : v.z); }
-template <class SM> __device__ __forceinline__ void ta_set(SM* S, int t, int k, uint8_t s) {
-    ((uint8_t*)&S->ta[t & (SM::kNT - 1)])[k] = s;
-}
 
 // ------------------------------------------------------------------ global plane access
 struct Ctx {
@@ -312,7 +310,7 @@ template <class SM, class R = typename SM::Real> __device__ __forceinline__ Plan
     e &= SM::kNE - 1;
     PlaneN<FA<R>> P;
     P.q = {{S->pq[e][0], fabs(S->pq[e][0])}, {S->pq[e][1], fabs(S->pq[e][1])}, {S->pq[e][2], fabs(S->pq[e][2])}};
-    P.b = {S->pq[e][3], S->pB[e]};
+    P.b = {S->pq[e][3], S->pm[e][1]};
     return P;
 }
 // homogeneous cell vertex (Dv, D) of the planes of triangle v, with magnitudes for the filter
@@ -323,6 +321,25 @@ template <class SM, class R = typename SM::Real> __device__ __forceinline__ VtxF
     FA<R> D;
     vertex_hom(Pa, Pb, Pc, Dv, D);
     return {{Dv.x.v, Dv.y.v, Dv.z.v, D.v}, {Dv.x.a, Dv.y.a, Dv.z.a, D.a}};
+}
+// A new cell vertex of a cut: the planes A, B of a boundary edge and the cutting plane M (rows
+// q, b and magnitudes |q|_1, |b| of the shared table).  Vs bounds the sum of the four filter
+// magnitudes (vertex_hom on absolute values) from above: each product of two components is a
+// term of a product of 1-norms, so the magnitudes sum to at most
+//   n_B n_M b_A + n_M n_A b_B + n_A n_B b_M + n_A n_B n_M,
+// 10 operations instead of the 33 of the magnitudes themselves.  It is about twice their sum;
+// a clip test that it leaves open is decided again with the magnitudes (rare: fewer than one
+// in 20 atoms of a globule meets one).
+__device__ __forceinline__ void new_vertex(const float4 A, const float2 am, const float4 B, const float2 bm,
+                                           const float4 M, const float2 mm, float* V, float& Vs) {
+    const P3<float> qa = {A.x, A.y, A.z}, qb = {B.x, B.y, B.z}, qm = {M.x, M.y, M.z};
+    const P3<float> xbm = cross3(qb, qm), xma = cross3(qm, qa), xab = cross3(qa, qb);
+    V[0] = xbm.x * A.w + xma.x * B.w + xab.x * M.w;
+    V[1] = xbm.y * A.w + xma.y * B.w + xab.y * M.w;
+    V[2] = xbm.z * A.w + xma.z * B.w + xab.z * M.w;
+    V[3] = dot3(qa, xbm);
+    const float nab = am.x * bm.x, nam = am.x * mm.x, nbm = bm.x * mm.x;
+    Vs = (nbm * am.y + nam * bm.y + nab * (mm.y + mm.x)) * 1.000001f;
 }
 // out of line (the kernels that also classify or evaluate terms keep their code small)
 template <class SM, class R = typename SM::Real> __device__ __noinline__ VtxFA<R> vertex_fa(const SM* S, uchar4 v) {
@@ -449,6 +466,33 @@ __device__ __noinline__ int psign(const SM* S, const Ctx& c, const FA<R>& wi, in
     return resolve_exact(c, kind, S->pg[e0 & M], S->pg[e1 & M], S->pg[e2 & M], S->pg[e3 & M], Gam<R>::try64);
 }
 
+// the clip test of cell vertex tv (three plane ids) against plane m that the loose filter left
+// open: the filter with its magnitudes, then the slow path (cold: out of line, and the centre
+// atom's data is fetched here so that no caller keeps it)
+template <class SM, class R = typename SM::Real>
+__device__ __noinline__ int clip_sign(const SM* S, const double* xyz, const double* Ra, int i, int n, int* status,
+                                      unsigned tv, int m) {
+    const uchar4 v = make_uchar4((uint8_t)tv, (uint8_t)(tv >> 8), (uint8_t)((tv >> 16) & 127u), 0);
+    const PlaneN<FA<R>> M = fplane(S, m);
+    const VtxFA<R> q = vertex_fa_inl(S, v);
+    FA<R> sv;
+    sv.v = M.q.x.v * q.v[0] + M.q.y.v * q.v[1] + M.q.z.v * q.v[2] - M.b.v * q.v[3];
+    sv.a = M.q.x.a * q.a[0] + M.q.y.a * q.a[1] + M.q.z.a * q.a[2] + M.b.a * q.a[3];
+    const int sg = fa_sign(sv, Gam<R>::gclip, Gam<R>::tiny);
+    if (sg != 0) return sg;
+    Ctx c;
+    c.xyz = xyz;
+    c.R = Ra;
+    for (int k = 0; k < 3; ++k) c.pi[k] = xyz[3 * i + k];
+    c.Ri = Ra[i];
+    c.h = ghost_h(c.Ri);
+    c.i = i;
+    c.n = n;
+    c.status = status;
+    constexpr int MK = SM::kNE - 1;
+    return resolve_exact(c, PK_CLIP, S->pg[v.x & MK], S->pg[v.y & MK], S->pg[v.z & MK], S->pg[m & MK], Gam<R>::try64);
+}
+
 // the filter alone (inline): the certified sign, or 0 when the filter leaves it open
 template <int KIND, class SM, class R = typename SM::Real>
 __device__ __forceinline__ int fsign(const SM* S, const FA<R>& wi, int e0, int e1, int e2 = 0) {
@@ -489,6 +533,21 @@ static_assert(CUBE_ADJ0 == 0x0302010007060504ull && CUBE_ADJ1 == 0x0507040602000
                   CUBE_ADJ2 == 0x0604070501030002ull,
               "every edge of the cube's triangulation has exactly one neighbour across it");
 
+// The planes of every corner, one byte per corner.
+__host__ __device__ constexpr unsigned long long cube_planes(int k) {
+    unsigned long long packed = 0;
+    for (int t = 0; t < 8; ++t) packed |= (unsigned long long)cube_corner_plane(t, k) << (8 * t);
+    return packed;
+}
+constexpr unsigned long long CUBE_PL0 = cube_planes(0), CUBE_PL1 = cube_planes(1), CUBE_PL2 = cube_planes(2);
+
+// Cell vertices and their neighbours as registers: three bytes x, y, z in one word (dead: NONE).
+constexpr unsigned DEADV = 0x00ffffffu;
+__device__ __forceinline__ unsigned pack3(unsigned x, unsigned y, unsigned z) { return x | y << 8 | z << 16; }
+__device__ __forceinline__ uchar4 unpack3(unsigned w) {
+    return make_uchar4((uint8_t)w, (uint8_t)(w >> 8), (uint8_t)(w >> 16), 0);
+}
+
 // ------------------------------------------------------------------ carried cells
 // The incremental update of C across MD steps.  On a call that reuses the neighbour lists
 // (every atom within half the skin of its last rebuild), the cell that the previous call
@@ -517,10 +576,9 @@ static_assert(CUBE_ADJ0 == 0x0302010007060504ull && CUBE_ADJ1 == 0x0507040602000
 // triangles pointing at each other with the edge reversed, every face's start slot on that
 // face, V = 2F - 4 for the closed triangulation of a sphere), renumbers the faces NG.. in
 // record order with the other candidates after them, and sets up the shared tables:
-// triangles, adjacency, free slots (the dead slots below the high-water mark), the test order
-// (ghost faces, faces, other candidates) and each face's start slot, staged in rem[] for the
-// caller.  It returns nc | ncert << 8 | nclip << 16 | nalive << 24, or 0 when the record
-// gives no usable structure.
+// triangles, adjacency, the test order (ghost faces, faces, other candidates) and each face's
+// start slot, staged in rem[] for the caller.  It returns nc | ncert << 8 | nclip << 16 |
+// nalive << 24, or 0 when the record gives no usable structure.
 template <class SM, class RC>
 __device__ __noinline__ int carry_cell(SM* S, const RC* rec, int i, int n, int nc, int lane) {
     constexpr int NE = SM::kNE, NT = SM::kNT, KMAX = NE - NG;
@@ -646,23 +704,13 @@ __device__ __noinline__ int carry_cell(SM* S, const RC* rec, int i, int n, int n
         if (gf) S->ord[__popc(bg & lanemask_lt())] = (uint8_t)lane;
     }
     for (int k = lane; k < ncn; k += 32) S->ord[ngf + k] = (uint8_t)(NG + k);
-    // triangles in the new numbering; the dead slots below the high-water mark are free
-    int nfree = 0;
-    for (int t0 = 0; t0 < hwo; t0 += 32) {
-        const int t = t0 + lane;
-        bool dead = false;
-        if (t < hwo) {
-            const uchar4 v = S->tv[t];
-            if (v.x == NONE) dead = true;
-            else S->tv[t] = make_uchar4(S->eslot[v.x], S->eslot[v.y], S->eslot[v.z], 0);
-        }
-        const unsigned bd = __ballot_sync(FULL, dead);
-        if (dead) S->fs[nfree + __popc(bd & lanemask_lt())] = (uint8_t)t;
-        nfree += __popc(bd);
+    // triangles in the new numbering
+    for (int t = lane; t < hwo; t += 32) {
+        const uchar4 v = S->tv[t];
+        if (v.x != NONE) S->tv[t] = make_uchar4(S->eslot[v.x], S->eslot[v.y], S->eslot[v.z], 0);
     }
     if (lane == 0) {
         S->hw = hwo;
-        S->nfree = nfree;
         S->bad = 0;
     }
     __syncwarp();
@@ -953,7 +1001,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
         // an atom whose record gives no usable structure, or whose carried cell is not certified
         // or is cut by a new candidate, goes to the redo list
         constexpr bool carried = CARRY;
-        int ncert = 0, nclip = nc;   // planes that certify the carried cell; the other candidates
+        int ncert = 0, nclip = 0;   // planes that certify the carried cell; all planes it is tested against
         if constexpr (CARRY) {
             const int cc = carry_cell(S, rec, i, A.n, nc, lane);
             if (cc == 0) { redo(); continue; }
@@ -976,8 +1024,9 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             S->pq[e][3] = (R)b;
             // magnitude proxy of b in float: |b_f| (1 + 2^-22) + 2^-26 babs, rounded up (the float
             // evaluation loses at most 2 ulp, covered by the larger factors)
-            if (sizeof(R) == 4) S->pB[e] = (R)(fabsf((float)b) * 1.0000003f + (float)babs * 1.5e-8f);
-            else S->pB[e] = (R)(ex ? fabs(b) : 8.0 * babs);
+            if (sizeof(R) == 4) S->pm[e][1] = (R)(fabsf((float)b) * 1.0000003f + (float)babs * 1.5e-8f);
+            else S->pm[e][1] = (R)(ex ? fabs(b) : 8.0 * babs);
+            S->pm[e][0] = (R)((fabsf((float)q[0]) + fabsf((float)q[1]) + fabsf((float)q[2])) * 1.000001f);
             S->start[e] = NONE;
             if (e >= NG) {
                 // sort key: signed distance of the bisector from p_i (ties: atom index)
@@ -1045,7 +1094,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
         // renumber the candidate planes in sorted order, so that every later summation
         // order depends only on the geometry (not on the order atoms sit in their cells)
         {
-            R tq[SPL][4], tb[SPL];
+            R tq[SPL][4], tb[SPL][2];
             int tg[SPL];
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
@@ -1053,7 +1102,8 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 if (e < nc) {
                     int src = pay[r] & (NE - 1);
                     for (int k = 0; k < 4; ++k) tq[r][k] = S->pq[src][k];
-                    tb[r] = S->pB[src];
+                    tb[r][0] = S->pm[src][0];
+                    tb[r][1] = S->pm[src][1];
                     tg[r] = S->pg[src];
                 }
             }
@@ -1063,55 +1113,39 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 int e = r * 32 + lane;
                 if (e < nc) {
                     for (int k = 0; k < 4; ++k) S->pq[NG + e][k] = tq[r][k];
-                    S->pB[NG + e] = tb[r];
+                    S->pm[NG + e][0] = tb[r][0];
+                    S->pm[NG + e][1] = tb[r][1];
                     S->pg[NG + e] = tg[r];
-                    S->ord[e] = (uint8_t)(NG + e);
                 }
             }
             __syncwarp();
         }
 
         // ---------------- initial cell: the cube of the 6 ghost planes (8 vertices)
-        for (int t = lane; t < NT; t += 32) {
-            uchar4 v = make_uchar4(NONE, NONE, NONE, 0);
-            if (t < 8)
-                v = make_uchar4((uint8_t)cube_corner_plane(t, 0), (uint8_t)cube_corner_plane(t, 1),
-                                (uint8_t)cube_corner_plane(t, 2), 0);
-            S->tv[t] = v;
-            S->rem[t] = 0;
-            S->kf[t] = 0;
-            S->tf[t] = 0;
-        }
-        if (lane == 0) { S->hw = 8; S->nfree = 0; S->bad = 0; }
-        if (lane < 8) {
-            const int sh = 8 * lane;
-            S->ta[lane] = make_uchar4((uint8_t)(CUBE_ADJ0 >> sh), (uint8_t)(CUBE_ADJ1 >> sh), (uint8_t)(CUBE_ADJ2 >> sh), 0);
-        }
         if (lane < NG) S->start[lane] = (lane & 1) ? 7 : 0;   // +x,+y,+z at corner 0; -x,-y,-z at 7
+        if (lane == 0) S->bad = 0;
         __syncwarp();
         } else {
-            // the carried faces' start slots (staged by carry_cell), the clipping marks cleared
+            // the carried faces' start slots (staged by carry_cell)
             for (int e = lane; e < NG + nc; e += 32) S->start[e] = S->rem[e];
-            __syncwarp();
-            for (int t = lane; t < NT; t += 32) S->rem[t] = 0;
             __syncwarp();
         }
 
-        const int hw0 = carried ? S->hw : 8;
-        nrounds = (hw0 + 31) >> 5;
-#pragma unroll
-        for (int r = 0; r < SPL; ++r) {
-            int t = r * 32 + lane;
-            if (t < hw0 && (!CARRY || S->tv[t].x != NONE)) { compute_vertex(r, t); alive |= 1u << r; }
-        }
         bool empty = false;
-        int nalive = 8;      // live cell vertices (warp-uniform)
+        unsigned TV[SPL], TA[SPL];   // the cell's vertices and their neighbours (not in PH_CARRY)
         if constexpr (CARRY) {
             // the certification: (i) every carried vertex has a certified positive orientation;
             // (ii) every face plane keeps every vertex not on it strictly inside.  The new
             // candidates are tested in the same sweep (planes outer, the lane's vertices inner,
             // one warp vote at the end): one that removes a vertex sends the atom to the redo list,
             // and so does any test that the FP32 (FP64) filter leaves open
+            const int hw0 = S->hw;
+            nrounds = (hw0 + 31) >> 5;
+#pragma unroll
+            for (int r = 0; r < SPL; ++r) {
+                int t = r * 32 + lane;
+                if (t < hw0 && S->tv[t].x != NONE) { compute_vertex(r, t); alive |= 1u << r; }
+            }
             bool fail = false, cut = false;
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
@@ -1147,178 +1181,207 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             if (__any_sync(FULL, fail || cut)) { redo(); continue; }
         }
 
-        // ---------------- clipping by the sorted neighbour planes.  The loop makes no call on
-        // the clip tests: a test that the filter leaves open ends the inner loop, that plane's
-        // tests are resolved outside it (tight magnitudes, then exact predicates), and the loop
-        // resumes at the same plane with the resolved signs.  (A call inside the loop made the
-        // compiler keep the loop's state in local memory.)
+        // ---------------- clipping by the sorted neighbour planes.  Slot t = 32 r + lane of the
+        // cell lives in lane t's registers: its planes TV, its neighbours TA, its homogeneous
+        // coordinates V and their filter magnitude.  A cut is then
+        //   * the ballot of the removed vertices; every lane tests its neighbours' bits in it;
+        //   * each removed vertex puts its boundary edges (a neighbour is kept) into shared
+        //     memory under their number (a prefix sum over two ballots);
+        //   * the lane that owns the slot of boundary edge e - the e-th removed slot, then the
+        //     slots on top of the free stack - fetches it and publishes its slot under the
+        //     edge's two planes; that is also how a kept vertex finds its new neighbour;
+        //   * the new vertices' lanes compute their coordinates, all of them at once.
+        // Free slots are a stack whose positions live with the slots (in TV): slot t starts at
+        // position 7 - t (the slots past the cube's 8, lowest on top), sp is the position above
+        // the top, and 8 - sp vertices are alive.
+        // The loop runs with one slot per lane (NR = 1) until a cut needs slot 32, which most
+        // cells never do, and goes on from there with NT / 32: the common loop then holds one
+        // vertex per lane in registers and tests one word of removed bits.
         if constexpr (!CARRY) {
-        int kk = 0;
-        unsigned rsv = 0;          // removal bits of plane kk resolved outside the loop
-        bool resolved = false, open_tests = false;
-        for (;;) {
-        for (; kk < nclip && !empty; ++kk) {
-            const int m = S->ord[kk] & (NE - 1);
-            unsigned remv = 0;
-            if (resolved) {
-                remv = rsv;
-                resolved = false;
-            } else {
-                const PlaneN<FA<R>> M = fplane(S, m);
-                // sum_k |q_k| a_k <= max_k |q_k| * sum_k a_k: the loose magnitude of the clip test
-                const R qmax = fmax(fmax(M.q.x.a, M.q.y.a), fmax(M.q.z.a, M.b.a));
-                bool open = false;
+        constexpr unsigned ALIVE = 0x80000000u;   // TV: a live vertex (else the slot's stack position)
+        const unsigned lt = lanemask_lt();
+        int hw = 8, sp = 0;   // slots used so far, free-stack pointer
 #pragma unroll
-                for (int r = 0; r < SPL; ++r) {
-                    if (r >= nrounds) break;
-                    if (!(alive >> r & 1)) continue;
-                    FA<R> sv;
-                    sv.v = M.q.x.v * V[r][0] + M.q.y.v * V[r][1] + M.q.z.v * V[r][2] - M.b.v * V[r][3];
-                    if constexpr (LOOSE) sv.a = qmax * Vs[r];
-                    else sv.a = M.q.x.a * Va[r][0] + M.q.y.a * Va[r][1] + M.q.z.a * Va[r][2] + M.b.a * Va[r][3];
-                    const int sg = fa_sign(sv, Gam<R>::gclip, Gam<R>::tiny);
-                    if (sg > 0) remv |= 1u << r;
-                    else if (sg == 0) open = true;
+        for (int r = 0; r < SPL; ++r) {
+            TV[r] = (unsigned)(1024 + 7 - (r * 32 + lane));
+            TA[r] = 0;
+        }
+        // the coordinates of the vertex on planes a, b (bytes of w) and m
+        auto make_vertex = [&](int r, unsigned w, int m) {
+            const int a = w & 255u, b = (w >> 8) & 255u;
+            if constexpr (LOOSE) {
+                new_vertex(*(const float4*)S->pq[a], *(const float2*)S->pm[a], *(const float4*)S->pq[b],
+                           *(const float2*)S->pm[b], *(const float4*)S->pq[m], *(const float2*)S->pm[m], V[r], Vs[r]);
+            } else {
+                const VtxFA<R> q = vertex_fa(S, make_uchar4((uint8_t)a, (uint8_t)b, (uint8_t)m, 0));
+                for (int k = 0; k < 4; ++k) {
+                    V[r][k] = q.v[k];
+                    Va[r][k] = q.a[k];
+                }
+            }
+        };
+        if (lane < 8) {
+            const int sh = 8 * lane;
+            TV[0] = ALIVE | pack3((unsigned)(CUBE_PL0 >> sh) & 255u, (unsigned)(CUBE_PL1 >> sh) & 255u,
+                                  (unsigned)(CUBE_PL2 >> sh) & 255u);
+            TA[0] = pack3((unsigned)(CUBE_ADJ0 >> sh) & 255u, (unsigned)(CUBE_ADJ1 >> sh) & 255u,
+                          (unsigned)(CUBE_ADJ2 >> sh) & 255u);
+            make_vertex(0, TV[0], (TV[0] >> 16) & 127u);
+        }
+        int kk = 0;
+        // clips by planes kk .. nc - 1 with NR slots per lane; true: a cut needs more slots
+        auto clip = [&](auto nrc) -> bool {
+        constexpr int NR = decltype(nrc)::value;
+        unsigned rsv = 0;          // removal bits of plane kk resolved outside the inner loop; bit 31: valid
+        for (;;) {
+        bool open_tests = false;
+        for (; kk < nc; ++kk) {
+            const int m = NG + kk;
+            unsigned remv = 0;
+            if (rsv) {
+                remv = rsv & ~ALIVE;
+                rsv = 0;
+            } else {
+                bool open = false;
+                if constexpr (LOOSE) {
+                    // |q . Dv - b D| errs by at most gamma times the sum of its magnitudes, which
+                    // is at most max(|q|_1, |b|) Vs; the floor stands for underflow
+                    const float4 M = *(const float4*)S->pq[m];
+                    const float2 mm = *(const float2*)S->pm[m];
+                    const float qm = fmaxf(mm.x, mm.y) * Gam<R>::gclip;
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) {
+                        const float sv = M.x * V[r][0] + M.y * V[r][1] + M.z * V[r][2] - M.w * V[r][3];
+                        const float lim = fmaf(qm, Vs[r], Gam<R>::tiny);
+                        const bool on = (int)TV[r] < 0;
+                        if (on && sv > lim) remv |= 1u << r;
+                        if (on && !(fabsf(sv) > lim)) open = true;
+                    }
+                } else {
+                    const PlaneN<FA<R>> M = fplane(S, m);
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) {
+                        if ((int)TV[r] >= 0) continue;
+                        FA<R> sv;
+                        sv.v = M.q.x.v * V[r][0] + M.q.y.v * V[r][1] + M.q.z.v * V[r][2] - M.b.v * V[r][3];
+                        sv.a = M.q.x.a * Va[r][0] + M.q.y.a * Va[r][1] + M.q.z.a * Va[r][2] + M.b.a * Va[r][3];
+                        const int sg = fa_sign(sv, Gam<R>::gclip, Gam<R>::tiny);
+                        if (sg > 0) remv |= 1u << r;
+                        else if (sg == 0) open = true;
+                    }
                 }
                 open_tests = __any_sync(FULL, open);
                 if (open_tests) break;
             }
-            unsigned bal[SPL];
+            unsigned bal[NR];
             int nrem = 0;
 #pragma unroll
-            for (int r = 0; r < SPL; ++r) {
-                bal[r] = r < nrounds ? __ballot_sync(FULL, remv >> r & 1) : 0u;
+            for (int r = 0; r < NR; ++r) {
+                bal[r] = __ballot_sync(FULL, remv >> r & 1);
                 nrem += __popc(bal[r]);
             }
             if (nrem == 0) continue;
-            if (nrem == nalive) { empty = true; break; }
-            // the ordered list of removed slots (round-major)
-            int before = 0;
-#pragma unroll
-            for (int r = 0; r < SPL; ++r) {
-                if (r >= nrounds) break;
-                int t = r * 32 + lane;
-                if (remv >> r & 1) S->rsl[before + __popc(bal[r] & lanemask_lt())] = (uint8_t)t;
-                before += __popc(bal[r]);
-            }
-            auto removed = [&](int t2) -> bool {   // slot t2 removed by this cut (ballot bits)
+            if (nrem == 8 - sp) { empty = true; break; }
+            auto removed = [&](unsigned t2) -> unsigned {   // bit 0: slot t2 removed by this cut
                 unsigned w = bal[0];
 #pragma unroll
-                for (int r = 1; r < SPL; ++r)
-                    if ((t2 >> 5) == r) w = bal[r];
-                return (w >> (t2 & 31)) & 1u;
+                for (int r = 1; r < NR; ++r)
+                    if ((t2 >> 5) == (unsigned)r) w = bal[r];
+                return w >> (t2 & 31u);
             };
-            __syncwarp();
-            // boundary edges of the removed region, one lane per edge of a removed triangle:
-            // edge (a -> b) whose neighbour is kept; the new face m gets the triangle (a, b, m)
-            // in the slot of boundary edge number e (the e-th removed slot, then free slots)
-            const int hw = S->hw, nfree = S->nfree;
+            // the removed neighbours of each vertex, and the boundary edges of the removed region:
+            // edge (a -> b) of a removed triangle whose neighbour is kept
+            unsigned nbr[NR];
             int nb = 0;
-            for (int c0 = 0; c0 < 3 * nrem; c0 += 32) {
-                const int e3 = c0 + lane;
-                bool isb = false;
-                uint8_t a = 0, b = 0, t2 = 0, k2 = 0;
-                if (e3 < 3 * nrem) {
-                    const int t = S->rsl[e3 / 3], k = e3 - 3 * (e3 / 3);
-                    const uchar4 v = S->tv[t], adj = S->ta[t];
-                    t2 = tv_get(adj, k) & (NT - 1);
-                    if (!removed(t2)) {
-                        isb = true;
-                        a = tv_get(v, k) & (NE - 1);
-                        b = tv_get(v, (k + 1) % 3) & (NE - 1);
-                        const uchar4 adj2 = S->ta[t2];
-                        k2 = adj2.x == t ? 0 : (adj2.y == t ? 1 : 2);
-                    }
-                }
-                const unsigned bb = __ballot_sync(FULL, isb);
-                if (isb) {
-                    const int e = nb + __popc(bb & lanemask_lt());
-                    int slot;
-                    if (e < nrem) slot = S->rsl[e];
-                    else {
-                        int x = e - nrem;
-                        slot = x < nfree ? S->fs[nfree - 1 - x] : hw + (x - nfree);
-                    }
-                    S->bedge[e & (NE - 1)] = (unsigned)a | ((unsigned)b << 7) | ((unsigned)t2 << 14) |
-                                             ((unsigned)(slot & 127) << 21) | ((unsigned)k2 << 28);
-                    S->bslot[a] = (uint8_t)slot;   // the new triangle on the edge that starts at a
-                    S->eslot[b] = (uint8_t)slot;   // ... and ends at b
-                }
-                nb += __popc(bb);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const unsigned ta = TA[r];
+                nbr[r] = (removed(ta & 255u) & 1u) | (removed((ta >> 8) & 255u) & 1u) << 1 |
+                         (removed(ta >> 16) & 1u) << 2;
+                const unsigned f = (remv >> r & 1) ? (~nbr[r] & 7u) : 0u;
+                const int cnt = __popc(f);
+                const unsigned c0 = __ballot_sync(FULL, cnt & 1), c1 = __ballot_sync(FULL, cnt & 2);
+                int e = nb + __popc(c0 & lt) + 2 * __popc(c1 & lt);
+                nb += __popc(c0) + 2 * __popc(c1);
+                if (f & 1u) S->bedge[e++ & (NE - 1)] = __byte_perm(TV[r], ta, 0x3410);
+                if (f & 2u) S->bedge[e++ & (NE - 1)] = __byte_perm(TV[r], ta, 0x3521);
+                if (f & 4u) S->bedge[e & (NE - 1)] = __byte_perm(TV[r], ta, 0x3602);
             }
-            const int extra = nb - nrem;
-            if (hw + max(0, extra - nfree) > NT || nb > NE) {
-                __syncwarp();
+            const int sp2 = sp + nrem - nb, hw2 = max(hw, 8 - sp2);
+            if (hw2 > 32 * NR && NR < SPL) return true;
+            if (hw2 > NT || nb > NE) {
                 if (lane == 0) S->bad = 2;
-                __syncwarp();
                 break;
             }
             __syncwarp();
-            for (int e = lane; e < nb; e += 32) {
-                const unsigned w = S->bedge[e];
-                const uint8_t a = w & 127, b = (w >> 7) & 127, t2 = (w >> 14) & 127;
-                const int sl = (w >> 21) & (NT - 1);
-                S->tv[sl] = make_uchar4(a, b, (uint8_t)m, 0);
-                S->ta[sl] = make_uchar4(t2, S->bslot[b & (NE - 1)], S->eslot[a & (NE - 1)], 0);
-                ta_set(S, t2, (w >> 28) & 3, (uint8_t)sl);
-                S->start[a] = (uint8_t)sl;
-                S->rem[sl] = 2;
-            }
-            if (lane == 0) S->start[m] = (uint8_t)((S->bedge[0] >> 21) & (NT - 1));
-            __syncwarp();
-            // leftover removed slots become free; update the slot allocator
-            if (extra < 0) {
-                for (int y = lane; y < -extra; y += 32) {
-                    int sl = S->rsl[nb + y];
-                    S->tv[sl] = make_uchar4(NONE, NONE, NONE, 0);
-                    S->fs[nfree + y] = (uint8_t)sl;
+            // the new vertices: the owner of boundary edge e's slot takes it
+            unsigned fresh[NR];   // ALIVE, kept neighbour, planes b and a; 0: not new
+            int before = 0;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const int t = r * 32 + lane;
+                const bool rm = remv >> r & 1;
+                const int e = rm ? before + __popc(bal[r] & lt) : nrem + sp + 1023 - (int)TV[r];
+                before += __popc(bal[r]);
+                fresh[r] = 0;
+                if ((rm || (int)TV[r] >= 0) && e < nb) {
+                    const unsigned w = S->bedge[e];   // (bit 31 set: the removed vertex was alive)
+                    S->start[w & 255u] = (uint8_t)t;            // the new triangle on the edge that starts at a
+                    S->eslot[(w >> 8) & 255u] = (uint8_t)t;     // ... and ends at b
+                    if (e == 0) S->start[m] = (uint8_t)t;
+                    fresh[r] = w;
+                } else if (rm) {   // a removed slot left over: onto the free stack
+                    TV[r] = (unsigned)(1024 + sp + e - nb);
                 }
             }
-            const int hw2 = extra <= nfree ? hw : hw + (extra - nfree);
-            if (lane == 0) {
-                if (extra <= nfree) S->nfree = nfree - extra;
-                else { S->nfree = 0; S->hw = hw2; }
-            }
-            nalive += extra;
-            nrounds = (hw2 + 31) >> 5;
+            sp = sp2;
+            hw = hw2;
             __syncwarp();
 #pragma unroll
-            for (int r = 0; r < SPL; ++r) {
-                if (r >= nrounds) break;
-                int t = r * 32 + lane;
-                if (S->rem[t] == 2) {
-                    compute_vertex(r, t);
-                    alive |= 1u << r;
-                    S->rem[t] = 0;
-                } else if (remv >> r & 1) {
-                    alive &= ~(1u << r);
+            for (int r = 0; r < NR; ++r) {
+                const unsigned w = fresh[r];
+                if (w) {
+                    TV[r] = __byte_perm(w, m, 0x3410);
+                    TA[r] = pack3((w >> 16) & 127u, S->start[(w >> 8) & 255u], S->eslot[w & 255u]);
+                    make_vertex(r, w, m);
+                } else if ((int)TV[r] < 0) {
+                    // a kept vertex: its edge (b -> a) towards a removed one now borders the new
+                    // triangle on the edge that starts at a
+                    const unsigned v = TV[r];
+                    if (nbr[r] & 1u) TA[r] = __byte_perm(TA[r], S->start[(v >> 8) & 255u], 0x3214);
+                    if (nbr[r] & 2u) TA[r] = __byte_perm(TA[r], S->start[(v >> 16) & 127u], 0x3240);
+                    if (nbr[r] & 4u) TA[r] = __byte_perm(TA[r], S->start[v & 255u], 0x3410);
                 }
             }
-            __syncwarp();
         }
-        if (!open_tests) break;
-        // the tests of plane kk that the filter left open: tight magnitudes, then exact
-        {
-            open_tests = false;
-            const int m = S->ord[kk] & (NE - 1);
-            const PlaneN<FA<R>> M = fplane(S, m);
-            rsv = 0;
-            for (int r = 0; r < nrounds; ++r) {
-                if (!(alive >> r & 1)) continue;
-                const uchar4 v = S->tv[r * 32 + lane];
-                const VtxFA<R> q = vertex_fa(S, v);
-                FA<R> sv;
-                sv.v = M.q.x.v * q.v[0] + M.q.y.v * q.v[1] + M.q.z.v * q.v[2] - M.b.v * q.v[3];
-                sv.a = M.q.x.a * q.a[0] + M.q.y.a * q.a[1] + M.q.z.a * q.a[2] + M.b.a * q.a[3];
-                int sg = fa_sign(sv, Gam<R>::gclip, Gam<R>::tiny);
-                if (sg == 0)
-                    sg = resolve_exact(c, PK_CLIP, S->pg[v.x & (NE - 1)], S->pg[v.y & (NE - 1)],
-                                       S->pg[v.z & (NE - 1)], S->pg[m], Gam<R>::try64);
-                if (sg > 0) rsv |= 1u << r;
+        if (!open_tests) return false;
+        // the tests of plane kk that the filter left open: tight magnitudes, then exact (out of
+        // the inner loop, which makes no call: with a call inside, the compiler kept the loop's
+        // state in local memory)
+        rsv = ALIVE;
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            if ((int)TV[r] < 0 && clip_sign(S, A.xyz, A.R, i, A.n, A.status, TV[r], NG + kk) > 0) rsv |= 1u << r;
+        }
+        };
+        if (clip(IntC<1>{})) {
+            if constexpr (SPL > 1) clip(IntC<SPL>{});
+        }
+        // the vertices alive, their planes alone (dead slots: NONE)
+        nrounds = (hw + 31) >> 5;
+#pragma unroll
+        for (int r = 0; r < SPL; ++r) {
+            if ((int)TV[r] < 0) alive |= 1u << r;
+            TV[r] = (int)TV[r] < 0 ? TV[r] & ~ALIVE : DEADV;
+        }
+        if constexpr (PH != PH_CELL) {   // the cell to shared memory, for the classification
+#pragma unroll
+            for (int r = 0; r < SPL; ++r) {
+                S->tv[r * 32 + lane] = unpack3(TV[r]);
+                S->ta[r * 32 + lane] = unpack3(TA[r]);
             }
-            resolved = true;
         }
-        }
+        if (lane == 0) S->hw = hw;
         }
         __syncwarp();
         const bool bad = S->bad != 0;
@@ -1361,13 +1424,16 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             const int np = NG + nc, hw = S->hw;
             for (int e = lane; e < np; e += 32) {
                 copy_row(rec->pq[e], S->pq[e]);
-                rec->pB[e] = S->pB[e];
+                rec->pB[e] = S->pm[e][1];
                 rec->pg[e] = S->pg[e];
                 rec->start[e] = S->start[e];
             }
-            for (int t = lane; t < hw; t += 32) {
-                rec->tv[t] = S->tv[t];
-                rec->ta[t] = S->ta[t];
+#pragma unroll
+            for (int r = 0; r < SPL; ++r) {
+                const int t = r * 32 + lane;
+                if (t >= hw) break;
+                rec->tv[t] = CARRY ? S->tv[t] : unpack3(TV[r]);
+                rec->ta[t] = CARRY ? S->ta[t] : unpack3(TA[r]);
             }
             if (lane == 0) {
                 rec->nc = nc;
@@ -1421,7 +1487,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                     const int e = lane + 32 * h;
                     if (e < np) {
                         store_row(S->pq[e], rq[h]);
-                        S->pB[e] = rb[h];
+                        S->pm[e][1] = rb[h];
                         S->pg[e] = rg[h];
                         S->start[e] = rs[h];
                         if constexpr (PH == PH_TERMS || PH == PH_VOL) S->eflag[e] = ref[h];
@@ -1438,7 +1504,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             } else {
                 for (int e = lane; e < np; e += 32) {
                     copy_row(S->pq[e], rec->pq[e]);
-                    S->pB[e] = rec->pB[e];
+                    S->pm[e][1] = rec->pB[e];
                     S->pg[e] = rec->pg[e];
                     S->start[e] = rec->start[e];
                 }
@@ -1817,7 +1883,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 if (st == NONE) continue;
                 uchar4 v = S->tv[st & (NT - 1)];
                 if (!(v.x == a || v.y == a || v.z == a)) continue;
-                FA<R> b = {S->pq[a][3], S->pB[a]};
+                FA<R> b = {S->pq[a][3], S->pm[a][1]};
                 int sg = fa_sign(b, Gam<R>::g, Gam<R>::tiny);
                 if (sg == 0) sg = resolve_exact(c, PK_VERT, S->pg[a], 0, 0, 0, Gam<R>::try64);
                 if (sg < 0) ok = false;
@@ -2062,18 +2128,20 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
 }  // namespace
 
 #ifndef DSASA_ATOMS_NO_LAUNCH
-// Whether every atom's warp of the cell kernel is resident at once (one wave).  Then the fused
-// cell + classification kernel runs an atom's classification while other atoms are still
-// clipping (the slowest cells set the end of the wave); with more atoms the split kernels keep
-// each kernel's instruction stream in the cache, which is worth more.
-template <class R> bool cells_in_one_wave(int n) {
+// Whether the cell construction and the classification run as one kernel: up to half as many
+// atoms as the GPU holds warps of it (2,432 on a GB300).  There an atom's classification
+// overlaps the slowest cells and one launch and the trip of the records through memory are
+// saved; with more atoms the split kernels win, whose smaller instruction streams stay in the
+// cache (fused / split, us per call with the gradient: 2,003 atoms 105 / 112, 2,500 116 / 115,
+// 3,500 136 / 131, 4,800 150.2 / 150.0).
+template <class R> bool cells_fused(int n) {
     static int cap = -1;
     if (cap < 0) {
         int dev = 0, sms = 0, per = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_atoms<R, false, 64, 64, PH_CC>, WARPS_CELL * 32, 0);
-        cap = sms * per * WARPS_CELL;
+        cap = sms * per * WARPS_CELL / 2;
     }
     return n <= cap;
 }
@@ -2113,7 +2181,7 @@ cudaError_t launch_atoms_t(const AtomArgs& a, bool grad, cudaStream_t s) {
     };
     if (a.cells) {
         auto nb = [&](int w) { return (a.n + w - 1) / w; };
-        if (!a.carry && cells_in_one_wave<R>(a.n)) {
+        if (!a.carry && cells_fused<R>(a.n)) {
             go(k_atoms<R, false, 64, 64, PH_CC>, nb(WARPS_CELL), WARPS_CELL * 32, fast);
             mark(0);
             mark(1);

@@ -52,6 +52,7 @@ struct dsasa_arena {
 
 struct dsasa_ctx {
     int device = 0;
+    int sms = 0;   // multiprocessors of the device
     cudaStream_t stream = nullptr;
     dsasa_config cfg{};
     // capacities
@@ -268,12 +269,10 @@ dsasa_status run(dsasa_ctx* c, const double* coords, const double* radii, double
         a.radii_in = radii;
     }
     a.skin_band = c->cfg.skin > 0.0;
-    // carried cells: always (carry 2), or (carry 1) for molecules of more than one wave of the
-    // fused cell kernel, where they pay (within one wave the fused kernel is faster)
-    if (lists && c->cfg.carry != 0) {
-        const bool one_wave = c->cfg.precision == DSASA_FP64 ? atoms_one_wave_f64((int)n) : atoms_one_wave_f32((int)n);
-        a.carry = c->cfg.carry == 2 || !one_wave;
-    }
+    // carried cells: always (carry 2), or (carry 1) for molecules of more than 36 atoms an SM
+    // (5,472 on a GB300), where they pay: below that the cells' latency sets the time, and a
+    // cell that is not carried costs a second kernel's
+    if (lists && c->cfg.carry != 0) a.carry = c->cfg.carry == 2 || n > 36 * (int64_t)c->sms;
     a.redo_list = c->redo;
     a.redo_count = c->status + 3;   // cleared by the cell-list build
     a.mol_off = offsets_dev;
@@ -352,6 +351,7 @@ dsasa_status dsasa_create(dsasa_ctx** out, int device, void* cuda_stream, const 
     c->device = device;
     c->stream = (cudaStream_t)cuda_stream;
     cudaError_t e = cudaSetDevice(device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = dev_alloc((void**)&c->status, 4 * sizeof(int));
     if (e == cudaSuccess) e = dev_alloc((void**)&c->nrec, sizeof(unsigned long long));
     if (e == cudaSuccess) e = dev_alloc((void**)&c->sr_tests, sizeof(unsigned long long));

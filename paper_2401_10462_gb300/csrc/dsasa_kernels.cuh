@@ -212,9 +212,6 @@ cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, co
 cudaError_t launch_sr(const SRArgs& a, cudaStream_t s);
 cudaError_t launch_atoms_f32(const AtomArgs& a, bool grad, cudaStream_t s);
 cudaError_t launch_atoms_f64(const AtomArgs& a, bool grad, cudaStream_t s);
-// whether n atoms fit one wave of the fused cell + classification kernel (mixed / FP64 form)
-bool atoms_one_wave_f32(int n);
-bool atoms_one_wave_f64(int n);
 size_t scan_scratch_ints(int max_cells);
 size_t cell_record_bytes();
 
