@@ -80,7 +80,7 @@ template <class R, int NE, int NT> struct Smem {
     uchar4 ta[NT];        // neighbour slots across edges (v0 v1), (v1 v2), (v2 v0)
     uint8_t kf[NT];       // 0 not in C, 1 tetrahedron of C, 2 involves a ghost plane
     unsigned tf[NT];      // bit k: the triangle of edge k is in C; bit 4+k: it is processed here
-    unsigned skey[NE];    // orderable sort key of each candidate
+    alignas(16) unsigned skey[NE];   // orderable sort key of each candidate
     uint16_t tl[NT * 3 / 2 + 2];   // compacted exterior triangles (slot << 2 | edge)
     uint8_t rem[NT];      // carried cells: start slots on the way to start[]
     int hw, bad;
@@ -1010,117 +1010,102 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             nclip = (cc >> 16) & 255;
         }
 
-        // ---------------- plane table: ghosts 0..5, candidates NG..NG+nc-1; sort keys
-        unsigned long long key[SPL];
-        unsigned pay[SPL];
-        for (int r = 0; r < SPL; ++r) { key[r] = ~0ull; pay[r] = 0; }
-        for (int e = lane; e < NG + nc; e += 32) {
-            double q[3], b, babs;
-            bool ex;
-            int g = e < NG ? -1 - e : S->pg[e];
-            plane64_of(c, g, q, b, babs, ex);
-            if (e < NG) S->pg[e] = g;
-            for (int k = 0; k < 3; ++k) S->pq[e][k] = (R)q[k];
-            S->pq[e][3] = (R)b;
-            // magnitude proxy of b in float: |b_f| (1 + 2^-22) + 2^-26 babs, rounded up (the float
-            // evaluation loses at most 2 ulp, covered by the larger factors)
-            if (sizeof(R) == 4) S->pm[e][1] = (R)(fabsf((float)b) * 1.0000003f + (float)babs * 1.5e-8f);
-            else S->pm[e][1] = (R)(ex ? fabs(b) : 8.0 * babs);
-            S->pm[e][0] = (R)((fabsf((float)q[0]) + fabsf((float)q[1]) + fabsf((float)q[2])) * 1.000001f);
-            S->start[e] = NONE;
-            if (e >= NG) {
-                // sort key: signed distance of the bisector from p_i (ties: atom index)
-                float qx = (float)q[0], qy = (float)q[1], qz = (float)q[2];
-                float kf = (float)b * rsqrtf(qx * qx + qy * qy + qz * qz + 1e-30f);
-                unsigned u = __float_as_uint(kf);
-                S->skey[e] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+        // ---------------- plane table: ghosts 0..5, then the candidates in the order of their
+        // bisectors' signed distances from p_i (ties: atom index), so that every later summation
+        // order depends only on the geometry and not on the order atoms sit in their cells.  A
+        // lane keeps its candidates' rows in registers, ranks them by counting the smaller keys
+        // (all keys read as broadcasts, four at a time) and writes each row once, where it belongs
+        R tq[SPL][4], tm[SPL][2];
+        int tg[SPL], rank[SPL];
+        unsigned key[SPL];
+#pragma unroll
+        for (int r = 0; r < SPL; ++r) {
+            const int el = r * 32 + lane;
+            rank[r] = el;
+            key[r] = ~0u;
+            if (el < nc) {
+                double q[3], b, babs;
+                bool ex;
+                tg[r] = S->pg[NG + el];
+                plane64_of(c, tg[r], q, b, babs, ex);
+                const float qx = (float)q[0], qy = (float)q[1], qz = (float)q[2];
+                for (int k = 0; k < 3; ++k) tq[r][k] = (R)q[k];
+                tq[r][3] = (R)b;
+                // magnitude proxy of b in float: |b_f| (1 + 2^-22) + 2^-26 babs, rounded up (the float
+                // evaluation loses at most 2 ulp, covered by the larger factors)
+                if (sizeof(R) == 4) tm[r][1] = (R)(fabsf((float)b) * 1.0000003f + (float)babs * 1.5e-8f);
+                else tm[r][1] = (R)(8.0 * babs);
+                tm[r][0] = (R)((fabsf(qx) + fabsf(qy) + fabsf(qz)) * 1.000001f);
+                const unsigned u = __float_as_uint((float)b * rsqrtf(qx * qx + qy * qy + qz * qz + 1e-30f));
+                key[r] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
             }
+        }
+        if (lane < NG) {
+            double q[3], b;
+            ghost_plane64(lane, c.h, q, b);
+            for (int k = 0; k < 3; ++k) S->pq[lane][k] = (R)q[k];
+            S->pq[lane][3] = (R)b;
+            S->pm[lane][0] = (R)(2.0 * c.h);
+            S->pm[lane][1] = sizeof(R) == 4 ? (R)(fabsf((float)b) * 1.0000004f) : (R)b;
+            S->pg[lane] = -1 - lane;
+        }
+        for (int e = lane; e < NG + nc; e += 32) {
+            S->start[e] = NONE;
             S->eflag[e] = 0;
         }
-        __syncwarp();
         if constexpr (!carried) {
-        for (int r = 0; r < SPL; ++r) {
-            int el = r * 32 + lane;
-            if (el < nc) {
-                key[r] = ((unsigned long long)S->skey[NG + el] << 32) | (unsigned)S->pg[NG + el];
-                pay[r] = NG + el;
+#pragma unroll
+            for (int r = 0; r < SPL; ++r) S->skey[r * 32 + lane] = key[r];   // (~0 past the last candidate)
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < SPL; ++r) rank[r] = 0;
+            const uint4* k4 = reinterpret_cast<const uint4*>(S->skey);
+            if (nc <= 32) {
+                for (int j = 0; j < nc; j += 4) {
+                    const uint4 k = k4[j >> 2];
+                    rank[0] += (k.x < key[0]) + (k.y < key[0]) + (k.z < key[0]) + (k.w < key[0]);
+                }
+            } else {
+                for (int j = 0; j < nc; j += 4) {
+                    const uint4 k = k4[j >> 2];
+#pragma unroll
+                    for (int r = 0; r < SPL; ++r)
+                        rank[r] += (k.x < key[r]) + (k.y < key[r]) + (k.z < key[r]) + (k.w < key[r]);
+                }
+            }
+            // equal keys give equal ranks: two candidates meet in one place, one of them is lost
+            bool tie = false;
+#pragma unroll
+            for (int r = 0; r < SPL; ++r)
+                if (r * 32 + lane < nc) S->bedge[rank[r]] = r * 32 + lane;
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < SPL; ++r)
+                if (r * 32 + lane < nc && S->bedge[rank[r]] != (unsigned)(r * 32 + lane)) tie = true;
+            if (__any_sync(FULL, tie)) {
+#pragma unroll
+                for (int r = 0; r < SPL; ++r) {
+                    rank[r] = 0;
+                    if (r * 32 + lane < nc)
+                        for (int j = 0; j < nc; ++j)
+                            rank[r] += S->skey[j] < key[r] || (S->skey[j] == key[r] && S->pg[NG + j] < tg[r]);
+                }
             }
         }
         __syncwarp();
-        // bitonic sort of the first ns (key, payload) pairs, element e = r*32 + lane; the
-        // padding keys are the largest, so sorting a power-of-two prefix that holds all nc
-        // candidates sorts them all
-        const int ns = nc <= 32 ? 32 : (nc <= 64 ? 64 : NT);
-        const int nsr = ns >> 5;
-        for (int k = 2; k <= ns; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                if (j >= 32) {
-                    // rounds r and r ^ (j / 32) in this lane's registers (the partner round is
-                    // a compile-time index in every unrolled branch, so key and pay stay in
-                    // registers)
-                    const int jr = j >> 5;
 #pragma unroll
-                    for (int JR = 1; JR < SPL; JR <<= 1) {
-                        if (jr != JR) continue;
-#pragma unroll
-                        for (int r = 0; r < SPL; ++r) {
-                            const int r2 = r ^ JR;
-                            if (r2 > r && r2 < nsr) {
-                                int e = r * 32 + lane;
-                                bool up = (e & k) == 0;
-                                bool sw = up ? (key[r] > key[r2]) : (key[r] < key[r2]);
-                                if (sw) {
-                                    unsigned long long tk = key[r]; key[r] = key[r2]; key[r2] = tk;
-                                    unsigned tp = pay[r]; pay[r] = pay[r2]; pay[r2] = tp;
-                                }
-                            }
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int r = 0; r < SPL; ++r) {
-                        if (r >= nsr) break;
-                        int e = r * 32 + lane;
-                        unsigned long long ok = __shfl_xor_sync(FULL, key[r], j);
-                        unsigned op = __shfl_xor_sync(FULL, pay[r], j);
-                        bool up = (e & k) == 0;
-                        bool lower = (lane & j) == 0;
-                        bool take = (lower == up) ? (ok < key[r]) : (ok > key[r]);
-                        if (take) { key[r] = ok; pay[r] = op; }
-                    }
-                }
+        for (int r = 0; r < SPL; ++r) {
+            if (r * 32 + lane < nc) {
+                const int e = NG + rank[r];
+                for (int k = 0; k < 4; ++k) S->pq[e][k] = tq[r][k];
+                S->pm[e][0] = tm[r][0];
+                S->pm[e][1] = tm[r][1];
+                S->pg[e] = tg[r];
             }
         }
-        // renumber the candidate planes in sorted order, so that every later summation
-        // order depends only on the geometry (not on the order atoms sit in their cells)
-        {
-            R tq[SPL][4], tb[SPL][2];
-            int tg[SPL];
-#pragma unroll
-            for (int r = 0; r < SPL; ++r) {
-                int e = r * 32 + lane;
-                if (e < nc) {
-                    int src = pay[r] & (NE - 1);
-                    for (int k = 0; k < 4; ++k) tq[r][k] = S->pq[src][k];
-                    tb[r][0] = S->pm[src][0];
-                    tb[r][1] = S->pm[src][1];
-                    tg[r] = S->pg[src];
-                }
-            }
-            __syncwarp();
-#pragma unroll
-            for (int r = 0; r < SPL; ++r) {
-                int e = r * 32 + lane;
-                if (e < nc) {
-                    for (int k = 0; k < 4; ++k) S->pq[NG + e][k] = tq[r][k];
-                    S->pm[NG + e][0] = tb[r][0];
-                    S->pm[NG + e][1] = tb[r][1];
-                    S->pg[NG + e] = tg[r];
-                }
-            }
-            __syncwarp();
-        }
+        __syncwarp();
 
+        if constexpr (!carried) {
         // ---------------- initial cell: the cube of the 6 ghost planes (8 vertices)
         if (lane < NG) S->start[lane] = (lane & 1) ? 7 : 0;   // +x,+y,+z at corner 0; -x,-y,-z at 7
         if (lane == 0) S->bad = 0;
