@@ -79,7 +79,9 @@ typedef enum {
  *                 whose gradient is below about 0.03 (nearly buried, or a sliver) can
  *                 therefore miss a 1e-3 relative bound with a 1e-2 floor.  DSASA_FP64 has no
  *                 such limit.
- *   DSASA_FP64  - every term in FP64; predicates filtered in FP64, then exact. */
+ *   DSASA_FP64  - every term in FP64, from the float64 coordinates; the cells are those of the
+ *                 FP32 -> FP64 -> exact predicates too (their decisions do not depend on the
+ *                 filter). */
 enum { DSASA_MIXED = 0, DSASA_FP64 = 1 };
 
 typedef struct {

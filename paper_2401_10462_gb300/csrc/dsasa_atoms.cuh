@@ -86,8 +86,9 @@ template <class R, int NE, int NT> struct Smem {
     int hw, bad;
 };
 
-// The cell of one atom between the two kernels (first NG + nc plane entries, first hw
-// vertex slots used).
+// The cell of one atom between the kernels (first NG + nc plane entries, first hw vertex slots
+// used).  Both precisions use the FP32 kernels' record: the structure of the cell is exact, and
+// the FP64 terms take their plane vectors from the float64 coordinates.
 template <class R, int NE, int NT> struct CellRec {
     alignas(16) R pq[NE][4];
     R pB[NE];
@@ -103,8 +104,7 @@ template <class R, int NE, int NT> struct CellRec {
     int atom;             // the atom whose cell this is (-1: no cell), for carrying it to the next call
 };
 using CellRecF = CellRec<float, 64, 64>;
-using CellRecD = CellRec<double, 64, 64>;
-static_assert(offsetof(CellRecF, iK) % 16 == 0 && offsetof(CellRecD, iK) % 16 == 0,
+static_assert(offsetof(CellRecF, iK) % 16 == 0,
               "the record header (iK, icl, nc, hw) is read as one 16-byte load");
 // The plane rows move in 16-byte pieces (copy_row, load_row, store_row): every row of the
 // shared table and of a record must start on a 16-byte boundary.  Records are indexed as an
@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
         c.status = A.status;
         const R Rr = (R)c.Ri;
         const FA<R> wi = {Rr * Rr, Rr * Rr};
-        CellRec<R, NE, NT>* rec = (CellRec<R, NE, NT>*)A.cells + s;
+        CellRec<float, NE, NT>* rec = (CellRec<float, NE, NT>*)A.cells + s;
         auto done = [&]() {   // the outputs of this atom are written: tell the terms kernel
             if ((PH == PH_CELL || PH == PH_CLASS || PH == PH_CC) && lane == 0) rec->flag = CELL_DONE;
         };
@@ -1123,7 +1123,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             // (ii) every face plane keeps every vertex not on it strictly inside.  The new
             // candidates are tested in the same sweep (planes outer, the lane's vertices inner,
             // one warp vote at the end): one that removes a vertex sends the atom to the redo list,
-            // and so does any test that the FP32 (FP64) filter leaves open
+            // and so does any test that the filter leaves open
             const int hw0 = S->hw;
             nrounds = (hw0 + 31) >> 5;
 #pragma unroll
@@ -1137,8 +1137,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 if (!(alive >> r & 1)) continue;
                 FA<R> D;
                 D.v = V[r][3];
-                if constexpr (LOOSE) D.a = Vs[r];
-                else D.a = Va[r][3];
+                D.a = Vs[r];
                 if (fa_sign(D, Gam<R>::g, Gam<R>::tiny) <= 0) fail = true;
             }
             for (int kk = 0; kk < nclip; ++kk) {
@@ -1154,8 +1153,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                     if (cert && (v.x == m || v.y == m || v.z == m)) continue;   // a vertex on the face
                     FA<R> sv;
                     sv.v = M.q.x.v * V[r][0] + M.q.y.v * V[r][1] + M.q.z.v * V[r][2] - M.b.v * V[r][3];
-                    if constexpr (LOOSE) sv.a = qmax * Vs[r];
-                    else sv.a = M.q.x.a * Va[r][0] + M.q.y.a * Va[r][1] + M.q.z.a * Va[r][2] + M.b.a * Va[r][3];
+                    sv.a = qmax * Vs[r];
                     // the filters only: a test they leave open sends the atom to the redo
                     // list (no call in the loop; such tests are rare)
                     const int sg = fa_sign(sv, Gam<R>::gclip, Gam<R>::tiny);
@@ -1408,7 +1406,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             // hand the cell to the terms kernel
             const int np = NG + nc, hw = S->hw;
             for (int e = lane; e < np; e += 32) {
-                copy_row(rec->pq[e], S->pq[e]);
+                copy_row(rec->pq[e], (const float*)S->pq[e]);
                 rec->pB[e] = S->pm[e][1];
                 rec->pg[e] = S->pg[e];
                 rec->start[e] = S->start[e];
@@ -1440,10 +1438,25 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             nc = hd.z;
             const int np = NG + nc, hw = hd.w;
             nrounds = (hw + 31) >> 5;
-            constexpr bool BATCH_LOADS = PH == PH_CLASS || PH == PH_VOL;
+            // the FP64 form's plane of entry e: its vector (and, for the volume, its offset) from
+            // the float64 coordinates (only atoms' planes are used after the classification;
+            // ghost faces only by the volume)
+            auto plane_of = [&](int e, int g) {
+                double q[3], b, babs;
+                bool ex;
+                if (PH == PH_VOL) {
+                    plane64_of(c, g, q, b, babs, ex);
+                    S->pq[e][3] = (R)b;
+                } else {
+                    g = DS_IDX(max(g, 0), A.n, A.status);
+                    for (int k = 0; k < 3; ++k) q[k] = A.xyz[3 * g + k] - c.pi[k];
+                }
+                for (int k = 0; k < 3; ++k) S->pq[e][k] = (R)q[k];
+            };
+            constexpr bool BATCH_LOADS = sizeof(R) == 4 && (PH == PH_CLASS || PH == PH_VOL);
             if constexpr (BATCH_LOADS) {
-                Row4<R> rq[2];
-                R rb[2];
+                Row4<float> rq[2];
+                float rb[2];
                 int rg[2];
                 uint8_t rs[2], ref[2] = {0, 0}, rkf[2] = {0, 0}, rtf[2] = {0, 0};
                 uchar4 rtv[2], rta[2];
@@ -1471,7 +1484,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 for (int h = 0; h < 2; ++h) {
                     const int e = lane + 32 * h;
                     if (e < np) {
-                        store_row(S->pq[e], rq[h]);
+                        store_row((float*)S->pq[e], rq[h]);
                         S->pm[e][1] = rb[h];
                         S->pg[e] = rg[h];
                         S->start[e] = rs[h];
@@ -1488,9 +1501,10 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 }
             } else {
                 for (int e = lane; e < np; e += 32) {
-                    copy_row(S->pq[e], rec->pq[e]);
-                    S->pm[e][1] = rec->pB[e];
-                    S->pg[e] = rec->pg[e];
+                    const int g = rec->pg[e];
+                    if constexpr (sizeof(R) == 4) copy_row((float*)S->pq[e], rec->pq[e]);
+                    else plane_of(e, g);
+                    S->pg[e] = g;
                     S->start[e] = rec->start[e];
                 }
                 for (int t = lane; t < 32 * nrounds; t += 32) {
@@ -2113,32 +2127,27 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
 }  // namespace
 
 #ifndef DSASA_ATOMS_NO_LAUNCH
-// Whether the cell construction and the classification run as one kernel: up to half as many
-// atoms as the GPU holds warps of it (2,432 on a GB300).  There an atom's classification
-// overlaps the slowest cells and one launch and the trip of the records through memory are
-// saved; with more atoms the split kernels win, whose smaller instruction streams stay in the
-// cache (fused / split, us per call with the gradient: 2,003 atoms 105 / 112, 2,500 116 / 115,
-// 3,500 136 / 131, 4,800 150.2 / 150.0).
-template <class R> bool cells_fused(int n) {
-    static int cap = -1;
-    if (cap < 0) {
-        int dev = 0, sms = 0, per = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_atoms<R, false, 64, 64, PH_CC>, WARPS_CELL * 32, 0);
-        cap = sms * per * WARPS_CELL / 2;
+// Fast pass (64 planes, 64 vertex slots) over all atoms: with a cell store, the cell and
+// classification kernels (the FP32 ones in both precisions: their decisions are exact), then
+// the terms kernel in R; without one, the fused kernel (mixed form only).  The atoms it defers
+// get the fused 128 / 128 pass, whose grid reads the deferred count from device memory (no host
+// sync).  The deferred count must be zero when the first kernel starts (the cell-list build
+// clears it).  Every kernel after the cell-list build is a programmatic dependent launch
+// (measured: 3 % faster on a 5k-atom molecule in the mixed form).
+struct AtomLaunch {
+    cudaStream_t s;
+    cudaError_t err = cudaSuccess;
+    template <class K> void operator()(K kernel, int grid, int block, const AtomArgs& args) {
+        const cudaError_t e = launch_dependent(kernel, grid, block, s, true, args);
+        if (err == cudaSuccess) err = e;
+        note_launches(1);
     }
-    return n <= cap;
-}
+};
 
-// Fast pass (64 planes, 64 vertex slots) over all atoms: with a cell store, the cell,
-// classification and terms kernels, else the fused kernel.  The atoms it defers get the fused 128 / 128
-// pass, whose grid reads the deferred count from device memory (no host sync).  The deferred
-// count must be zero when the first kernel starts (the cell-list build clears it).
 template <class R>
 cudaError_t launch_atoms_t(const AtomArgs& a, bool grad, cudaStream_t s) {
     if (a.n <= 0) return cudaSuccess;
-    int blocks = (a.n + WARPS - 1) / WARPS;
+    const int blocks = (a.n + WARPS - 1) / WARPS;
     AtomArgs fast = a;
     fast.work_list = nullptr;
     fast.work_count = nullptr;
@@ -2150,59 +2159,35 @@ cudaError_t launch_atoms_t(const AtomArgs& a, bool grad, cudaStream_t s) {
     big.cells = nullptr;
     fast.ev = big.ev = nullptr;
     // the deferred atoms are few: a small grid that loops over them (most calls have none)
-    int big_blocks = blocks < 64 ? blocks : 64;
+    const int big_blocks = blocks < 64 ? blocks : 64;
     const bool g = grad && a.rec == nullptr;
     auto mark = [&](int k) {
         if (a.ev) cudaEventRecord(a.ev[k], s);
     };
-    // every kernel after the cell-list build is a programmatic dependent launch in the mixed
-    // form (measured: 3 % faster on a 5k-atom molecule); the all-FP64 form's kernels ran 3 %
-    // slower that way and are launched in plain stream order
-    cudaError_t err = cudaSuccess;
-    auto go = [&](auto kernel, int grid, int block, const AtomArgs& args) {
-        cudaError_t e = launch_dependent(kernel, grid, block, s, sizeof(R) == 4, args);
-        if (err == cudaSuccess) err = e;
-        note_launches(1);
-    };
+    AtomLaunch go{s};
     if (a.cells) {
-        auto nb = [&](int w) { return (a.n + w - 1) / w; };
-        if (!a.carry && cells_fused<R>(a.n)) {
-            go(k_atoms<R, false, 64, 64, PH_CC>, nb(WARPS_CELL), WARPS_CELL * 32, fast);
-            mark(0);
-            mark(1);
-        } else {
-            if (a.carry) {
-                // the carried cells, then the cell kernel over the redo list (its grid covers
-                // every atom; the warps past the list's length return at once)
-                go(k_atoms<R, false, 64, 64, PH_CARRY>, nb(WARPS_CELL), WARPS_CELL * 32, fast);
-                AtomArgs redo = fast;
-                redo.work_list = a.redo_list;
-                redo.work_count = a.redo_count;
-                go(k_atoms<R, false, 64, 64, PH_CELL>, nb(WARPS_CELL), WARPS_CELL * 32, redo);
-            } else {
-                go(k_atoms<R, false, 64, 64, PH_CELL>, nb(WARPS_CELL), WARPS_CELL * 32, fast);
-            }
-            mark(0);
-            go(k_atoms<R, false, 64, 64, PH_CLASS>, nb(WARPS_CLASS), WARPS_CLASS * 32, fast);
-            mark(1);
-        }
-        if (g) go(k_atoms<R, true, 64, 64, PH_TERMS>, nb(WARPS_TERMS), WARPS_TERMS * 32, fast);
-        else go(k_atoms<R, false, 64, 64, PH_TERMS>, nb(WARPS_TERMS), WARPS_TERMS * 32, fast);
-        if (a.vol) go(k_atoms<R, false, 64, 64, PH_VOL>, nb(WARPS_TERMS), WARPS_TERMS * 32, fast);
+        const int grid = (a.n + WARPS_TERMS - 1) / WARPS_TERMS;
+        const cudaError_t e = launch_cells(a, s);
+        if (e != cudaSuccess) return e;
+        if (g) go(k_atoms<R, true, 64, 64, PH_TERMS>, grid, WARPS_TERMS * 32, fast);
+        else go(k_atoms<R, false, 64, 64, PH_TERMS>, grid, WARPS_TERMS * 32, fast);
+        if (a.vol) go(k_atoms<R, false, 64, 64, PH_VOL>, grid, WARPS_TERMS * 32, fast);
         mark(2);
-    } else {
+    } else if constexpr (sizeof(R) == 4) {
         if (g) go(k_atoms<R, true, 64, 64, PH_ALL>, blocks, WARPS * 32, fast);
         else go(k_atoms<R, false, 64, 64, PH_ALL>, blocks, WARPS * 32, fast);
         mark(0);
         mark(1);
         mark(2);
+    } else {
+        return cudaErrorInvalidValue;   // every context has a cell store
     }
     if (a.defer_list) {
         if (g) go(k_atoms<R, true, 128, 128, PH_ALL>, big_blocks, WARPS * 32, big);
         else go(k_atoms<R, false, 128, 128, PH_ALL>, big_blocks, WARPS * 32, big);
     }
     mark(3);
-    return err != cudaSuccess ? err : cudaGetLastError();
+    return go.err != cudaSuccess ? go.err : cudaGetLastError();
 }
 #endif
 

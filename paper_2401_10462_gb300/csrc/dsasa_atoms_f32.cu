@@ -1,12 +1,65 @@
-// Mixed-precision instantiation of the per-atom kernel: FP32 terms, FP32 -> FP64 -> exact
-// predicates (see dsasa_atoms.cuh).
+// FP32 instantiations of the per-atom kernels: the cell construction and classification of both
+// precisions (FP32 -> FP64 -> exact predicates) and the mixed form's terms (see
+// dsasa_atoms.cuh).
 #include "dsasa_atoms.cuh"
 
 namespace dsasa {
-cudaError_t launch_atoms_f32(const AtomArgs& a, bool grad, cudaStream_t s) { return launch_atoms_t<float>(a, grad, s); }
-// bytes of one atom's cell record between the two kernels (the larger of the two precisions)
-size_t cell_record_bytes() {
-    return sizeof(CellRec<double, 64, 64>) > sizeof(CellRec<float, 64, 64>) ? sizeof(CellRec<double, 64, 64>)
-                                                                            : sizeof(CellRec<float, 64, 64>);
+namespace {
+
+// Whether the cell construction and the classification run as one kernel: up to half as many
+// atoms as the GPU holds warps of it (2,432 on a GB300).  There an atom's classification
+// overlaps the slowest cells and one launch and the trip of the records through memory are
+// saved; with more atoms the split kernels win, whose smaller instruction streams stay in the
+// cache (fused / split, us per call with the gradient: 2,003 atoms 105 / 112, 2,500 116 / 115,
+// 3,500 136 / 131, 4,800 150.2 / 150.0).
+bool cells_fused(int n) {
+    static int cap = -1;
+    if (cap < 0) {
+        int dev = 0, sms = 0, per = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_atoms<float, false, 64, 64, PH_CC>, WARPS_CELL * 32, 0);
+        cap = sms * per * WARPS_CELL / 2;
+    }
+    return n <= cap;
 }
+
+}  // namespace
+
+// The cell records of every atom, classified (Steps 1 and 2).
+cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s) {
+    AtomArgs fast = a;
+    fast.work_list = nullptr;
+    fast.work_count = nullptr;
+    fast.ev = nullptr;
+    auto mark = [&](int k) {
+        if (a.ev) cudaEventRecord(a.ev[k], s);
+    };
+    auto nb = [&](int w) { return (a.n + w - 1) / w; };
+    AtomLaunch go{s};
+    if (!a.carry && cells_fused(a.n)) {
+        go(k_atoms<float, false, 64, 64, PH_CC>, nb(WARPS_CELL), WARPS_CELL * 32, fast);
+        mark(0);
+    } else {
+        if (a.carry) {
+            // the carried cells, then the cell kernel over the redo list (its grid covers every
+            // atom; the warps past the list's length return at once)
+            go(k_atoms<float, false, 64, 64, PH_CARRY>, nb(WARPS_CELL), WARPS_CELL * 32, fast);
+            AtomArgs redo = fast;
+            redo.work_list = a.redo_list;
+            redo.work_count = a.redo_count;
+            go(k_atoms<float, false, 64, 64, PH_CELL>, nb(WARPS_CELL), WARPS_CELL * 32, redo);
+        } else {
+            go(k_atoms<float, false, 64, 64, PH_CELL>, nb(WARPS_CELL), WARPS_CELL * 32, fast);
+        }
+        mark(0);
+        go(k_atoms<float, false, 64, 64, PH_CLASS>, nb(WARPS_CLASS), WARPS_CLASS * 32, fast);
+    }
+    mark(1);
+    return go.err;
+}
+
+cudaError_t launch_atoms_f32(const AtomArgs& a, bool grad, cudaStream_t s) { return launch_atoms_t<float>(a, grad, s); }
+// bytes of one atom's cell record between the kernels
+size_t cell_record_bytes() { return sizeof(CellRecF); }
 }  // namespace dsasa

@@ -1,5 +1,5 @@
-// All-FP64 instantiation of the per-atom kernel: FP64 terms, FP64 -> exact predicates
-// (see dsasa_atoms.cuh).
+// FP64 instantiations of the per-atom kernels: the all-FP64 terms over the cells that the FP32
+// kernels certify (see dsasa_atoms.cuh).
 #include "dsasa_atoms.cuh"
 
 namespace dsasa {

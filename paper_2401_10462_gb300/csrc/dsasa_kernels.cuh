@@ -210,6 +210,8 @@ cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, co
                                       const long long* base, int n, int n_mol, double skin, int* vmol, int* reuse,
                                       cudaStream_t s);
 cudaError_t launch_sr(const SRArgs& a, cudaStream_t s);
+// the classified cell records of every atom (a.cells), for the terms of either precision
+cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s);
 cudaError_t launch_atoms_f32(const AtomArgs& a, bool grad, cudaStream_t s);
 cudaError_t launch_atoms_f64(const AtomArgs& a, bool grad, cudaStream_t s);
 size_t scan_scratch_ints(int max_cells);
