@@ -21,8 +21,8 @@
 // One warp per atom (two per block); the cell lives in shared memory (plane table, triangle
 // table) and in registers (each lane caches the homogeneous coordinates of up to NT / 32
 // cell vertices).  The fast path runs the steps as separate kernels that hand the cell over
-// through a per-atom record in HBM (PH_CELL: Step 1; PH_CLASS: Step 2; PH_TERMS: Step 3;
-// PH_VOL: the volume), so that each kernel's code fits the instruction cache.  On small
+// through a per-atom record in HBM (PH_CELL: Step 1; PH_CLASS: Step 2; k_terms in
+// dsasa_terms.cuh: Step 3; PH_VOL: the volume), so that each kernel's code fits the instruction cache.  On small
 // molecules Steps 1 and 2 run as one kernel (PH_CC, cells_fused), so that classifications
 // overlap the slowest cells.  With carried cells, Step 1 is PH_CARRY (on calls reusing the neighbour
 // lists, each atom's cell from the previous call, kept when exact predicates certify it) and
@@ -54,7 +54,7 @@ constexpr int MINB = 32, MINB_CELL = 16, MINB_CLASS = 18, MINB_TERMS = 18;
 // through a global record per atom: the cell construction (gather, sort, clipping), the
 // classification (Steps 2a-2c: which simplices of the cell are in C), and the area terms and
 // gradient.  Each kernel's code then fits the instruction cache.
-enum { PH_ALL = 0, PH_CELL = 1, PH_CLASS = 2, PH_TERMS = 3, PH_VOL = 4, PH_CC = 5, PH_CARRY = 6 };
+enum { PH_ALL = 0, PH_CELL = 1, PH_CLASS = 2, PH_VOL = 4, PH_CC = 5, PH_CARRY = 6 };
 template <int N> struct IntC { static constexpr int value = N; };
 enum { CELL_OK = 0, CELL_DONE = 1 };   // record flag: CELL_DONE = outputs already written
 
@@ -254,6 +254,21 @@ __device__ __noinline__ void molecule_count(const AtomArgs& A, int i) {
         __threadfence_system();
         *(volatile int*)(A.mol_ready + m) = 1;
     }
+}
+
+// diagnostic export: the simplex {v0, v1, v2, v3} of C as seen by atom i (-1: unused slots)
+__device__ __noinline__ void export_simplex(const AtomArgs& A, int i, int v0, int v1, int v2, int v3) {
+    const unsigned long long at = atomicAdd(A.nrec, 1ull);
+    if ((long long)at >= A.max_rec) return;
+    int* rr = A.rec + 5 * at;
+    int tmp[4] = {v0, v1, v2, v3};
+    // sort the atom indices (-1 last)
+    for (int p = 0; p < 4; ++p)
+        for (int q = p + 1; q < 4; ++q) {
+            const bool sw = (tmp[q] >= 0) && (tmp[p] < 0 || tmp[q] < tmp[p]);
+            if (sw) { const int x = tmp[p]; tmp[p] = tmp[q]; tmp[q] = x; }
+        }
+    rr[0] = i; rr[1] = tmp[0]; rr[2] = tmp[1]; rr[3] = tmp[2]; rr[4] = tmp[3];
 }
 
 // predicate kinds
@@ -719,10 +734,10 @@ __device__ __noinline__ int carry_cell(SM* S, const RC* rec, int i, int n, int n
 
 // ------------------------------------------------------------------ the kernel
 __host__ __device__ constexpr int minb(int ph) {
-    return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? MINB_CELL : (ph == PH_CLASS ? MINB_CLASS : ((ph == PH_TERMS || ph == PH_VOL) ? MINB_TERMS : MINB));
+    return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? MINB_CELL : (ph == PH_CLASS ? MINB_CLASS : (ph == PH_VOL ? MINB_TERMS : MINB));
 }
 __host__ __device__ constexpr int warps_of(int ph) {
-    return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? WARPS_CELL : (ph == PH_CLASS ? WARPS_CLASS : ((ph == PH_TERMS || ph == PH_VOL) ? WARPS_TERMS : WARPS));
+    return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? WARPS_CELL : (ph == PH_CLASS ? WARPS_CLASS : (ph == PH_VOL ? WARPS_TERMS : WARPS));
 }
 template <class R, bool GRAD, int NE, int NT, int PHX>
 __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArgs A) {
@@ -1438,27 +1453,12 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             nc = hd.z;
             const int np = NG + nc, hw = hd.w;
             nrounds = (hw + 31) >> 5;
-            // the FP64 form's plane of entry e: its vector (and, for the volume, its offset) from
-            // the float64 coordinates (only atoms' planes are used after the classification;
-            // ghost faces only by the volume)
-            auto plane_of = [&](int e, int g) {
-                double q[3], b, babs;
-                bool ex;
-                if (PH == PH_VOL) {
-                    plane64_of(c, g, q, b, babs, ex);
-                    S->pq[e][3] = (R)b;
-                } else {
-                    g = DS_IDX(max(g, 0), A.n, A.status);
-                    for (int k = 0; k < 3; ++k) q[k] = A.xyz[3 * g + k] - c.pi[k];
-                }
-                for (int k = 0; k < 3; ++k) S->pq[e][k] = (R)q[k];
-            };
             constexpr bool BATCH_LOADS = sizeof(R) == 4 && (PH == PH_CLASS || PH == PH_VOL);
             if constexpr (BATCH_LOADS) {
                 Row4<float> rq[2];
                 float rb[2];
                 int rg[2];
-                uint8_t rs[2], ref[2] = {0, 0}, rkf[2] = {0, 0}, rtf[2] = {0, 0};
+                uint8_t rs[2], ref[2] = {0, 0};
                 uchar4 rtv[2], rta[2];
     #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -1468,16 +1468,12 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                         rb[h] = rec->pB[e];
                         rg[h] = rec->pg[e];
                         rs[h] = rec->start[e];
-                        if constexpr (PH == PH_TERMS || PH == PH_VOL) ref[h] = rec->eflag[e];
+                        if constexpr (PH == PH_VOL) ref[h] = rec->eflag[e];
                     }
                     rtv[h] = rta[h] = make_uchar4(NONE, NONE, NONE, 0);
                     if (e < hw) {
                         rtv[h] = rec->tv[e];
                         rta[h] = rec->ta[e];
-                        if constexpr (PH == PH_TERMS) {
-                            rkf[h] = rec->kf[e];
-                            rtf[h] = rec->tf[e];
-                        }
                     }
                 }
     #pragma unroll
@@ -1488,22 +1484,22 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                         S->pm[e][1] = rb[h];
                         S->pg[e] = rg[h];
                         S->start[e] = rs[h];
-                        if constexpr (PH == PH_TERMS || PH == PH_VOL) S->eflag[e] = ref[h];
+                        if constexpr (PH == PH_VOL) S->eflag[e] = ref[h];
                     }
                     if (e < 32 * nrounds) {
                         S->tv[e] = rtv[h];
                         S->ta[e] = rta[h];
-                        if constexpr (PH == PH_TERMS) {
-                            S->kf[e] = rkf[h];
-                            S->tf[e] = rtf[h];
-                        }
                     }
                 }
             } else {
+                // the FP64 volume: planes from the float64 coordinates
                 for (int e = lane; e < np; e += 32) {
                     const int g = rec->pg[e];
-                    if constexpr (sizeof(R) == 4) copy_row((float*)S->pq[e], rec->pq[e]);
-                    else plane_of(e, g);
+                    double q[3], b, babs;
+                    bool ex;
+                    plane64_of(c, g, q, b, babs, ex);
+                    for (int k = 0; k < 3; ++k) S->pq[e][k] = (R)q[k];
+                    S->pq[e][3] = (R)b;
                     S->pg[e] = g;
                     S->start[e] = rec->start[e];
                 }
@@ -1511,14 +1507,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                     S->tv[t] = t < hw ? rec->tv[t] : make_uchar4(NONE, NONE, NONE, 0);
                     S->ta[t] = t < hw ? rec->ta[t] : make_uchar4(NONE, NONE, NONE, 0);
                 }
-                if constexpr (PH == PH_TERMS || PH == PH_VOL)
-                    for (int e = lane; e < np; e += 32) S->eflag[e] = rec->eflag[e];
-                if constexpr (PH == PH_TERMS) {
-                    for (int t = lane; t < 32 * nrounds; t += 32) {
-                        S->kf[t] = t < hw ? rec->kf[t] : 0;
-                        S->tf[t] = t < hw ? rec->tf[t] : 0;
-                    }
-                }
+                for (int e = lane; e < np; e += 32) S->eflag[e] = rec->eflag[e];
             }
             if (lane == 0) { S->hw = hw; S->bad = 0; }
             __syncwarp();
@@ -1548,11 +1537,6 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
 
         // ---------------- Step 2a: tetrahedra of C (cell vertices inside B_i)
         unsigned kmask = 0;
-        if constexpr (PH == PH_TERMS) {
-#pragma unroll
-            for (int r = 0; r < SPL; ++r)
-                if ((alive >> r & 1) && S->kf[r * 32 + lane] == 1) kmask |= 1u << r;
-        } else {
         // The classification loops make no call on their predicates: a test that the filter
         // leaves open is marked and resolved after the loop (tight magnitudes, exact).
         unsigned open2a = 0;   // rounds whose tetrahedron test the loose filter left open
@@ -1658,7 +1642,6 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             }
         }
         __syncwarp();
-        }
 
         // ---------------- Step 2c / 3: faces (edges of C), area terms, gradient gathers
         // Vectors, angles and the gradient are evaluated in R (float in the mixed mode).  The
@@ -1717,7 +1700,6 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 gacc.add(kap * gsum.x + cf * pa.x, kap * gsum.y + cf * pa.y, kap * gsum.z + cf * pa.z);
             }
         };
-        if constexpr (PH != PH_TERMS) {
         // faces whose edge test the filters left open (bit = the lane's face iteration), and
         // which of them are closed; resolved after the loop (the fused kernel decides in place)
         unsigned open2c = 0, closed2c = 0;
@@ -1837,38 +1819,8 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             }
         }
         __syncwarp();
-        } else {
-        // the faces that are edges of C and not closed (classified by the previous kernel)
-        for (int a = NG + lane; a < NG + nc; a += 32) {
-            if ((S->eflag[a] & 3) != 1) continue;
-            const int st = S->start[a] & (NT - 1);
-            const P3<R> O = {zero, zero, zero};
-            const P3<R> pa = ppos(S, a);
-            R phi_sum = zero;
-            P3<R> gsum = {zero, zero, zero};
-            int t = st;
-            for (int step = 0; step < NT; ++step) {
-                uchar4 v = S->tv[t];
-                int k = v.x == a ? 0 : (v.y == a ? 1 : 2);
-                if (S->kf[t] == 1) {
-                    P3<R> pb = ppos(S, tv_get(v, (k + 1) % 3)), pc = ppos(S, tv_get(v, (k + 2) % 3));
-                    phi_sum += dihedral(O, pa, pb, pc);
-                    if (GRAD) gsum = gsum + dihedral_grad_u_in(O, pa, pb, pc, (R)1);
-                }
-                t = tv_get(S->ta[t], k) & (NT - 1);
-                if (t == st) break;
-            }
-            edge_term(a, pa, phi_sum, gsum);
-        }
-        __syncwarp();
-        }
-
         // vertex i in C?  (an edge of C holds it, or p_i lies in its own cell)
         bool iK, icl;
-        if constexpr (PH == PH_TERMS) {
-            iK = rec->iK != 0;
-            icl = rec->icl != 0;
-        } else {
         iK = __any_sync(FULL, myEK);
         icl = true;   // cell entirely inside B_i: interior vertex
 #pragma unroll
@@ -1888,8 +1840,6 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 if (sg < 0) ok = false;
             }
             iK = __all_sync(FULL, ok);
-        }
-
         }
         if constexpr (PH == PH_CLASS || PH == PH_CC) {
             __syncwarp();
@@ -2092,32 +2042,18 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
 
         // ---------------- optional export of the simplices of C containing i
         if (EXPORT) {
-            auto emit = [&](int v0, int v1, int v2, int v3) {
-                unsigned long long pos = atomicAdd(A.nrec, 1ull);
-                if ((long long)pos < A.max_rec) {
-                    int* rr = A.rec + 5 * pos;
-                    int tmp[4] = {v0, v1, v2, v3};
-                    // sort the atom indices (-1 last)
-                    for (int p = 0; p < 4; ++p)
-                        for (int q2 = p + 1; q2 < 4; ++q2) {
-                            bool sw = (tmp[q2] >= 0) && (tmp[p] < 0 || tmp[q2] < tmp[p]);
-                            if (sw) { int x = tmp[p]; tmp[p] = tmp[q2]; tmp[q2] = x; }
-                        }
-                    rr[0] = i; rr[1] = tmp[0]; rr[2] = tmp[1]; rr[3] = tmp[2]; rr[4] = tmp[3];
-                }
-            };
-            if (lane == 0 && iK) emit(i, -1, -1, -1);
+            if (lane == 0 && iK) export_simplex(A, i, i, -1, -1, -1);
             for (int a = NG + lane; a < NG + nc; a += 32)
-                if (S->eflag[a] & 1) emit(i, S->pg[a], -1, -1);
+                if (S->eflag[a] & 1) export_simplex(A, i, i, S->pg[a], -1, -1);
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
                 if (!(alive >> r & 1)) continue;
                 int t = r * 32 + lane;
                 uchar4 v = S->tv[t];
-                if (kmask >> r & 1) emit(i, S->pg[v.x], S->pg[v.y], S->pg[v.z]);
+                if (kmask >> r & 1) export_simplex(A, i, i, S->pg[v.x], S->pg[v.y], S->pg[v.z]);
                 unsigned f = S->tf[t];
                 for (int k = 0; k < 3; ++k)
-                    if ((f >> (4 + k)) & 1) emit(i, S->pg[tv_get(v, k)], S->pg[tv_get(v, (k + 1) % 3)], -1);
+                    if ((f >> (4 + k)) & 1) export_simplex(A, i, i, S->pg[tv_get(v, k)], S->pg[tv_get(v, (k + 1) % 3)], -1);
             }
         }
         __syncwarp();
@@ -2126,7 +2062,12 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
 
 }  // namespace
 
-#ifndef DSASA_ATOMS_NO_LAUNCH
+}  // namespace dsasa
+
+#include "dsasa_terms.cuh"
+
+namespace dsasa {
+
 // Fast pass (64 planes, 64 vertex slots) over all atoms: with a cell store, the cell and
 // classification kernels (the FP32 ones in both precisions: their decisions are exact), then
 // the terms kernel in R; without one, the fused kernel (mixed form only).  The atoms it defers
@@ -2169,8 +2110,8 @@ cudaError_t launch_atoms_t(const AtomArgs& a, bool grad, cudaStream_t s) {
         const int grid = (a.n + WARPS_TERMS - 1) / WARPS_TERMS;
         const cudaError_t e = launch_cells(a, s);
         if (e != cudaSuccess) return e;
-        if (g) go(k_atoms<R, true, 64, 64, PH_TERMS>, grid, WARPS_TERMS * 32, fast);
-        else go(k_atoms<R, false, 64, 64, PH_TERMS>, grid, WARPS_TERMS * 32, fast);
+        if (g) go(k_terms<R, true>, grid, WARPS_TERMS * 32, fast);
+        else go(k_terms<R, false>, grid, WARPS_TERMS * 32, fast);
         if (a.vol) go(k_atoms<R, false, 64, 64, PH_VOL>, grid, WARPS_TERMS * 32, fast);
         mark(2);
     } else if constexpr (sizeof(R) == 4) {
@@ -2189,6 +2130,5 @@ cudaError_t launch_atoms_t(const AtomArgs& a, bool grad, cudaStream_t s) {
     mark(3);
     return go.err != cudaSuccess ? go.err : cudaGetLastError();
 }
-#endif
 
 }  // namespace dsasa
