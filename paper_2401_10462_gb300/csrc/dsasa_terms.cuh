@@ -306,13 +306,26 @@ __global__ void __launch_bounds__(WARPS_TERMS * 32, TermBlocks<R>::value) k_term
 
     // ---------------- exterior triangles: c_iab S_iab^(i) (Eq. trianglev) and the gradient of the
     // triangle terms of i, a and b (Eq. triangle) and of the dihedral (wing) terms that do not
-    // cancel.  Mixed form: with the gradient, four lanes per triangle: parts 0-2 evaluate the
-    // lens gradient of owner i, a or b (one call on all those lanes), part 3 the area term;
-    // part 0 adds the wing dihedral term when one tetrahedron of C holds the triangle
+    // cancel.  Mixed form: one lane per triangle for the area term, then three for the gradient
+    // (lanes 30 and 31 idle), the lens gradients of the owners i, a and b; part 0 adds the wing
+    // dihedral term when one tetrahedron of C holds the triangle
     if constexpr (FFM) {
-        constexpr int GT = GRAD ? 4 : 1;
-        for (int j = lane; j < GT * nt; j += 32) {
-            const int e = j / GT, part = GRAD ? (j & 3) : 3;
+        for (int j = lane; j < nt; j += 32) {
+            const int t = S->tri[j] >> 2, k = S->tri[j] & 3;
+            const uchar4 v = S->tv[t];
+            const int a = tv_get(v, k), b = tv_get(v, (k + 1) % 3);
+            const int nk = (v.w == 1) + (S->tv[tv_get(S->ta[t], k) & 63].w == 1);
+            const float cff = 1.f - 0.5f * (float)nk;
+            const int ga = DS_IDX(S->pg[a & 63], A.n, A.status), gb = DS_IDX(S->pg[b & 63], A.n, A.status);
+            const float2 ra2 = A.Rhl[ga], rb2 = A.Rhl[gb];
+            const FF Ra = {ra2.x, ra2.y}, Rb = {rb2.x, rb2.y};
+            const FF x = tri_term_ff(pos(a), pos(b), Ri_ff, Ra, Rb, Ri2_ff, -1.f);
+            acc_ff = ff_add(acc_ff, FF{cff * x.h, cff * x.l});
+            cf_sum += cff;
+        }
+        if constexpr (GRAD)
+        for (int j = lane < 30 ? lane : 3 * nt; j < 3 * nt; j += 30) {
+            const int e = j / 3, part = j - 3 * e;
             const int t = S->tri[e] >> 2, k = S->tri[e] & 3;
             const uchar4 v = S->tv[t];
             const uint8_t a = tv_get(v, k), b = tv_get(v, (k + 1) % 3), cc = tv_get(v, (k + 2) % 3);
@@ -324,11 +337,6 @@ __global__ void __launch_bounds__(WARPS_TERMS * 32, TermBlocks<R>::value) k_term
             const int ga = DS_IDX(S->pg[a & 63], A.n, A.status), gb = DS_IDX(S->pg[b & 63], A.n, A.status);
             const float2 ra2 = A.Rhl[ga], rb2 = A.Rhl[gb];
             const FF Ra = {ra2.x, ra2.y}, Rb = {rb2.x, rb2.y};
-            if (part == 3) {
-                const FF x = tri_term_ff(pa, pb, Ri_ff, Ra, Rb, Ri2_ff, -1.f);
-                acc_ff = ff_add(acc_ff, FF{cff * x.h, cff * x.l});
-                cf_sum += cff;
-            }
             const R Raf = Ra.h, Rbf = Rb.h, dRab = ff_mul(ff_sub(Ra, Rb), ff_add(Ra, Rb)).h;
             if (GRAD && part < 3) {
                 const P3<R> O = {zero, zero, zero};
