@@ -925,7 +925,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                     if (lane < 9) {
                         const int z = cz + lane / 3 - 1, y = cy + lane % 3 - 1;
                         if (z >= 0 && z < G.dims[2] && y >= 0 && y < G.dims[1]) {
-                            const int row = G.base + (z * G.dims[1] + y) * G.dims[0];
+                            const int row = grid_row(G, z, y);
                             const int x0 = max(cx - 1, 0), x1 = min(cx + 1, G.dims[0] - 1);
                             rbeg = A.cstart[row + x0];
                             rend = A.cstart[row + x1 + 1];
@@ -969,7 +969,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                         for (int dy = -1; dy <= 1; ++dy) {
                             int y = cy + dy;
                             if (y < 0 || y >= G.dims[1]) continue;
-                            int row = G.base + (z * G.dims[1] + y) * G.dims[0];
+                            int row = grid_row(G, z, y);
                             int x0 = max(cx - 1, 0), x1 = min(cx + 1, G.dims[0] - 1);
                             gather_range(A.cstart[row + x0], A.cstart[row + x1 + 1]);
                         }

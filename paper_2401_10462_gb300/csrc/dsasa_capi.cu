@@ -72,8 +72,7 @@ struct dsasa_ctx {
     MolGrid* grids = nullptr;
     int* counts = nullptr;
     int* cstart = nullptr;
-    int* blocksums = nullptr;
-    unsigned* bsync = nullptr;   // single-molecule build: partial boxes + ticket (zero between calls)
+    unsigned* bsync = nullptr;   // exchange area of the cell-list build
     long long* offsets = nullptr;
     int* defer = nullptr;       // atoms the fast kernel pass defers to the large pass
     int* redo = nullptr;        // atoms whose cell the carry kernel could not keep
@@ -89,7 +88,7 @@ struct dsasa_ctx {
     int* nbn = nullptr;
     double* ref_xyz = nullptr;
     double* ref_rad = nullptr;
-    int* vstate = nullptr;        // [0] max displacement^2 (float bits), [1] radii changed, [2] reuse, [3] overflow
+    int* vstate = nullptr;        // [0] max displacement^2 (float bits), [1] radii changed, [2] reuse, [3] overflow, [4] ticket
     int64_t lists_n = 0;          // the lists hold this many atoms of the last single-molecule call
     double lists_probe = -1.0;
     int* status = nullptr;      // [0] status bits, [1] total cells, [2] deferred count, [3] redo count
@@ -135,7 +134,7 @@ template <class T> void dfree(T*& p) {
 
 void free_scratch(dsasa_ctx* c) {
     dfree(c->R); dfree(c->Rhl); dfree(c->f4); dfree(c->molid); dfree(c->rank); dfree(c->cell); dfree(c->sidx); dfree(c->sf4);
-    dfree(c->bbox); dfree(c->grids); dfree(c->counts); dfree(c->cstart); dfree(c->blocksums); dfree(c->bsync); dfree(c->offsets);
+    dfree(c->bbox); dfree(c->grids); dfree(c->counts); dfree(c->cstart); dfree(c->bsync); dfree(c->offsets);
     dfree(c->defer); dfree(c->redo); dfree(c->cells); dfree(c->mol_base); dfree(c->mol_reuse); dfree(c->vmol); dfree(c->mol_done);
     dfree(c->nbl); dfree(c->nbn); dfree(c->ref_xyz); dfree(c->ref_rad); dfree(c->vstate);
     c->lists_n = 0;
@@ -164,22 +163,27 @@ dsasa_status ensure(dsasa_ctx* c, int64_t n, int64_t n_mol) {
     if (c->cfg.max_atoms > 0) { na = std::max<int64_t>(n, c->cfg.max_atoms); nm = std::max<int64_t>(nm, 4096); }
     int64_t nc = cells_for(na, nm);
     if (c->cfg.max_cells > 0 && c->cfg.max_cells < nc) nc = std::max<int64_t>(c->cfg.max_cells, 64);
-    int64_t nbs = (int64_t)scan_scratch_ints((int)nc) + 16;
 #define ALLOC(ptr, count)                                                               \
     e = dev_alloc((void**)&c->ptr, sizeof(*c->ptr) * (size_t)(count));                 \
     if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "cudaMalloc " #ptr); }
     ALLOC(R, na) ALLOC(Rhl, na) ALLOC(f4, na) ALLOC(molid, na) ALLOC(rank, na) ALLOC(cell, na) ALLOC(sidx, na) ALLOC(sf4, na)
-    ALLOC(bbox, 8 * nm) ALLOC(grids, nm) ALLOC(counts, nc + 1) ALLOC(cstart, nc + 1) ALLOC(blocksums, nbs)
+    ALLOC(bbox, 8 * nm) ALLOC(grids, nm) ALLOC(counts, nc + 1) ALLOC(cstart, nc + 1)
     ALLOC(offsets, nm + 1) ALLOC(defer, na) ALLOC(redo, na) ALLOC(cells, na * (int64_t)cell_record_bytes()) ALLOC(bsync, BUILD_SYNC_WORDS)
-    ALLOC(mol_base, nm) ALLOC(mol_reuse, nm) ALLOC(vmol, 3 * nm) ALLOC(mol_done, nm)
+    ALLOC(mol_base, nm) ALLOC(mol_reuse, nm) ALLOC(vmol, 3 * nm + 1) ALLOC(mol_done, nm)
+    // what the kernels expect to be zero, and leave zero
     e = cudaMemsetAsync(c->bsync, 0, sizeof(unsigned) * BUILD_SYNC_WORDS, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->bbox, 0, sizeof(unsigned) * 8 * (size_t)nm, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->counts, 0, sizeof(int) * (size_t)(nc + 1), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->vmol, 0, sizeof(int) * (3 * (size_t)nm + 1), c->stream);
     if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "memset"); }
     if (c->cfg.skin > 0.0) {
-        ALLOC(nbl, na * NBL_CAP) ALLOC(nbn, na) ALLOC(ref_xyz, 3 * na) ALLOC(ref_rad, na) ALLOC(vstate, 4)
-        e = cudaMemsetAsync(c->vstate, 0, 4 * sizeof(int), c->stream);
+        ALLOC(nbl, na * NBL_CAP) ALLOC(nbn, na) ALLOC(ref_xyz, 3 * na) ALLOC(ref_rad, na) ALLOC(vstate, 8)
+        e = cudaMemsetAsync(c->vstate, 0, 8 * sizeof(int), c->stream);
         if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "memset"); }
     }
 #undef ALLOC
+    e = cudaStreamSynchronize(c->stream);   // cleared before a call on any stream
+    if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "memset"); }
     c->cap_atoms = na;
     c->cap_mol = nm;
     c->cap_cells = nc;
@@ -202,7 +206,7 @@ cudaError_t build_cells(dsasa_ctx* c, const double* coords, const double* radii,
     b.max_cells = (int)c->cap_cells;
     b.R = c->R; b.Rhl = c->Rhl; b.f4 = c->f4; b.molid = c->molid; b.rank = c->rank; b.cell = c->cell;
     b.bbox = c->bbox; b.grids = c->grids; b.counts = c->counts; b.cstart = c->cstart; b.sidx = c->sidx;
-    b.sf4 = c->sf4; b.blocksums = c->blocksums; b.sync = c->bsync; b.zero_word = zero_word; b.status = c->status; b.ncells_out = c->status + 1;
+    b.sf4 = c->sf4; b.sync = c->bsync; b.zero_word = zero_word; b.status = c->status; b.ncells_out = c->status + 1;
     return launch_build(b, c->stream);
 }
 
@@ -584,7 +588,8 @@ dsasa_status dsasa_compute_batch_resident(dsasa_ctx* c, dsasa_arena* arena, int 
                             c->stream);
         if (e == cudaSuccess)
             e = launch_verlet_check_batch(coords, radii, arena->ref_xyz, arena->ref_rad, arena->nbn, c->offsets,
-                                          c->mol_base, (int)n, n_mol, c->cfg.skin, c->vmol, c->mol_reuse, c->stream);
+                                          c->mol_base, (int)n, n_mol, c->cfg.skin, c->vmol,
+                                          (unsigned*)c->vmol + 3 * c->cap_mol, c->mol_reuse, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "resident list check");
         bx.arena = arena;
     }

@@ -2,10 +2,15 @@
 //
 // Atoms are binned per molecule into cubic cells of edge >= 2 R_max + skin + slack, so every
 // pair of overlapping balls |p_i - p_j| < R_i + R_j lies in the same or adjacent cells.  The
-// binning is a counting sort (atomic counts -> exclusive scan -> scatter); the order inside a
-// cell is not deterministic, which is harmless because each atom later sorts its candidate
-// list by (plane distance, atom index).  The sorted float4 copy (x, y, z, R) gives coalesced
-// neighbour-tile loads in the atom kernel.
+// binning is a counting sort in four kernels that start early behind one another (programmatic
+// dependent launch): input pass, bounding boxes and grids (the last block makes the grids, so
+// nothing waits); counts; starts; scatter.  The neighbour search reads runs of up to three cells
+// that are adjacent along x, so only the cells of one row (fixed y, z) need consecutive starts:
+// a row takes its place in the sorted order with one atomic add and needs no scan over all
+// cells.  The order of rows and of the atoms inside a cell is not deterministic, which is
+// harmless because each atom later sorts its candidate list by (plane distance, atom index).
+// The sorted float4 copy (x, y, z, R) gives coalesced neighbour-tile loads in the atom kernel.
+// Bound: the latency of the dependent launches and of their atomics.
 #include "dsasa_kernels.cuh"
 
 #include <math.h>
@@ -22,31 +27,16 @@ __device__ __forceinline__ float fdec(unsigned u) {
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
-__global__ void k_bbox_init(unsigned* bbox, int n_mol, int* zero_word) {
-    int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m == 0 && zero_word) { zero_word[0] = 0; zero_word[1] = 0; }
-    if (m >= n_mol) return;
-    unsigned lo = fenc(INFINITY), hi = fenc(-INFINITY);
-    for (int k = 0; k < 3; ++k) { bbox[8 * m + k] = lo; bbox[8 * m + 3 + k] = hi; }
-    bbox[8 * m + 6] = fenc(0.0f);
-    bbox[8 * m + 7] = 0;
+// The box of a molecule in 7 words that atomicMax grows from zero: ~min x y z, max x y z, max R
+// (fenc of a finite float is above zero, and so is its complement).
+__device__ __forceinline__ void box_words(float4 f, unsigned* w) {
+    w[0] = ~fenc(f.x); w[1] = ~fenc(f.y); w[2] = ~fenc(f.z);
+    w[3] = fenc(f.x); w[4] = fenc(f.y); w[5] = fenc(f.z);
+    w[6] = fenc(f.w);
 }
 
-__global__ void k_prep(BuildArgs a) {
-    if (a.skip && *a.skip) return;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool act = i < a.n;
-    const unsigned mask = __ballot_sync(0xffffffffu, act);
-    if (!act) return;
-    int m = 0;
-    if (a.offsets) {
-        int lo = 0, hi = a.n_mol - 1;   // last m with offsets[m] <= i
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (a.offsets[mid] <= i) lo = mid; else hi = mid - 1;
-        }
-        m = lo;
-    }
+// atom i's input pass: inflated radius, float copies; non-finite inputs are replaced and reported
+__device__ __forceinline__ float4 prep_atom(const BuildArgs& a, int i, int m) {
     double x = a.xyz[3 * i], y = a.xyz[3 * i + 1], z = a.xyz[3 * i + 2];
     double R = a.radii[i] + a.probe;
     if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(R)) || !(R > 0.0)) {
@@ -55,46 +45,40 @@ __global__ void k_prep(BuildArgs a) {
         R = 1.0;
     }
     a.R[i] = R;
-    { float h = (float)R; a.Rhl[i] = make_float2(h, (float)(R - (double)h)); }
+    const float h = (float)R;
+    a.Rhl[i] = make_float2(h, (float)(R - (double)h));
     a.molid[i] = m;
-    float4 f = make_float4((float)x, (float)y, (float)z, (float)R);
+    const float4 f = make_float4((float)x, (float)y, (float)z, h);
     a.f4[i] = f;
-    // bounding box of the molecule: reduced over the warp first when its atoms share one
-    // molecule (one atomic per warp instead of one per atom on the same 7 words)
-    unsigned lo3[3] = {fenc(f.x), fenc(f.y), fenc(f.z)};
-    unsigned hi4[4] = {lo3[0], lo3[1], lo3[2], fenc(f.w)};
-    const int first = __ffs(mask) - 1;
-    const int m0 = __shfl_sync(mask, m, first);
-    unsigned* bb = a.bbox + 8 * m;
-    if (__all_sync(mask, m == m0)) {
-        for (int k = 0; k < 3; ++k) lo3[k] = __reduce_min_sync(mask, lo3[k]);
-        for (int k = 0; k < 4; ++k) hi4[k] = __reduce_max_sync(mask, hi4[k]);
-        if ((int)(threadIdx.x & 31) != first) return;
-    }
-    atomicMin(bb + 0, lo3[0]);
-    atomicMin(bb + 1, lo3[1]);
-    atomicMin(bb + 2, lo3[2]);
-    atomicMax(bb + 3, hi4[0]);
-    atomicMax(bb + 4, hi4[1]);
-    atomicMax(bb + 5, hi4[2]);
-    atomicMax(bb + 6, hi4[3]);
+    return f;
 }
 
-// Grid of one molecule from its encoded bounding box (bb: min x y z, max x y z, max R) and
-// atom count: cell size and dimensions; the cell count is returned in base.
+// the molecule of atom i: the last m with offsets[m] <= i
+__device__ __forceinline__ int molecule_of(const long long* offsets, int n_mol, int i) {
+    int lo = 0, hi = n_mol - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (offsets[mid] <= i) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Grid of one molecule from its box (box_words) and atom count: cell size and dimensions; the
+// cell count is returned in base, with one more entry per row of cells for the row's end.
 __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
     MolGrid g;
     if (nm <= 0) {
-        for (int k = 0; k < 3; ++k) { g.lo[k] = 0.f; g.dims[k] = 1; }
+        for (int k = 0; k < 3; ++k) { g.lo[k] = 0.f; g.dims[k] = 0; }
         g.inv_cell = 1.f;
         g.margin = 0.f;
         g.rmax = 0.f;
-        g.base = 1;
+        g.base = 0;
+        g.row0 = 0;
         return g;
     }
     float lo[3], hi[3], amax = 0.f;
     for (int k = 0; k < 3; ++k) {
-        lo[k] = fdec(bb[k]);
+        lo[k] = fdec(~bb[k]);
         hi[k] = fdec(bb[3 + k]);
         amax = fmaxf(amax, fmaxf(fabsf(lo[k]), fabsf(hi[k])));
     }
@@ -108,7 +92,7 @@ __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
         double prod = 1.0;
         for (int k = 0; k < 3; ++k) {
             dims[k] = (int)fminf((hi[k] - lo[k]) / cell, 1e6f) + 1;
-            prod *= dims[k];
+            prod *= dims[k] + (k == 0);
         }
         if (prod <= cap) break;
         cell *= (float)fmax(1.01, cbrt(prod / cap) * 1.01);
@@ -117,256 +101,254 @@ __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
     g.inv_cell = 1.0f / cell;
     g.margin = margin + (float)skin;   // candidates within R_i + R_j + skin (Verlet lists)
     g.rmax = rmax;
-    g.base = dims[0] * dims[1] * dims[2];
+    g.base = (dims[0] + 1) * dims[1] * dims[2];
+    g.row0 = 0;
     return g;
-}
-
-// per molecule: cell size and dimensions (cell count stored in base for the scan below)
-__global__ void k_grid_local(BuildArgs a) {
-    if (a.skip && *a.skip) return;
-    int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= a.n_mol) return;
-    long long nm = a.offsets ? (a.offsets[m + 1] - a.offsets[m]) : a.n;
-    a.grids[m] = make_grid(a.bbox + 8 * m, nm, a.skin);
-}
-
-// exclusive scan of the per-molecule cell counts (one block)
-__global__ void k_grid_scan(BuildArgs a) {
-    if (a.skip && *a.skip) return;
-    __shared__ int carry;
-    __shared__ int ws[32];
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int b0 = 0; b0 < a.n_mol; b0 += blockDim.x) {
-        int m = b0 + threadIdx.x;
-        int v = m < a.n_mol ? a.grids[m].base : 0;
-        int x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, x, o);
-            if ((threadIdx.x & 31) >= o) x += y;
-        }
-        if ((threadIdx.x & 31) == 31) ws[threadIdx.x >> 5] = x;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            int s = threadIdx.x < (blockDim.x >> 5) ? ws[threadIdx.x] : 0;
-            for (int o = 1; o < 32; o <<= 1) {
-                int y = __shfl_up_sync(0xffffffffu, s, o);
-                if (threadIdx.x >= o) s += y;
-            }
-            ws[threadIdx.x] = s;
-        }
-        __syncthreads();
-        int wpre = (threadIdx.x >= 32) ? ws[(threadIdx.x >> 5) - 1] : 0;
-        int excl = carry + wpre + x - v;
-        if (m < a.n_mol) a.grids[m].base = excl;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = excl + v;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        *a.ncells_out = carry;
-        if (carry > a.max_cells) atomicOr(a.status, ST_GRID_OVF);
-    }
 }
 
 __device__ __forceinline__ int cell_of(const MolGrid& g, float4 f) {
     int cx = min(max((int)floorf((f.x - g.lo[0]) * g.inv_cell), 0), g.dims[0] - 1);
     int cy = min(max((int)floorf((f.y - g.lo[1]) * g.inv_cell), 0), g.dims[1] - 1);
     int cz = min(max((int)floorf((f.z - g.lo[2]) * g.inv_cell), 0), g.dims[2] - 1);
-    return g.base + (cz * g.dims[1] + cy) * g.dims[0] + cx;
+    return grid_row(g, cz, cy) + cx;
 }
 
-__global__ void k_count(BuildArgs a) {
+constexpr int PREP_T = 256;
+
+// exclusive sums of v and w over the block's threads (in thread order) and their totals
+__device__ void block_excl_scan2(int v, int w, int& ev, int& ew, int& tv, int& tw) {
+    __shared__ int sv[PREP_T / 32], sw[PREP_T / 32];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    int x = v, y = w;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int p = __shfl_up_sync(0xffffffffu, x, o), q = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= o) { x += p; y += q; }
+    }
+    if (lane == 31) { sv[wp] = x; sw[wp] = y; }
+    __syncthreads();
+    int pv = 0, pw = 0;
+    tv = tw = 0;
+    for (int k = 0; k < PREP_T / 32; ++k) {
+        if (k == wp) { pv = tv; pw = tw; }
+        tv += sv[k];
+        tw += sw[k];
+    }
+    ev = pv + x - v;
+    ew = pw + y - w;
+    __syncthreads();
+}
+
+// Input pass and bounding boxes; the block that finishes last makes every molecule's grid and
+// clears the boxes and the ticket for the next call.
+__global__ void __launch_bounds__(PREP_T) k_prep(BuildArgs a) {
+    grid_dep_trigger();
+    grid_dep_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (a.zero_word) { a.zero_word[0] = 0; a.zero_word[1] = 0; }
+    }
     if (a.skip && *a.skip) return;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
+    __shared__ unsigned bb[7];
+    __shared__ bool last;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid < 7) bb[tid] = 0;
+    __syncthreads();
+    const int i0 = blockIdx.x * PREP_T, i = i0 + tid;
+    // one molecule in the whole block: its box is gathered in shared memory first
+    int m = 0, mb = 0;
+    bool one = true;
+    if (a.offsets) {
+        const int i1 = min(i0 + PREP_T, a.n) - 1;
+        mb = molecule_of(a.offsets, a.n_mol, i0);
+        one = a.offsets[mb + 1] > i1;
+        m = one ? mb : molecule_of(a.offsets, a.n_mol, min(i, a.n - 1));
+    }
+    unsigned w[7] = {0, 0, 0, 0, 0, 0, 0};
+    if (i < a.n) box_words(prep_atom(a, i, m), w);
+    if (one) {
+        for (int k = 0; k < 7; ++k) {
+            const unsigned v = __reduce_max_sync(0xffffffffu, w[k]);
+            if (lane == 0) atomicMax(&bb[k], v);
+        }
+        __syncthreads();
+        if (tid < 7) atomicMax(a.bbox + 8 * mb + tid, bb[tid]);
+    } else if (i < a.n) {
+        for (int k = 0; k < 7; ++k) atomicMax(a.bbox + 8 * m + k, w[k]);
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(a.sync + BUILD_TICKET, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    int cells = 0, rows = 0;   // totals over the molecules so far
+    for (int m0 = 0; m0 < a.n_mol; m0 += PREP_T) {
+        const int mm = m0 + tid;
+        MolGrid g;
+        int nc = 0, nr = 0;
+        if (mm < a.n_mol) {
+            unsigned bx[7];
+            for (int k = 0; k < 7; ++k) {
+                bx[k] = __ldcg(a.bbox + 8 * mm + k);
+                a.bbox[8 * mm + k] = 0;
+            }
+            const long long nm = a.offsets ? (a.offsets[mm + 1] - a.offsets[mm]) : a.n;
+            g = make_grid(bx, nm, a.skin);
+            nc = g.base;
+            nr = g.dims[1] * g.dims[2];
+        }
+        int ec, er, tc, tr;
+        block_excl_scan2(nc, nr, ec, er, tc, tr);
+        if (mm < a.n_mol) {
+            g.base = cells + ec;
+            g.row0 = rows + er;
+            if (g.base + nc > a.max_cells) {   // reported below; an empty grid keeps every index in range
+                for (int k = 0; k < 3; ++k) g.dims[k] = 0;
+                g.base = 0;
+            }
+            a.grids[mm] = g;
+        }
+        cells += tc;
+        rows += tr;
+    }
+    if (tid == 0) {
+        *a.ncells_out = cells;
+        a.sync[BUILD_ROWS] = (unsigned)rows;
+        a.sync[BUILD_CURSOR] = 0u;
+        a.sync[BUILD_TICKET] = 0u;
+        if (cells > a.max_cells) atomicOr(a.status, ST_GRID_OVF);
+    }
+}
+
+// each atom's cell and its rank there (the counts are zero when this starts)
+__global__ void k_count(BuildArgs a) {
+    grid_dep_trigger();
+    grid_dep_wait();
+    if (a.skip && *a.skip) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= a.n || *a.ncells_out > a.max_cells) return;
     const MolGrid g = a.grids[a.molid[i]];
-    int c = cell_of(g, a.f4[i]);
-    if (c >= a.max_cells) c = a.max_cells - 1;   // only after a reported overflow
+    const int c = cell_of(g, a.f4[i]);
     a.cell[i] = c;
     a.rank[i] = atomicAdd(&a.counts[c], 1);
 }
 
-// ---- exclusive scan of counts[0..len) into cstart (3 phases, tile = 256 threads x 16)
-constexpr int SCAN_T = 256, SCAN_V = 16, SCAN_TILE = SCAN_T * SCAN_V;
-
-__device__ int block_excl_scan(int v, int* total) {
-    __shared__ int ws[SCAN_T / 32];
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) ws[w] = x;
-    __syncthreads();
-    if (w == 0) {
-        int s = lane < SCAN_T / 32 ? ws[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
+// the starts of every row's cells, one warp per row; the counts are zero again afterwards
+__global__ void __launch_bounds__(256) k_rows(BuildArgs a) {
+    grid_dep_trigger();
+    grid_dep_wait();
+    if (a.skip && *a.skip) return;
+    if (*a.ncells_out > a.max_cells) return;
+    const int rows = (int)a.sync[BUILD_ROWS];
+    const int lane = threadIdx.x & 31;
+    for (int r = (blockIdx.x * 256 + threadIdx.x) >> 5; r < rows; r += gridDim.x * 8) {
+        int lo = 0, hi = a.n_mol - 1;   // the last molecule with row0 <= r (empty ones hold no row)
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.grids[mid].row0 <= r) lo = mid; else hi = mid - 1;
         }
-        if (lane < SCAN_T / 32) ws[lane] = s;
-    }
-    __syncthreads();
-    int pre = (w > 0 ? ws[w - 1] : 0) + x - v;
-    *total = ws[SCAN_T / 32 - 1];
-    __syncthreads();
-    return pre;
-}
-
-__global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const int* in, int len, int* bsum) {
-    int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
-    int s = 0;
-    for (int k = 0; k < SCAN_V; ++k) s += (base + k < len) ? in[base + k] : 0;
-    int tot;
-    block_excl_scan(s, &tot);
-    if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
-}
-__global__ void __launch_bounds__(SCAN_T) k_scan_top(int* bsum, int nb) {
-    __shared__ int carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int b0 = 0; b0 < nb; b0 += SCAN_T) {
-        int v = (b0 + threadIdx.x < nb) ? bsum[b0 + threadIdx.x] : 0;
-        int tot;
-        int pre = block_excl_scan(v, &tot);
-        if (b0 + threadIdx.x < nb) bsum[b0 + threadIdx.x] = carry + pre;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += tot;
-        __syncthreads();
-    }
-}
-__global__ void __launch_bounds__(SCAN_T) k_scan_down(const int* in, int len, const int* bsum, int* out) {
-    int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
-    int v[SCAN_V];
-    int s = 0;
-    for (int k = 0; k < SCAN_V; ++k) { v[k] = (base + k < len) ? in[base + k] : 0; s += v[k]; }
-    int tot;
-    int pre = block_excl_scan(s, &tot) + bsum[blockIdx.x];
-    for (int k = 0; k < SCAN_V; ++k) {
-        if (base + k <= len) out[base + k] = pre;   // out has len + 1 entries
-        pre += v[k];
+        const int d0 = a.grids[lo].dims[0];
+        const int c0 = a.grids[lo].base + (r - a.grids[lo].row0) * (d0 + 1);
+        int tot = 0;
+        for (int x = lane; x < d0; x += 32) tot += a.counts[c0 + x];
+        tot = __reduce_add_sync(0xffffffffu, tot);
+        int pos = 0;
+        if (lane == 0) pos = (int)atomicAdd(a.sync + BUILD_CURSOR, (unsigned)tot);
+        pos = __shfl_sync(0xffffffffu, pos, 0);
+        for (int x0 = 0; x0 <= d0; x0 += 32) {   // entry d0: the row's end
+            const int x = x0 + lane;
+            const int v = x < d0 ? a.counts[c0 + x] : 0;
+            int y = v;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int p = __shfl_up_sync(0xffffffffu, y, o);
+                if (lane >= o) y += p;
+            }
+            if (x <= d0) a.cstart[c0 + x] = pos + y - v;
+            if (x < d0) a.counts[c0 + x] = 0;
+            pos += __shfl_sync(0xffffffffu, y, 31);
+        }
     }
 }
 
 __global__ void k_scatter(BuildArgs a) {
     grid_dep_trigger();
+    grid_dep_wait();
     if (a.skip && *a.skip) return;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.n) return;
-    int pos = a.cstart[a.cell[i]] + a.rank[i];
+    const int pos = *a.ncells_out > a.max_cells ? i : a.cstart[a.cell[i]] + a.rank[i];
     a.sidx[pos] = i;
     a.sf4[pos] = a.f4[i];
 }
 
-// The whole build for one molecule of at most kSmallAtoms atoms in one kernel (the
-// multi-kernel path's launch overheads dominate at that size).  Same grid, same cells.  One
-// thread per atom for the input pass (its FP64 work and conversions spread over several SMs);
-// each block leaves its partial bounding box in a.sync and takes a ticket, and the block that
-// takes the last ticket (nothing waits) finishes the build: box, grid, counting sort in shared
-// memory, scan, scatter.  It then resets the ticket for the next call.
-constexpr int kSmallAtoms = 16384, kSmallT = 1024, kSmallCells = 8192, kSmallBlocks = kSmallAtoms / kSmallT;
-static_assert(kSmallBlocks * 8 + 1 <= BUILD_SYNC_WORDS, "block-exchange area too small");
-__device__ __forceinline__ unsigned box_init(int k) {
-    return k < 3 ? fenc(INFINITY) : (k < 6 ? fenc(-INFINITY) : (k == 6 ? fenc(0.0f) : 0u));
-}
+// The whole build for one molecule of at most kSmallAtoms atoms in one block (below that size
+// the launches of the four kernels cost more than their width gains).  Same grid, same cells;
+// counts in shared memory, starts by one scan over all cells (which also ends every row where
+// the next one starts).
+constexpr int kSmallT = 1024, kSmallAtoms = 2 * kSmallT, kSmallCells = 8 * kSmallAtoms + 64;
 __global__ void __launch_bounds__(kSmallT) k_build_small(BuildArgs a) {
-    if (blockIdx.x == 0 && threadIdx.x == 0 && a.zero_word) { a.zero_word[0] = 0; a.zero_word[1] = 0; }
     grid_dep_trigger();
+    grid_dep_wait();
+    if (threadIdx.x == 0 && a.zero_word) { a.zero_word[0] = 0; a.zero_word[1] = 0; }
     if (a.skip && *a.skip) return;
-    __shared__ unsigned bb[8];
+    __shared__ unsigned bb[7];
     __shared__ MolGrid g;
     __shared__ int ws[kSmallT / 32];
-    __shared__ int scount[kSmallCells];
-    __shared__ bool last;
+    extern __shared__ int cnt[];   // kSmallCells + 1
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    if (tid < 8) bb[tid] = box_init(tid);
+    if (tid < 7) bb[tid] = 0;
     __syncthreads();
-    unsigned lo[3] = {fenc(INFINITY), fenc(INFINITY), fenc(INFINITY)};
-    unsigned hi[4] = {fenc(-INFINITY), fenc(-INFINITY), fenc(-INFINITY), fenc(0.0f)};
-    {
-        const int i = blockIdx.x * kSmallT + tid;
+    float4 f[2];
+    unsigned bw[7] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int i = tid + h * kSmallT;
         if (i < a.n) {
-            double x = a.xyz[3 * i], y = a.xyz[3 * i + 1], z = a.xyz[3 * i + 2];
-            double R = a.radii[i] + a.probe;
-            if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(R)) || !(R > 0.0)) {
-                atomicOr(a.status, ST_INPUT);
-                x = y = z = 0.0;
-                R = 1.0;
-            }
-            a.R[i] = R;
-            { float h = (float)R; a.Rhl[i] = make_float2(h, (float)(R - (double)h)); }
-            a.molid[i] = 0;
-            float4 f = make_float4((float)x, (float)y, (float)z, (float)R);
-            a.f4[i] = f;
-            unsigned e[4] = {fenc(f.x), fenc(f.y), fenc(f.z), fenc(f.w)};
-            for (int k = 0; k < 3; ++k) { lo[k] = min(lo[k], e[k]); hi[k] = max(hi[k], e[k]); }
-            hi[3] = max(hi[3], e[3]);
+            f[h] = prep_atom(a, i, 0);
+            unsigned v[7];
+            box_words(f[h], v);
+            for (int k = 0; k < 7; ++k) bw[k] = max(bw[k], v[k]);
         }
     }
-    for (int k = 0; k < 3; ++k) {
-        lo[k] = __reduce_min_sync(0xffffffffu, lo[k]);
-        hi[k] = __reduce_max_sync(0xffffffffu, hi[k]);
+    for (int k = 0; k < 7; ++k) {
+        const unsigned v = __reduce_max_sync(0xffffffffu, bw[k]);
+        if (lane == 0) atomicMax(&bb[k], v);
     }
-    hi[3] = __reduce_max_sync(0xffffffffu, hi[3]);
-    if (lane == 0) {
-        for (int k = 0; k < 3; ++k) { atomicMin(&bb[k], lo[k]); atomicMax(&bb[3 + k], hi[k]); }
-        atomicMax(&bb[6], hi[3]);
-    }
-    __syncthreads();
-    // partial box out, every thread's writes made visible, then the ticket
-    if (tid < 8) a.sync[8 * blockIdx.x + tid] = bb[tid];
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(a.sync + 8 * kSmallBlocks, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    if (tid < 8) {
-        unsigned v = box_init(tid);
-        for (int b = 0; b < (int)gridDim.x; ++b) {
-            const unsigned p = __ldcg(a.sync + 8 * b + tid);
-            v = tid < 3 ? min(v, p) : (tid < 7 ? max(v, p) : 0u);
-        }
-        bb[tid] = v;
-    }
-    if (tid == 0) a.sync[8 * kSmallBlocks] = 0u;   // ticket back to zero for the next call
     __syncthreads();
     if (tid == 0) {
         MolGrid gg = make_grid(bb, a.n, a.skin);
         const int ncells = gg.base;
         gg.base = 0;
+        if (ncells > a.max_cells) {   // an empty grid keeps every index in range
+            for (int k = 0; k < 3; ++k) gg.dims[k] = 0;
+            atomicOr(a.status, ST_GRID_OVF);
+        }
         g = gg;
         a.grids[0] = gg;
         *a.ncells_out = ncells;
-        if (ncells > a.max_cells) atomicOr(a.status, ST_GRID_OVF);
-        for (int k = 0; k < 8; ++k) a.bbox[k] = bb[k];
     }
     __syncthreads();
-    const int ncells = min(g.dims[0] * g.dims[1] * g.dims[2], a.max_cells);
-    // counts in shared memory when the grid is small enough (the usual case), else in HBM
-    const bool sm = ncells + 1 <= kSmallCells;
-    int* cnt = sm ? scount : a.counts;
+    const bool ovf = g.dims[0] == 0;
+    const int ncells = (g.dims[0] + 1) * g.dims[1] * g.dims[2];
     for (int c = tid; c <= ncells; c += kSmallT) cnt[c] = 0;
     __syncthreads();
-#pragma unroll 4
-    for (int i = tid; i < a.n; i += kSmallT) {
-        int c = cell_of(g, __ldcg(a.f4 + i));   // written by other blocks of this grid
-        if (c >= a.max_cells) c = a.max_cells - 1;   // only after a reported overflow
-        a.cell[i] = c;
-        a.rank[i] = atomicAdd(&cnt[c], 1);
+    int cell[2], rank[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (tid + h * kSmallT < a.n && !ovf) {
+            cell[h] = cell_of(g, f[h]);
+            rank[h] = atomicAdd(&cnt[cell[h]], 1);
+        }
     }
     __syncthreads();
-    // exclusive scan of counts[0 .. ncells] into cstart: each thread scans a contiguous run
-    // of cells, one block scan over the run totals (the shared copy keeps the starts)
+    // exclusive scan of the counts: each thread scans a contiguous run of cells, one block scan
+    // over the run totals
     const int per = (ncells + 1 + kSmallT - 1) / kSmallT;
     const int c0 = min(tid * per, ncells + 1), c1 = min(c0 + per, ncells + 1);
     int run = 0;
-    for (int c = c0; c < c1; ++c) run += c < ncells ? cnt[c] : 0;
+    for (int c = c0; c < c1; ++c) run += cnt[c];
     int x = run;
     for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= o) x += y;
     }
     if (lane == 31) ws[w] = x;
@@ -374,7 +356,7 @@ __global__ void __launch_bounds__(kSmallT) k_build_small(BuildArgs a) {
     if (w == 0) {
         int t = ws[lane];
         for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, t, o);
+            const int y = __shfl_up_sync(0xffffffffu, t, o);
             if (lane >= o) t += y;
         }
         ws[lane] = t;
@@ -382,52 +364,66 @@ __global__ void __launch_bounds__(kSmallT) k_build_small(BuildArgs a) {
     __syncthreads();
     int pre = (w > 0 ? ws[w - 1] : 0) + x - run;
     for (int c = c0; c < c1; ++c) {
-        const int v = c < ncells ? cnt[c] : 0;
-        a.cstart[c] = pre;
-        if (sm) cnt[c] = pre;
+        const int v = cnt[c];
+        if (c < ncells) a.cstart[c] = pre;
+        cnt[c] = pre;
         pre += v;
     }
     __syncthreads();
-#pragma unroll 4
-    for (int i = tid; i < a.n; i += kSmallT) {
-        int pos = (sm ? cnt[a.cell[i]] : a.cstart[a.cell[i]]) + a.rank[i];
-        a.sidx[pos] = i;
-        a.sf4[pos] = __ldcg(a.f4 + i);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int i = tid + h * kSmallT;
+        if (i < a.n) {
+            const int pos = ovf ? i : cnt[cell[h]] + rank[h];
+            a.sidx[pos] = i;
+            a.sf4[pos] = f[h];
+        }
     }
 }
 
-cudaError_t launch_build_multi(const BuildArgs& a, cudaStream_t s) {
-    const int T = 256;
-    int nb = (a.n + T - 1) / T;
-    k_bbox_init<<<(a.n_mol + T - 1) / T, T, 0, s>>>(a.bbox, a.n_mol, a.zero_word);
-    k_prep<<<nb, T, 0, s>>>(a);
-    k_grid_local<<<(a.n_mol + T - 1) / T, T, 0, s>>>(a);
-    k_grid_scan<<<1, 1024, 0, s>>>(a);
-    cudaMemsetAsync(a.counts, 0, sizeof(int) * (size_t)(a.max_cells + 1), s);
-    k_count<<<nb, T, 0, s>>>(a);
-    int len = a.max_cells;   // scan the whole capacity: cells past the used range are zero
-    int nt = (len + 1 + SCAN_TILE - 1) / SCAN_TILE;
-    k_scan_reduce<<<nt, SCAN_T, 0, s>>>(a.counts, len, a.blocksums);
-    k_scan_top<<<1, SCAN_T, 0, s>>>(a.blocksums, nt);
-    k_scan_down<<<nt, SCAN_T, 0, s>>>(a.counts, len, a.blocksums, a.cstart);
-    k_scatter<<<nb, T, 0, s>>>(a);
-    note_launches(9);
-    return cudaGetLastError();
+cudaError_t launch_build_multi(const BuildArgs& a, bool early, cudaStream_t s) {
+    const int T = 256, nb = (a.n + T - 1) / T;
+    // rows of cells: about one for every 32 atoms of a dense molecule; each warp takes several
+    const int rb = min(nb, 1216);
+    static_assert(PREP_T == 256, "one thread per atom");
+    cudaError_t e = launch_dependent(k_prep, nb, PREP_T, s, early, a);
+    if (e == cudaSuccess) e = launch_dependent(k_count, nb, T, s, true, a);
+    if (e == cudaSuccess) e = launch_dependent(k_rows, rb, T, s, true, a);
+    if (e == cudaSuccess) e = launch_dependent(k_scatter, nb, T, s, true, a);
+    note_launches(4);
+    return e;
 }
 
 }  // namespace
 
-size_t scan_scratch_ints(int max_cells) { return (size_t)(max_cells + 1 + SCAN_TILE - 1) / SCAN_TILE + 1; }
-
 namespace {
 
-// Verlet skin test (see dsasa_kernels.cuh)
-__global__ void k_verlet_check(const double* xyz, const double* radii, const double* ref_xyz, const double* ref_rad,
-                               int n, int* vstate) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+constexpr int CHECK_T = 256;
+
+// whether this block is the last of the grid to come here (every thread's writes before it are
+// visible to the last block after it); the ticket is zero again for the next call
+__device__ bool last_block(unsigned* ticket) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+        if (last) *ticket = 0;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
+// Verlet skin test (see dsasa_kernels.cuh): the largest displacement and any changed radius go
+// to vstate[0..1] (zero between calls); the last block decides and clears them.
+__global__ void __launch_bounds__(CHECK_T) k_verlet_check(const double* xyz, const double* radii, const double* ref_xyz,
+                                                          const double* ref_rad, int n, int valid, float lim2, int* vstate) {
+    grid_dep_trigger();
+    const int i = blockIdx.x * CHECK_T + threadIdx.x;
     float d2 = 0.f;
     int changed = 0;
-    if (i < n) {
+    if (valid && i < n) {
         double dx = xyz[3 * i] - ref_xyz[3 * i], dy = xyz[3 * i + 1] - ref_xyz[3 * i + 1], dz = xyz[3 * i + 2] - ref_xyz[3 * i + 2];
         double dd = dx * dx + dy * dy + dz * dz;
         d2 = (float)dd * (1.f + 1e-6f);   // rounded up: the test stays conservative
@@ -437,13 +433,14 @@ __global__ void k_verlet_check(const double* xyz, const double* radii, const dou
     const unsigned d2max = __reduce_max_sync(0xffffffffu, __float_as_uint(d2));   // d2 >= 0: bits order as values
     changed = __reduce_or_sync(0xffffffffu, changed);
     if ((threadIdx.x & 31) == 0) {
-        atomicMax((unsigned*)&vstate[0], d2max);
+        if (d2max) atomicMax((unsigned*)&vstate[0], d2max);
         if (changed) atomicOr(&vstate[1], 1);
     }
-}
-__global__ void k_verlet_decide(int* vstate, int valid, float lim2) {
-    const float d2 = __uint_as_float((unsigned)vstate[0]);
-    const int reuse = valid && vstate[1] == 0 && vstate[3] == 0 && d2 <= lim2;
+    if (!last_block((unsigned*)vstate + 4) || threadIdx.x != 0) return;
+    const float dm = __uint_as_float((unsigned)__ldcg(vstate));
+    const int reuse = valid && __ldcg(vstate + 1) == 0 && vstate[3] == 0 && dm <= lim2;
+    vstate[0] = 0;
+    vstate[1] = 0;
     vstate[2] = reuse;
     if (!reuse) vstate[3] = 0;   // the lists are rebuilt by this call
 }
@@ -451,75 +448,88 @@ __global__ void k_verlet_decide(int* vstate, int valid, float lim2) {
 // The same test for a batch of resident molecules, per molecule m (atoms [off[m], off[m+1]),
 // lists at arena slot base[m] + local index; base[m] < 0: no lists): vmol[3m] the largest
 // squared displacement since the lists were built (float bits, rounded up), vmol[3m + 1] a
-// radius changed, vmol[3m + 2] some atom has no valid list (negative length).
-__global__ void k_verlet_check_batch(const double* xyz, const double* radii, const double* ref_xyz,
-                                     const double* ref_rad, const int* nbn, const long long* off,
-                                     const long long* base, int n, int n_mol, int* vmol) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int lo = 0, hi = n_mol - 1;   // last m with off[m] <= i
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (off[mid] <= i) lo = mid; else hi = mid - 1;
+// radius changed, vmol[3m + 2] some atom has no valid list (negative length).  vmol and the
+// ticket are zero between calls.
+__global__ void __launch_bounds__(CHECK_T) k_verlet_check_batch(const double* xyz, const double* radii,
+                                                                const double* ref_xyz, const double* ref_rad,
+                                                                const int* nbn, const long long* off,
+                                                                const long long* base, int n, int n_mol, float lim2,
+                                                                int* vmol, unsigned* ticket, int* reuse) {
+    grid_dep_trigger();
+    const int i = blockIdx.x * CHECK_T + threadIdx.x;
+    int m = -1;
+    unsigned d2b = 0;
+    int changed = 0, none = 0;
+    if (i < n) {
+        m = molecule_of(off, n_mol, i);
+        if (base[m] >= 0) {
+            const size_t li = (size_t)(base[m] + (i - off[m]));
+            const double dx = xyz[3 * i] - ref_xyz[3 * li], dy = xyz[3 * i + 1] - ref_xyz[3 * li + 1],
+                         dz = xyz[3 * i + 2] - ref_xyz[3 * li + 2];
+            const double dd = dx * dx + dy * dy + dz * dz;
+            d2b = __float_as_uint(dd == dd ? (float)dd * (1.f + 1e-6f) : INFINITY);
+            changed = radii[i] != ref_rad[li];
+            none = nbn[li] < 0;
+        }
     }
-    const int m = lo;
-    if (base[m] < 0) return;
-    const size_t li = (size_t)(base[m] + (i - off[m]));
-    const double dx = xyz[3 * i] - ref_xyz[3 * li], dy = xyz[3 * i + 1] - ref_xyz[3 * li + 1],
-                 dz = xyz[3 * i + 2] - ref_xyz[3 * li + 2];
-    const double dd = dx * dx + dy * dy + dz * dz;
-    const float d2 = dd == dd ? (float)dd * (1.f + 1e-6f) : INFINITY;
-    atomicMax((unsigned*)&vmol[3 * m], __float_as_uint(d2));
-    if (radii[i] != ref_rad[li]) atomicOr(&vmol[3 * m + 1], 1);
-    if (nbn[li] < 0) atomicOr(&vmol[3 * m + 2], 1);
-}
-__global__ void k_verlet_decide_batch(const int* vmol, const long long* base, int n_mol, float lim2, int* reuse) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= n_mol) return;
-    reuse[m] = base[m] >= 0 && vmol[3 * m + 1] == 0 && vmol[3 * m + 2] == 0 &&
-               __uint_as_float((unsigned)vmol[3 * m]) <= lim2;
+    // one atomic per warp where its atoms share a molecule
+    const int m0 = __shfl_sync(0xffffffffu, m, 0);
+    if (__all_sync(0xffffffffu, m == m0)) {
+        d2b = __reduce_max_sync(0xffffffffu, d2b);
+        changed = __reduce_or_sync(0xffffffffu, changed);
+        none = __reduce_or_sync(0xffffffffu, none);
+        if (threadIdx.x & 31) m = -1;
+    }
+    if (m >= 0) {
+        if (d2b) atomicMax((unsigned*)&vmol[3 * m], d2b);
+        if (changed) atomicOr(&vmol[3 * m + 1], 1);
+        if (none) atomicOr(&vmol[3 * m + 2], 1);
+    }
+    if (!last_block(ticket)) return;
+    for (int k = threadIdx.x; k < n_mol; k += CHECK_T) {
+        reuse[k] = base[k] >= 0 && __ldcg(vmol + 3 * k + 1) == 0 && __ldcg(vmol + 3 * k + 2) == 0 &&
+                   __uint_as_float((unsigned)__ldcg(vmol + 3 * k)) <= lim2;
+        vmol[3 * k] = vmol[3 * k + 1] = vmol[3 * k + 2] = 0;
+    }
 }
 
 }  // namespace
 
 cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, const double* ref_xyz,
                                       const double* ref_rad, const int* nbn, const long long* off,
-                                      const long long* base, int n, int n_mol, double skin, int* vmol, int* reuse,
-                                      cudaStream_t s) {
-    cudaError_t e = cudaMemsetAsync(vmol, 0, sizeof(int) * 3 * (size_t)n_mol, s);
-    if (e != cudaSuccess) return e;
-    if (n > 0) {
-        k_verlet_check_batch<<<(n + 255) / 256, 256, 0, s>>>(xyz, radii, ref_xyz, ref_rad, nbn, off, base, n, n_mol, vmol);
-        note_launches(1);
-    }
+                                      const long long* base, int n, int n_mol, double skin, int* vmol,
+                                      unsigned* ticket, int* reuse, cudaStream_t s) {
     const float lim2 = (float)(0.25 * skin * skin) * (1.f - 1e-6f);
-    k_verlet_decide_batch<<<(n_mol + 127) / 128, 128, 0, s>>>(vmol, base, n_mol, lim2, reuse);
+    const int nb = n > 0 ? (n + CHECK_T - 1) / CHECK_T : 1;
+    k_verlet_check_batch<<<nb, CHECK_T, 0, s>>>(xyz, radii, ref_xyz, ref_rad, nbn, off, base, n, n_mol, lim2, vmol, ticket, reuse);
     note_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_verlet_check(const double* xyz, const double* radii, const double* ref_xyz, const double* ref_rad,
                                 int n, int valid, double skin, int* vstate, cudaStream_t s) {
-    cudaMemsetAsync(vstate, 0, 2 * sizeof(int), s);
-    if (valid && n > 0) {
-        k_verlet_check<<<(n + 255) / 256, 256, 0, s>>>(xyz, radii, ref_xyz, ref_rad, n, vstate);
-        note_launches(1);
-    }
     // (skin / 2)^2, rounded down in float
-    float lim2 = (float)(0.25 * skin * skin) * (1.f - 1e-6f);
-    k_verlet_decide<<<1, 1, 0, s>>>(vstate, valid, lim2);
+    const float lim2 = (float)(0.25 * skin * skin) * (1.f - 1e-6f);
+    const int nb = valid && n > 0 ? (n + CHECK_T - 1) / CHECK_T : 1;
+    k_verlet_check<<<nb, CHECK_T, 0, s>>>(xyz, radii, ref_xyz, ref_rad, n, valid, lim2, vstate);
     note_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t launch_build(const BuildArgs& a, cudaStream_t s) {
     if (a.n <= 0) return cudaSuccess;
+    // (behind the skin test, the first kernel of the build starts early too)
+    const bool early = a.skip != nullptr;
     if (a.n_mol == 1 && a.n <= kSmallAtoms) {
-        k_build_small<<<(a.n + kSmallT - 1) / kSmallT, kSmallT, 0, s>>>(a);
+        constexpr size_t smem = sizeof(int) * (kSmallCells + 1);
+        // idempotent, and needed once per context: above 48 KB a kernel has to ask
+        cudaError_t e = cudaFuncSetAttribute(k_build_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        e = launch_dependent_smem(k_build_small, 1, kSmallT, smem, s, early, a);
         note_launches(1);
-        return cudaGetLastError();
+        return e;
     }
-    return launch_build_multi(a, s);
+    return launch_build_multi(a, early, s);
 }
 
 }  // namespace dsasa

@@ -18,11 +18,12 @@ __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.w
 __device__ __forceinline__ void grid_dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
 template <class... K, class... A>
-cudaError_t launch_dependent(void (*kernel)(K...), int grid, int block, cudaStream_t s, bool early, A&&... args) {
+cudaError_t launch_dependent_smem(void (*kernel)(K...), int grid, int block, size_t smem, cudaStream_t s, bool early,
+                                  A&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -31,13 +32,17 @@ cudaError_t launch_dependent(void (*kernel)(K...), int grid, int block, cudaStre
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
+template <class... K, class... A>
+cudaError_t launch_dependent(void (*kernel)(K...), int grid, int block, cudaStream_t s, bool early, A&&... args) {
+    return launch_dependent_smem(kernel, grid, block, 0, s, early, std::forward<A>(args)...);
+}
 
 // host: adds k to the library-wide count of kernel launches (dsasa_kernel_launches)
 void note_launches(int k);
 
-// words of the single-molecule cell-list build's block-exchange area: 16 partial bounding
-// boxes of 8 words, then the completion ticket
-constexpr int BUILD_SYNC_WORDS = 16 * 8 + 1;
+// words of the cell-list build's exchange area: the ticket of the input pass (zero between
+// calls), the rows of all grids, and the cursor of the sorted order
+enum { BUILD_TICKET = 0, BUILD_ROWS = 1, BUILD_CURSOR = 2, BUILD_SYNC_WORDS = 4 };
 
 // device status bits (ORed by kernels, read by dsasa_status_sync)
 enum : int {
@@ -75,8 +80,13 @@ struct MolGrid {
     int base;         // first global cell of this molecule
     float margin;     // conservative slack of the FP32 neighbour test (A)
     float rmax;       // largest probe-inflated radius of the molecule
-    int pad[2];
+    int row0;         // first row of cells of this molecule among all molecules' rows
+    int pad;
 };
+// the first cell of row (z, y): a row holds dims[0] cells and one more entry for its end
+__host__ __device__ inline int grid_row(const MolGrid& g, int z, int y) {
+    return g.base + (z * g.dims[1] + y) * (g.dims[0] + 1);
+}
 
 struct BuildArgs {
     const double* xyz;
@@ -97,14 +107,13 @@ struct BuildArgs {
     int* molid;        // n
     int* rank;         // n
     int* cell;         // n
-    unsigned* bbox;    // n_mol * 8 (ordered-int encoded: min xyz, max xyz, rmax, pad)
+    unsigned* bbox;    // n_mol * 8, zero between calls (box words, pad)
     MolGrid* grids;    // n_mol
-    int* counts;       // max_cells + 1
+    int* counts;       // max_cells + 1, zero between calls
     int* cstart;       // max_cells + 1
     int* sidx;         // n
     float4* sf4;       // n
-    int* blocksums;    // scan scratch
-    unsigned* sync;    // BUILD_SYNC_WORDS, zero between calls: single-molecule build's partial boxes + ticket
+    unsigned* sync;    // BUILD_SYNC_WORDS
     int* status;
     int* ncells_out;   // device int: total cells used
 };
@@ -200,21 +209,21 @@ struct SRArgs {
 
 cudaError_t launch_build(const BuildArgs& a, cudaStream_t s);
 // Verlet skin test: vstate[2] = reuse the lists (valid, every atom within skin/2 of its
-// reference position, radii unchanged, no list overflow); vstate[0..1] scratch, [3] overflow
+// reference position, radii unchanged, no list overflow); vstate[3] overflow, the other words
+// scratch (zero between calls; 8 words)
 cudaError_t launch_verlet_check(const double* xyz, const double* radii, const double* ref_xyz, const double* ref_rad,
                                 int n, int valid, double skin, int* vstate, cudaStream_t s);
 // the Verlet skin test of a batch of resident molecules: reuse[m] for each molecule (see
-// k_verlet_check_batch); vmol: 3 ints per molecule of scratch
+// k_verlet_check_batch); vmol: 3 ints per molecule of scratch, ticket: one more, zero between calls
 cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, const double* ref_xyz,
                                       const double* ref_rad, const int* nbn, const long long* off,
-                                      const long long* base, int n, int n_mol, double skin, int* vmol, int* reuse,
-                                      cudaStream_t s);
+                                      const long long* base, int n, int n_mol, double skin, int* vmol,
+                                      unsigned* ticket, int* reuse, cudaStream_t s);
 cudaError_t launch_sr(const SRArgs& a, cudaStream_t s);
 // the classified cell records of every atom (a.cells), for the terms of either precision
 cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s);
 cudaError_t launch_atoms_f32(const AtomArgs& a, bool grad, cudaStream_t s);
 cudaError_t launch_atoms_f64(const AtomArgs& a, bool grad, cudaStream_t s);
-size_t scan_scratch_ints(int max_cells);
 size_t cell_record_bytes();
 
 }  // namespace dsasa

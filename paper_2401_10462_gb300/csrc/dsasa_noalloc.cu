@@ -35,10 +35,9 @@ constexpr size_t OFF_BBOX = al(OFF_SF4 + sizeof(float4) * kMaxAtoms);
 constexpr size_t OFF_GRID = al(OFF_BBOX + sizeof(unsigned) * 8);
 constexpr size_t OFF_COUNTS = al(OFF_GRID + sizeof(MolGrid));
 constexpr size_t OFF_CSTART = al(OFF_COUNTS + sizeof(int) * (kMaxCells + 1));
-constexpr size_t OFF_BSUM = al(OFF_CSTART + sizeof(int) * (kMaxCells + 1));
-constexpr size_t OFF_DEFER = al(OFF_BSUM + sizeof(int) * 4096);
+constexpr size_t OFF_DEFER = al(OFF_CSTART + sizeof(int) * (kMaxCells + 1));
 constexpr size_t OFF_STATUS = al(OFF_DEFER + sizeof(int) * kMaxAtoms);
-constexpr size_t OFF_SYNC = al(OFF_STATUS + sizeof(int) * 4);   // zero at load; the build leaves it zero
+constexpr size_t OFF_SYNC = al(OFF_STATUS + sizeof(int) * 4);
 constexpr size_t kScratchBytes = al(OFF_SYNC + sizeof(unsigned) * BUILD_SYNC_WORDS);
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -51,7 +50,6 @@ extern "C" dsasa_status dsasa_compute_noalloc(const double* coords, const double
     if (n == 0) return DSASA_OK;
     if (!coords || !radii || !areas_out) return DSASA_ERR_ARG;
     if (n > kMaxAtoms) return DSASA_ERR_CAPACITY;   // more atoms than the static scratch holds
-    if ((long long)scan_scratch_ints((int)kMaxCells) > 4096) return DSASA_ERR_CAPACITY;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     // The host-side name of the array is only a stand-in; its device address belongs to the
     // CUDA context that is current now (it changes after a device reset or under another
@@ -66,9 +64,14 @@ extern "C" dsasa_status dsasa_compute_noalloc(const double* coords, const double
         base = (unsigned char*)p;
     }
     int* status = (int*)(base + OFF_STATUS);
-    // the array keeps the previous call's contents: clear what must start at zero (the
-    // status word here; the cell counts are cleared inside the cell-list build)
-    if (cudaMemsetAsync(status, 0, sizeof(int) * 4, s) != cudaSuccess) return DSASA_ERR_CUDA;
+    // the array keeps the previous call's contents: clear what must start at zero (the status
+    // words and, although the cell-list build leaves them zero, its boxes, counts and ticket:
+    // a call that overlapped this one must not spoil the later ones)
+    static_assert(OFF_SYNC == OFF_STATUS + 256 && OFF_GRID == OFF_BBOX + 256, "cleared together");
+    if (cudaMemsetAsync(status, 0, 256 + sizeof(unsigned) * BUILD_SYNC_WORDS, s) != cudaSuccess ||
+        cudaMemsetAsync(base + OFF_BBOX, 0, 256, s) != cudaSuccess ||
+        cudaMemsetAsync(base + OFF_COUNTS, 0, sizeof(int) * (size_t)(8 * n + 129), s) != cudaSuccess)
+        return DSASA_ERR_CUDA;
     BuildArgs b{};
     b.xyz = coords;
     b.radii = radii;
@@ -90,7 +93,6 @@ extern "C" dsasa_status dsasa_compute_noalloc(const double* coords, const double
     b.grids = (MolGrid*)(base + OFF_GRID);
     b.counts = (int*)(base + OFF_COUNTS);
     b.cstart = (int*)(base + OFF_CSTART);
-    b.blocksums = (int*)(base + OFF_BSUM);
     b.sync = (unsigned*)(base + OFF_SYNC);
     b.zero_word = status + 2;   // the deferred count of the atom kernels (and a spare word)
     b.status = status;

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(SR_WARPS * 32) k_shrake_rupley(SRArgs A) {
             for (int dy = -1; dy <= 1; ++dy) {
                 int y = cy + dy;
                 if (y < 0 || y >= G.dims[1]) continue;
-                int row = G.base + (z * G.dims[1] + y) * G.dims[0];
+                int row = grid_row(G, z, y);
                 int x0 = max(cx - 1, 0), x1 = min(cx + 1, G.dims[0] - 1);
                 int beg = A.cstart[row + x0], end = A.cstart[row + x1 + 1];
                 for (int b0 = beg; b0 < end; b0 += 32) {
