@@ -72,7 +72,8 @@ struct dsasa_ctx {
     MolGrid* grids = nullptr;
     int* counts = nullptr;
     int* cstart = nullptr;
-    unsigned* bsync = nullptr;   // exchange area of the cell-list build
+    int* blocksums = nullptr;
+    unsigned* bsync = nullptr;   // exchange area of the single-molecule build
     long long* offsets = nullptr;
     int* defer = nullptr;       // atoms the fast kernel pass defers to the large pass
     int* redo = nullptr;        // atoms whose cell the carry kernel could not keep
@@ -134,7 +135,7 @@ template <class T> void dfree(T*& p) {
 
 void free_scratch(dsasa_ctx* c) {
     dfree(c->R); dfree(c->Rhl); dfree(c->f4); dfree(c->molid); dfree(c->rank); dfree(c->cell); dfree(c->sidx); dfree(c->sf4);
-    dfree(c->bbox); dfree(c->grids); dfree(c->counts); dfree(c->cstart); dfree(c->bsync); dfree(c->offsets);
+    dfree(c->bbox); dfree(c->grids); dfree(c->counts); dfree(c->cstart); dfree(c->blocksums); dfree(c->bsync); dfree(c->offsets);
     dfree(c->defer); dfree(c->redo); dfree(c->cells); dfree(c->mol_base); dfree(c->mol_reuse); dfree(c->vmol); dfree(c->mol_done);
     dfree(c->nbl); dfree(c->nbn); dfree(c->ref_xyz); dfree(c->ref_rad); dfree(c->vstate);
     c->lists_n = 0;
@@ -167,7 +168,7 @@ dsasa_status ensure(dsasa_ctx* c, int64_t n, int64_t n_mol) {
     e = dev_alloc((void**)&c->ptr, sizeof(*c->ptr) * (size_t)(count));                 \
     if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "cudaMalloc " #ptr); }
     ALLOC(R, na) ALLOC(Rhl, na) ALLOC(f4, na) ALLOC(molid, na) ALLOC(rank, na) ALLOC(cell, na) ALLOC(sidx, na) ALLOC(sf4, na)
-    ALLOC(bbox, 8 * nm) ALLOC(grids, nm) ALLOC(counts, nc + 1) ALLOC(cstart, nc + 1)
+    ALLOC(bbox, 8 * nm) ALLOC(grids, nm) ALLOC(counts, nc + 1) ALLOC(cstart, nc + 1) ALLOC(blocksums, (int64_t)scan_scratch_ints((int)nc) + 16)
     ALLOC(offsets, nm + 1) ALLOC(defer, na) ALLOC(redo, na) ALLOC(cells, na * (int64_t)cell_record_bytes()) ALLOC(bsync, BUILD_SYNC_WORDS)
     ALLOC(mol_base, nm) ALLOC(mol_reuse, nm) ALLOC(vmol, 3 * nm + 1) ALLOC(mol_done, nm)
     // what the kernels expect to be zero, and leave zero
@@ -206,7 +207,7 @@ cudaError_t build_cells(dsasa_ctx* c, const double* coords, const double* radii,
     b.max_cells = (int)c->cap_cells;
     b.R = c->R; b.Rhl = c->Rhl; b.f4 = c->f4; b.molid = c->molid; b.rank = c->rank; b.cell = c->cell;
     b.bbox = c->bbox; b.grids = c->grids; b.counts = c->counts; b.cstart = c->cstart; b.sidx = c->sidx;
-    b.sf4 = c->sf4; b.sync = c->bsync; b.zero_word = zero_word; b.status = c->status; b.ncells_out = c->status + 1;
+    b.sf4 = c->sf4; b.blocksums = c->blocksums; b.sync = c->bsync; b.zero_word = zero_word; b.status = c->status; b.ncells_out = c->status + 1;
     return launch_build(b, c->stream);
 }
 
@@ -432,7 +433,10 @@ dsasa_status dsasa_compute_sr(dsasa_ctx* c, const double* coords, const double* 
     if (!unit_points || m <= 0) return fail(c, DSASA_ERR_ARG, "need m > 0 unit points");
     st = ensure(c, n, 1);
     if (st != DSASA_OK) return st;
-    cudaError_t e = build_cells(c, coords, radii, probe, n, 1, nullptr);
+    // (cleared before the build, so that the last kernel follows the build's directly)
+    cudaError_t e = cudaMemsetAsync(c->sr_tests, 0, sizeof(unsigned long long), c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "memset");
+    e = build_cells(c, coords, radii, probe, n, 1, nullptr);
     if (e != cudaSuccess) return cuda_fail(c, e, "cell-list launch");
     c->lists_n = 0;   // the cell list now belongs to this call
     SRArgs a{};
@@ -450,7 +454,6 @@ dsasa_status dsasa_compute_sr(dsasa_ctx* c, const double* coords, const double* 
     a.exposed = exposed_out;
     a.tests = c->sr_tests;
     a.status = c->status;
-    if (c->sr_tests) cudaMemsetAsync(c->sr_tests, 0, sizeof(unsigned long long), c->stream);
     e = launch_sr(a, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "Shrake-Rupley launch");
     return DSASA_OK;

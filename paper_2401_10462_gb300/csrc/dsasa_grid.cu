@@ -7,7 +7,8 @@
 // nothing waits); counts; starts; scatter.  The neighbour search reads runs of up to three cells
 // that are adjacent along x, so only the cells of one row (fixed y, z) need consecutive starts:
 // a row takes its place in the sorted order with one atomic add and needs no scan over all
-// cells.  The order of rows and of the atoms inside a cell is not deterministic, which is
+// cells.  (A batch is built in nine kernels, with its grids and a scan over all cells in
+// kernels of their own.)  The order of rows and of the atoms inside a cell is not deterministic, which is
 // harmless because each atom later sorts its candidate list by (plane distance, atom index).
 // The sorted float4 copy (x, y, z, R) gives coalesced neighbour-tile loads in the atom kernel.
 // Bound: the latency of the dependent launches and of their atomics.
@@ -73,7 +74,6 @@ __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
         g.margin = 0.f;
         g.rmax = 0.f;
         g.base = 0;
-        g.row0 = 0;
         return g;
     }
     float lo[3], hi[3], amax = 0.f;
@@ -102,7 +102,6 @@ __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
     g.margin = margin + (float)skin;   // candidates within R_i + R_j + skin (Verlet lists)
     g.rmax = rmax;
     g.base = (dims[0] + 1) * dims[1] * dims[2];
-    g.row0 = 0;
     return g;
 }
 
@@ -115,37 +114,34 @@ __device__ __forceinline__ int cell_of(const MolGrid& g, float4 f) {
 
 constexpr int PREP_T = 256;
 
-// exclusive sums of v and w over the block's threads (in thread order) and their totals
-__device__ void block_excl_scan2(int v, int w, int& ev, int& ew, int& tv, int& tw) {
-    __shared__ int sv[PREP_T / 32], sw[PREP_T / 32];
+// exclusive sum of v over the block's threads (in thread order) and the total
+__device__ void block_excl_scan(int v, int& ev, int& tv) {
+    __shared__ int sv[PREP_T / 32];
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-    int x = v, y = w;
+    int x = v;
     for (int o = 1; o < 32; o <<= 1) {
-        const int p = __shfl_up_sync(0xffffffffu, x, o), q = __shfl_up_sync(0xffffffffu, y, o);
-        if (lane >= o) { x += p; y += q; }
+        const int p = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += p;
     }
-    if (lane == 31) { sv[wp] = x; sw[wp] = y; }
+    if (lane == 31) sv[wp] = x;
     __syncthreads();
-    int pv = 0, pw = 0;
-    tv = tw = 0;
+    int pv = 0;
+    tv = 0;
     for (int k = 0; k < PREP_T / 32; ++k) {
-        if (k == wp) { pv = tv; pw = tw; }
+        if (k == wp) pv = tv;
         tv += sv[k];
-        tw += sw[k];
     }
     ev = pv + x - v;
-    ew = pw + y - w;
     __syncthreads();
 }
 
-// Input pass and bounding boxes; the block that finishes last makes every molecule's grid and
-// clears the boxes and the ticket for the next call.
+// Input pass and bounding boxes.  GRIDS: the block that finishes last makes the grid, and clears
+// the box and the ticket for the next call.
+template <bool GRIDS>
 __global__ void __launch_bounds__(PREP_T) k_prep(BuildArgs a) {
     grid_dep_trigger();
     grid_dep_wait();
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        if (a.zero_word) { a.zero_word[0] = 0; a.zero_word[1] = 0; }
-    }
+    if (GRIDS && blockIdx.x == 0 && threadIdx.x == 0 && a.zero_word) { a.zero_word[0] = 0; a.zero_word[1] = 0; }
     if (a.skip && *a.skip) return;
     __shared__ unsigned bb[7];
     __shared__ bool last;
@@ -174,47 +170,71 @@ __global__ void __launch_bounds__(PREP_T) k_prep(BuildArgs a) {
     } else if (i < a.n) {
         for (int k = 0; k < 7; ++k) atomicMax(a.bbox + 8 * m + k, w[k]);
     }
+    if constexpr (!GRIDS) return;
     __threadfence();
     __syncthreads();
     if (tid == 0) last = atomicAdd(a.sync + BUILD_TICKET, 1u) == gridDim.x - 1;
     __syncthreads();
-    if (!last) return;
+    if (!last || tid != 0) return;
     __threadfence();
-    int cells = 0, rows = 0;   // totals over the molecules so far
-    for (int m0 = 0; m0 < a.n_mol; m0 += PREP_T) {
-        const int mm = m0 + tid;
-        MolGrid g;
-        int nc = 0, nr = 0;
-        if (mm < a.n_mol) {
-            unsigned bx[7];
-            for (int k = 0; k < 7; ++k) {
-                bx[k] = __ldcg(a.bbox + 8 * mm + k);
-                a.bbox[8 * mm + k] = 0;
-            }
-            const long long nm = a.offsets ? (a.offsets[mm + 1] - a.offsets[mm]) : a.n;
-            g = make_grid(bx, nm, a.skin);
-            nc = g.base;
-            nr = g.dims[1] * g.dims[2];
-        }
-        int ec, er, tc, tr;
-        block_excl_scan2(nc, nr, ec, er, tc, tr);
-        if (mm < a.n_mol) {
-            g.base = cells + ec;
-            g.row0 = rows + er;
-            if (g.base + nc > a.max_cells) {   // reported below; an empty grid keeps every index in range
-                for (int k = 0; k < 3; ++k) g.dims[k] = 0;
-                g.base = 0;
-            }
-            a.grids[mm] = g;
-        }
-        cells += tc;
-        rows += tr;
+    unsigned bx[7];
+    for (int k = 0; k < 7; ++k) {
+        bx[k] = __ldcg(a.bbox + k);
+        a.bbox[k] = 0;
     }
-    if (tid == 0) {
+    MolGrid g = make_grid(bx, a.n, a.skin);
+    const int cells = g.base;
+    g.base = 0;
+    a.sync[BUILD_ROWS] = (unsigned)(g.dims[1] * g.dims[2]);
+    a.sync[BUILD_CURSOR] = 0u;
+    a.sync[BUILD_TICKET] = 0u;
+    *a.ncells_out = cells;
+    if (cells > a.max_cells) {   // an empty grid keeps every index in range
+        for (int k = 0; k < 3; ++k) g.dims[k] = 0;
+        atomicOr(a.status, ST_GRID_OVF);
+    }
+    a.grids[0] = g;
+}
+
+// batches: the boxes and the atom kernels' counts cleared
+__global__ void k_bbox_init(BuildArgs a) {
+    grid_dep_trigger();
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m == 0 && a.zero_word) { a.zero_word[0] = 0; a.zero_word[1] = 0; }
+    if (m >= a.n_mol) return;
+    for (int k = 0; k < 8; ++k) a.bbox[8 * m + k] = 0;
+}
+
+// batches: each molecule's grid, its cell count in base
+__global__ void k_grid_local(BuildArgs a) {
+    grid_dep_trigger();
+    grid_dep_wait();
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m >= a.n_mol) return;
+    a.grids[m] = make_grid(a.bbox + 8 * m, a.offsets[m + 1] - a.offsets[m], a.skin);
+    for (int k = 0; k < 8; ++k) a.bbox[8 * m + k] = 0;
+}
+
+// batches: the first cell of each molecule (one block)
+__global__ void __launch_bounds__(PREP_T) k_grid_scan(BuildArgs a) {
+    grid_dep_trigger();
+    grid_dep_wait();
+    int cells = 0;
+    for (int m0 = 0; m0 < a.n_mol; m0 += PREP_T) {
+        const int m = m0 + threadIdx.x;
+        const int v = m < a.n_mol ? a.grids[m].base : 0;
+        int e, tot;
+        block_excl_scan(v, e, tot);
+        if (m < a.n_mol) {
+            const bool fits = cells + e + v <= a.max_cells;   // (reported below; an empty grid keeps every index in range)
+            a.grids[m].base = fits ? cells + e : 0;
+            if (!fits)
+                for (int k = 0; k < 3; ++k) a.grids[m].dims[k] = 0;
+        }
+        cells += tot;
+    }
+    if (threadIdx.x == 0) {
         *a.ncells_out = cells;
-        a.sync[BUILD_ROWS] = (unsigned)rows;
-        a.sync[BUILD_CURSOR] = 0u;
-        a.sync[BUILD_TICKET] = 0u;
         if (cells > a.max_cells) atomicOr(a.status, ST_GRID_OVF);
     }
 }
@@ -232,7 +252,8 @@ __global__ void k_count(BuildArgs a) {
     a.rank[i] = atomicAdd(&a.counts[c], 1);
 }
 
-// the starts of every row's cells, one warp per row; the counts are zero again afterwards
+// one molecule: the starts of every row's cells, one warp per row; the counts are zero again
+// afterwards
 __global__ void __launch_bounds__(256) k_rows(BuildArgs a) {
     grid_dep_trigger();
     grid_dep_wait();
@@ -241,13 +262,7 @@ __global__ void __launch_bounds__(256) k_rows(BuildArgs a) {
     const int rows = (int)a.sync[BUILD_ROWS];
     const int lane = threadIdx.x & 31;
     for (int r = (blockIdx.x * 256 + threadIdx.x) >> 5; r < rows; r += gridDim.x * 8) {
-        int lo = 0, hi = a.n_mol - 1;   // the last molecule with row0 <= r (empty ones hold no row)
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (a.grids[mid].row0 <= r) lo = mid; else hi = mid - 1;
-        }
-        const int d0 = a.grids[lo].dims[0];
-        const int c0 = a.grids[lo].base + (r - a.grids[lo].row0) * (d0 + 1);
+        const int d0 = a.grids[0].dims[0], c0 = r * (d0 + 1);
         int tot = 0;
         for (int x = lane; x < d0; x += 32) tot += a.counts[c0 + x];
         tot = __reduce_add_sync(0xffffffffu, tot);
@@ -266,6 +281,53 @@ __global__ void __launch_bounds__(256) k_rows(BuildArgs a) {
             if (x < d0) a.counts[c0 + x] = 0;
             pos += __shfl_sync(0xffffffffu, y, 31);
         }
+    }
+}
+
+// batches: exclusive scan of the counts of the cells in use into cstart (three kernels; the counts
+// are zero again afterwards)
+constexpr int SCAN_V = 16, SCAN_TILE = PREP_T * SCAN_V;
+__global__ void __launch_bounds__(PREP_T) k_scan_reduce(BuildArgs a, int* bsum) {
+    grid_dep_trigger();
+    grid_dep_wait();
+    const int used = min(*a.ncells_out, a.max_cells), base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
+    if (blockIdx.x * SCAN_TILE >= used) return;
+    int s = 0, e, tot;
+    for (int k = 0; k < SCAN_V; ++k) s += (base + k < used) ? a.counts[base + k] : 0;
+    block_excl_scan(s, e, tot);
+    if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
+}
+__global__ void __launch_bounds__(PREP_T) k_scan_top(BuildArgs a, int* bsum) {
+    grid_dep_trigger();
+    grid_dep_wait();
+    const int nb = (min(*a.ncells_out, a.max_cells) + SCAN_TILE - 1) / SCAN_TILE;
+    int carry = 0;
+    for (int b0 = 0; b0 < nb; b0 += PREP_T) {
+        const int b = b0 + threadIdx.x;
+        int e, tot;
+        block_excl_scan(b < nb ? bsum[b] : 0, e, tot);
+        if (b < nb) bsum[b] = carry + e;
+        carry += tot;
+    }
+}
+__global__ void __launch_bounds__(PREP_T) k_scan_down(BuildArgs a, const int* bsum) {
+    grid_dep_trigger();
+    grid_dep_wait();
+    const int used = min(*a.ncells_out, a.max_cells), base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
+    if (blockIdx.x * SCAN_TILE >= used) return;
+    int v[SCAN_V], s = 0, e, tot;
+    for (int k = 0; k < SCAN_V; ++k) {
+        v[k] = (base + k < used) ? a.counts[base + k] : 0;
+        s += v[k];
+    }
+    block_excl_scan(s, e, tot);
+    int pre = e + bsum[blockIdx.x];
+    for (int k = 0; k < SCAN_V; ++k) {
+        if (base + k < used) {
+            a.cstart[base + k] = pre;
+            a.counts[base + k] = 0;
+        }
+        pre += v[k];
     }
 }
 
@@ -381,20 +443,37 @@ __global__ void __launch_bounds__(kSmallT) k_build_small(BuildArgs a) {
     }
 }
 
-cudaError_t launch_build_multi(const BuildArgs& a, bool early, cudaStream_t s) {
+cudaError_t launch_build_one(const BuildArgs& a, bool early, cudaStream_t s) {
     const int T = 256, nb = (a.n + T - 1) / T;
-    // rows of cells: about one for every 32 atoms of a dense molecule; each warp takes several
-    const int rb = min(nb, 1216);
     static_assert(PREP_T == 256, "one thread per atom");
-    cudaError_t e = launch_dependent(k_prep, nb, PREP_T, s, early, a);
+    cudaError_t e = launch_dependent(k_prep<true>, nb, PREP_T, s, early, a);
     if (e == cudaSuccess) e = launch_dependent(k_count, nb, T, s, true, a);
-    if (e == cudaSuccess) e = launch_dependent(k_rows, rb, T, s, true, a);
+    // rows of cells: about one for every 32 atoms of a dense molecule; each warp takes several
+    if (e == cudaSuccess) e = launch_dependent(k_rows, min(nb, 1216), T, s, true, a);
     if (e == cudaSuccess) e = launch_dependent(k_scatter, nb, T, s, true, a);
     note_launches(4);
     return e;
 }
 
+cudaError_t launch_build_batch(const BuildArgs& a, cudaStream_t s) {
+    const int T = 256, nb = (a.n + T - 1) / T, mb = (a.n_mol + T - 1) / T;
+    const int nt = (int)scan_scratch_ints(a.max_cells) - 1;   // (blocks past the cells in use return at once)
+    cudaError_t e = launch_dependent(k_bbox_init, mb, T, s, false, a);
+    if (e == cudaSuccess) e = launch_dependent(k_prep<false>, nb, PREP_T, s, true, a);
+    if (e == cudaSuccess) e = launch_dependent(k_grid_local, mb, T, s, true, a);
+    if (e == cudaSuccess) e = launch_dependent(k_grid_scan, 1, PREP_T, s, true, a);
+    if (e == cudaSuccess) e = launch_dependent(k_count, nb, T, s, true, a);
+    if (e == cudaSuccess) e = launch_dependent(k_scan_reduce, nt, PREP_T, s, true, a, a.blocksums);
+    if (e == cudaSuccess) e = launch_dependent(k_scan_top, 1, PREP_T, s, true, a, a.blocksums);
+    if (e == cudaSuccess) e = launch_dependent(k_scan_down, nt, PREP_T, s, true, a, (const int*)a.blocksums);
+    if (e == cudaSuccess) e = launch_dependent(k_scatter, nb, T, s, true, a);
+    note_launches(9);
+    return e;
+}
+
 }  // namespace
+
+size_t scan_scratch_ints(int max_cells) { return (size_t)(max_cells + SCAN_TILE - 1) / SCAN_TILE + 1; }
 
 namespace {
 
@@ -529,7 +608,7 @@ cudaError_t launch_build(const BuildArgs& a, cudaStream_t s) {
         note_launches(1);
         return e;
     }
-    return launch_build_multi(a, early, s);
+    return a.n_mol == 1 ? launch_build_one(a, early, s) : launch_build_batch(a, s);
 }
 
 }  // namespace dsasa

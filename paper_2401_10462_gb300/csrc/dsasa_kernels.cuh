@@ -40,8 +40,8 @@ cudaError_t launch_dependent(void (*kernel)(K...), int grid, int block, cudaStre
 // host: adds k to the library-wide count of kernel launches (dsasa_kernel_launches)
 void note_launches(int k);
 
-// words of the cell-list build's exchange area: the ticket of the input pass (zero between
-// calls), the rows of all grids, and the cursor of the sorted order
+// words of the single-molecule build's exchange area: the ticket of the input pass (zero between
+// calls), the rows of the grid, and the cursor of the sorted order
 enum { BUILD_TICKET = 0, BUILD_ROWS = 1, BUILD_CURSOR = 2, BUILD_SYNC_WORDS = 4 };
 
 // device status bits (ORed by kernels, read by dsasa_status_sync)
@@ -80,8 +80,7 @@ struct MolGrid {
     int base;         // first global cell of this molecule
     float margin;     // conservative slack of the FP32 neighbour test (A)
     float rmax;       // largest probe-inflated radius of the molecule
-    int row0;         // first row of cells of this molecule among all molecules' rows
-    int pad;
+    int pad[2];
 };
 // the first cell of row (z, y): a row holds dims[0] cells and one more entry for its end
 __host__ __device__ inline int grid_row(const MolGrid& g, int z, int y) {
@@ -113,6 +112,7 @@ struct BuildArgs {
     int* cstart;       // max_cells + 1
     int* sidx;         // n
     float4* sf4;       // n
+    int* blocksums;    // scan scratch (batches)
     unsigned* sync;    // BUILD_SYNC_WORDS
     int* status;
     int* ncells_out;   // device int: total cells used
@@ -224,6 +224,7 @@ cudaError_t launch_sr(const SRArgs& a, cudaStream_t s);
 cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s);
 cudaError_t launch_atoms_f32(const AtomArgs& a, bool grad, cudaStream_t s);
 cudaError_t launch_atoms_f64(const AtomArgs& a, bool grad, cudaStream_t s);
+size_t scan_scratch_ints(int max_cells);
 size_t cell_record_bytes();
 
 }  // namespace dsasa
