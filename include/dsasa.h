@@ -170,8 +170,8 @@ dsasa_status dsasa_lists_reused(dsasa_ctx* ctx, int* reused);
  * from the previous call (dsasa_config.carry), else 0. */
 dsasa_status dsasa_cells_carried(dsasa_ctx* ctx, int64_t* carried);
 
-/* Diagnostics: synchronises and writes the number of point-neighbour tests the last
- * dsasa_compute_sr call performed (sum over atoms of m x overlapping neighbours). */
+/* Diagnostics: synchronises and writes the number of point-neighbour pairs the last
+ * dsasa_compute_sr call decided (sum over atoms of m x overlapping neighbours). */
 dsasa_status dsasa_sr_tests(dsasa_ctx* ctx, int64_t* tests);
 
 /* As dsasa_compute, with grad_out[j] = d(sum_i w_i A_i)/d(p_j) for area_weights w

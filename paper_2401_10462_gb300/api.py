@@ -236,7 +236,7 @@ class Context:
         return int(t.value)
 
     def sr_tests(self) -> int:
-        """Point-neighbour tests of the last compute_sr call."""
+        """Point-neighbour pairs that the last compute_sr call decided."""
         t = ctypes.c_int64(0)
         self._raise(_lib.dsasa_sr_tests(self._h, ctypes.byref(t)))
         return int(t.value)
