@@ -21,8 +21,8 @@
 // One warp per atom (two per block); the cell lives in shared memory (plane table, triangle
 // table) and in registers (each lane caches the homogeneous coordinates of up to NT / 32
 // cell vertices).  The fast path runs the steps as separate kernels that hand the cell over
-// through a per-atom record in HBM (PH_CELL: Step 1; PH_CLASS: Step 2; k_terms in
-// dsasa_terms.cuh: Step 3; PH_VOL: the volume), so that each kernel's code fits the instruction cache.  On small
+// through a per-atom record in HBM (PH_CELL: Step 1; k_class in dsasa_class.cuh: Step 2;
+// k_terms in dsasa_terms.cuh: Step 3; PH_VOL: the volume), so that each kernel's code fits the instruction cache.  On small
 // molecules Steps 1 and 2 run as one kernel (PH_CC, cells_fused), so that classifications
 // overlap the slowest cells.  With carried cells, Step 1 is PH_CARRY (on calls reusing the neighbour
 // lists, each atom's cell from the previous call, kept when exact predicates certify it) and
@@ -48,13 +48,13 @@ constexpr int WARPS = 1, WARPS_CELL = 2, WARPS_CLASS = 2, WARPS_TERMS = 2;
 // resident blocks per SM that each kernel's register budget is sized for (one warp each)
 // (the cell kernels: 64 registers and 32 warps an SM; 20,003-atom globule 176 us, against 186 at
 // 18 blocks of 56 registers, 182 at 14, 194 at 12 and 251 at 21)
-constexpr int MINB = 32, MINB_CELL = 16, MINB_CLASS = 18, MINB_TERMS = 18;
+constexpr int MINB = 32, MINB_CELL = 16, MINB_TERMS = 18;
 
 // kernel phases: the whole computation in one kernel, or three kernels that pass the cell
 // through a global record per atom: the cell construction (gather, sort, clipping), the
 // classification (Steps 2a-2c: which simplices of the cell are in C), and the area terms and
 // gradient.  Each kernel's code then fits the instruction cache.
-enum { PH_ALL = 0, PH_CELL = 1, PH_CLASS = 2, PH_VOL = 4, PH_CC = 5, PH_CARRY = 6 };
+enum { PH_ALL = 0, PH_CELL = 1, PH_VOL = 4, PH_CC = 5, PH_CARRY = 6 };
 template <int N> struct IntC { static constexpr int value = N; };
 enum { CELL_OK = 0, CELL_DONE = 1 };   // record flag: CELL_DONE = outputs already written
 
@@ -345,8 +345,8 @@ template <class SM, class R = typename SM::Real> __device__ __forceinline__ VtxF
 // 10 operations instead of the 33 of the magnitudes themselves.  It is about twice their sum;
 // a clip test that it leaves open is decided again with the magnitudes (rare: fewer than one
 // in 20 atoms of a globule meets one).
-__device__ __forceinline__ void new_vertex(const float4 A, const float2 am, const float4 B, const float2 bm,
-                                           const float4 M, const float2 mm, float* V, float& Vs) {
+__device__ __forceinline__ void hom_vertex(const float4 A, const float2 am, const float4 B, const float2 bm,
+                                           const float4 M, const float2 mm, float* V, float& Vd, float& Vw) {
     const P3<float> qa = {A.x, A.y, A.z}, qb = {B.x, B.y, B.z}, qm = {M.x, M.y, M.z};
     const P3<float> xbm = cross3(qb, qm), xma = cross3(qm, qa), xab = cross3(qa, qb);
     V[0] = xbm.x * A.w + xma.x * B.w + xab.x * M.w;
@@ -354,7 +354,14 @@ __device__ __forceinline__ void new_vertex(const float4 A, const float2 am, cons
     V[2] = xbm.z * A.w + xma.z * B.w + xab.z * M.w;
     V[3] = dot3(qa, xbm);
     const float nab = am.x * bm.x, nam = am.x * mm.x, nbm = bm.x * mm.x;
-    Vs = (nbm * am.y + nam * bm.y + nab * (mm.y + mm.x)) * 1.000001f;
+    Vd = nbm * am.y + nam * bm.y + nab * mm.y;   // the three of Dv
+    Vw = nab * mm.x;                             // that of D
+}
+__device__ __forceinline__ void new_vertex(const float4 A, const float2 am, const float4 B, const float2 bm,
+                                           const float4 M, const float2 mm, float* V, float& Vs) {
+    float Vd, Vw;
+    hom_vertex(A, am, B, bm, M, mm, V, Vd, Vw);
+    Vs = (Vd + Vw) * 1.000001f;
 }
 // out of line (the kernels that also classify or evaluate terms keep their code small)
 template <class SM, class R = typename SM::Real> __device__ __noinline__ VtxFA<R> vertex_fa(const SM* S, uchar4 v) {
@@ -563,6 +570,16 @@ __device__ __forceinline__ uchar4 unpack3(unsigned w) {
     return make_uchar4((uint8_t)w, (uint8_t)(w >> 8), (uint8_t)(w >> 16), 0);
 }
 
+}  // namespace
+
+}  // namespace dsasa
+
+#include "dsasa_class.cuh"
+
+namespace dsasa {
+
+namespace {
+
 // ------------------------------------------------------------------ carried cells
 // The incremental update of C across MD steps.  On a call that reuses the neighbour lists
 // (every atom within half the skin of its last rebuild), the cell that the previous call
@@ -734,10 +751,10 @@ __device__ __noinline__ int carry_cell(SM* S, const RC* rec, int i, int n, int n
 
 // ------------------------------------------------------------------ the kernel
 __host__ __device__ constexpr int minb(int ph) {
-    return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? MINB_CELL : (ph == PH_CLASS ? MINB_CLASS : (ph == PH_VOL ? MINB_TERMS : MINB));
+    return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? MINB_CELL : (ph == PH_VOL ? MINB_TERMS : MINB);
 }
 __host__ __device__ constexpr int warps_of(int ph) {
-    return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? WARPS_CELL : (ph == PH_CLASS ? WARPS_CLASS : (ph == PH_VOL ? WARPS_TERMS : WARPS));
+    return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? WARPS_CELL : (ph == PH_VOL ? WARPS_TERMS : WARPS);
 }
 template <class R, bool GRAD, int NE, int NT, int PHX>
 __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArgs A) {
@@ -755,6 +772,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     Smem<R, NE, NT>* S = &smem_all[wib];
+    __shared__ ClassTmp class_tmp[PHX == PH_CC ? WARPS : 1];   // (used by PH_CC only)
     const int nwarps = gridDim.x * WARPS;
     grid_dep_trigger();
     grid_dep_wait();   // the previous kernel of the call (cell list, cell records) is complete
@@ -780,7 +798,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
         const FA<R> wi = {Rr * Rr, Rr * Rr};
         CellRec<float, NE, NT>* rec = (CellRec<float, NE, NT>*)A.cells + s;
         auto done = [&]() {   // the outputs of this atom are written: tell the terms kernel
-            if ((PH == PH_CELL || PH == PH_CLASS || PH == PH_CC) && lane == 0) rec->flag = CELL_DONE;
+            if ((PH == PH_CELL || PH == PH_CC) && lane == 0) rec->flag = CELL_DONE;
         };
         auto no_cell = [&]() {   // the record holds no cell of this atom (nothing to carry)
             if ((PH == PH_CELL || PH == PH_CC) && lane == 0) rec->atom = -1;
@@ -807,10 +825,10 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
         R V[SPL][4], Vs[SPL], Va[SPL][LOOSE ? 1 : 4];
         unsigned alive = 0;
         auto compute_vertex = [&](int r, int t) {
-            // inline in the split cell and classification kernels (measured faster there), a
-            // call in the kernels that hold more code
+            // inline in the split cell kernel (measured faster there), a call in the kernels that
+            // hold more code
             VtxFA<R> q;
-            if constexpr (PH == PH_CELL || PH == PH_CLASS) q = vertex_fa_inl(S, S->tv[t]);
+            if constexpr (PH == PH_CELL) q = vertex_fa_inl(S, S->tv[t]);
             else q = vertex_fa(S, S->tv[t]);
             for (int k = 0; k < 4; ++k) V[r][k] = q.v[k];
             if constexpr (LOOSE) Vs[r] = ((q.a[0] + q.a[1]) + (q.a[2] + q.a[3])) * (R)1.000001;
@@ -1372,7 +1390,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             if ((int)TV[r] < 0) alive |= 1u << r;
             TV[r] = (int)TV[r] < 0 ? TV[r] & ~ALIVE : DEADV;
         }
-        if constexpr (PH != PH_CELL) {   // the cell to shared memory, for the classification
+        if constexpr (PH == PH_ALL) {   // the cell to shared memory, for the classification
 #pragma unroll
             for (int r = 0; r < SPL; ++r) {
                 S->tv[r * 32 + lane] = unpack3(TV[r]);
@@ -1440,7 +1458,16 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 rec->atom = i;
             }
             __syncwarp();
-            if constexpr (PH == PH_CELL) continue;
+            if constexpr (PH == PH_CC) {
+                FA<R> P[SPL];
+#pragma unroll
+                for (int r = 0; r < SPL; ++r) {
+                    P[r].v = V[r][0] * V[r][0] + V[r][1] * V[r][1] + V[r][2] * V[r][2] - wi.v * V[r][3] * V[r][3];
+                    P[r].a = fmax((R)1, wi.a) * Vs[r] * Vs[r] * (R)1.000001;   // at least sum_k a_k^2 + w a_3^2
+                }
+                classify_cell(S, &class_tmp[wib], A, i, rec, nc, hw, TV, TA, P, Rr * Rr);
+            }
+            if constexpr (PH != PH_ALL) continue;
         }
         } else {
             // ---------------- the cell built by the cell kernel: the header, then every load of
@@ -1453,8 +1480,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             nc = hd.z;
             const int np = NG + nc, hw = hd.w;
             nrounds = (hw + 31) >> 5;
-            constexpr bool BATCH_LOADS = sizeof(R) == 4 && (PH == PH_CLASS || PH == PH_VOL);
-            if constexpr (BATCH_LOADS) {
+            if constexpr (sizeof(R) == 4) {
                 Row4<float> rq[2];
                 float rb[2];
                 int rg[2];
@@ -1468,7 +1494,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                         rb[h] = rec->pB[e];
                         rg[h] = rec->pg[e];
                         rs[h] = rec->start[e];
-                        if constexpr (PH == PH_VOL) ref[h] = rec->eflag[e];
+                        ref[h] = rec->eflag[e];
                     }
                     rtv[h] = rta[h] = make_uchar4(NONE, NONE, NONE, 0);
                     if (e < hw) {
@@ -1484,7 +1510,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                         S->pm[e][1] = rb[h];
                         S->pg[e] = rg[h];
                         S->start[e] = rs[h];
-                        if constexpr (PH == PH_VOL) S->eflag[e] = ref[h];
+                        S->eflag[e] = ref[h];
                     }
                     if (e < 32 * nrounds) {
                         S->tv[e] = rtv[h];
@@ -1510,16 +1536,6 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 for (int e = lane; e < np; e += 32) S->eflag[e] = rec->eflag[e];
             }
             if (lane == 0) { S->hw = hw; S->bad = 0; }
-            __syncwarp();
-#pragma unroll
-            for (int r = 0; r < SPL; ++r) {
-                if (r >= nrounds) break;
-                int t = r * 32 + lane;
-                if (S->tv[t].x != NONE) {
-                    if constexpr (PH == PH_CLASS) compute_vertex(r, t);
-                    alive |= 1u << r;
-                }
-            }
             __syncwarp();
             if constexpr (PH == PH_VOL) {
                 if (!(rec->iK)) {
@@ -1700,11 +1716,7 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 gacc.add(kap * gsum.x + cf * pa.x, kap * gsum.y + cf * pa.y, kap * gsum.z + cf * pa.z);
             }
         };
-        // faces whose edge test the filters left open (bit = the lane's face iteration), and
-        // which of them are closed; resolved after the loop (the fused kernel decides in place)
-        unsigned open2c = 0, closed2c = 0;
-        int it2c = 0;
-        for (int a = NG + lane; a < NG + nc; a += 32, ++it2c) {
+        for (int a = NG + lane; a < NG + nc; a += 32) {
             uint8_t flag = 0;
             R phi_sum = zero;
             int st = S->start[a];
@@ -1757,32 +1769,6 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                         }
                         eK = inside;
                     }
-                } else if (!eK) {
-                    // the same tests with the filters only; an open one defers the face
-                    const int se = fsign<PK_EDGE>(S, wi, a, a);
-                    bool open = se == 0;
-                    if (se < 0) {
-                        bool out = false;
-                        t = st & (NT - 1);
-                        for (int step = 0; step < NT; ++step) {
-                            uchar4 v = S->tv[t];
-                            int k = v.x == a ? 0 : (v.y == a ? 1 : 2);
-                            uint8_t b = tv_get(v, (k + 1) % 3);
-                            if (b >= NG) {
-                                const int sb = fsign<PK_EDGEB>(S, wi, a, b);
-                                if (sb > 0) { out = true; break; }
-                                if (sb == 0) open = true;
-                            }
-                            t = tv_get(S->ta[t], k) & (NT - 1);
-                            if (t == (st & (NT - 1))) break;
-                        }
-                        if (out) open = false;
-                        else if (!open) eK = true;
-                    }
-                    if (open) {
-                        open2c |= 1u << it2c;
-                        if (closed) closed2c |= 1u << it2c;
-                    }
                 }
                 if (eK) {
                     flag = 1 | (closed ? 2 : 0);
@@ -1793,32 +1779,8 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             }
             S->eflag[a] = flag;
         }
-        if (PH != PH_ALL && __any_sync(FULL, open2c != 0)) {
-            // the deferred faces, with exact predicates
-            it2c = 0;
-            for (int a = NG + lane; a < NG + nc; a += 32, ++it2c) {
-                if (!(open2c >> it2c & 1)) continue;
-                const int st = S->start[a] & (NT - 1);
-                bool eK = false;
-                if (psign<PK_EDGE>(S, c, wi, a, 0) <= 0) {
-                    eK = true;
-                    int t = st;
-                    for (int step = 0; step < NT; ++step) {
-                        const uchar4 v = S->tv[t];
-                        const int k = v.x == a ? 0 : (v.y == a ? 1 : 2);
-                        const uint8_t b = tv_get(v, (k + 1) % 3);
-                        if (b >= NG && psign<PK_EDGEB>(S, c, wi, a, b) > 0) { eK = false; break; }
-                        t = tv_get(S->ta[t], k) & (NT - 1);
-                        if (t == st) break;
-                    }
-                }
-                if (eK) {
-                    S->eflag[a] = 1 | ((closed2c >> it2c & 1) ? 2 : 0);
-                    myEK = 1;
-                }
-            }
-        }
         __syncwarp();
+
         // vertex i in C?  (an edge of C holds it, or p_i lies in its own cell)
         bool iK, icl;
         iK = __any_sync(FULL, myEK);
@@ -1841,46 +1803,6 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             }
             iK = __all_sync(FULL, ok);
         }
-        if constexpr (PH == PH_CLASS || PH == PH_CC) {
-            __syncwarp();
-            if (S->bad) {
-                if (lane == 0) {
-                    atomicOr(A.status, ST_BADCELL);
-                    A.areas[i] = __longlong_as_double(0x7ff8000000000000ll);
-                    if (A.grad) { A.grad[3 * i] = A.grad[3 * i + 1] = A.grad[3 * i + 2] = __longlong_as_double(0x7ff8000000000000ll); }
-                    if (A.vol) A.vol[i] = __longlong_as_double(0x7ff8000000000000ll);
-                }
-                finished();
-                done();
-                __syncwarp();
-                continue;
-            }
-            if (!iK && !EXPORT) {
-                // no simplex of C holds i: A_i = 0 (and V_i = 0) and no gradient gathers
-                if (lane == 0) {
-                    A.areas[i] = 0.0;
-                    if (A.grad) { A.grad[3 * i] = A.grad[3 * i + 1] = A.grad[3 * i + 2] = 0.0; }
-                    if (A.vol) A.vol[i] = 0.0;
-                    if (A.vgrad) { A.vgrad[3 * i] = A.vgrad[3 * i + 1] = A.vgrad[3 * i + 2] = 0.0; }
-                }
-                finished();
-                done();
-                __syncwarp();
-                continue;
-            }
-            for (int e = lane; e < NG + nc; e += 32) rec->eflag[e] = S->eflag[e];
-            for (int t = lane; t < S->hw; t += 32) {
-                rec->kf[t] = S->kf[t];
-                rec->tf[t] = (uint8_t)S->tf[t];
-            }
-            if (lane == 0) {
-                rec->iK = iK;
-                rec->icl = icl;
-            }
-            __syncwarp();
-            continue;
-        }
-
         // vertex term Omega_i 4 pi R_i^2 (Eq. vertex), Omega_i = 1 - sum of solid angles / 4 pi
         // (with the half solid angles h_T of its tetrahedra: Omega_i 4 pi R_i^2 = 4 pi R_i^2 - 2 R_i^2 sum h_T)
         if (iK && !icl) {

@@ -53,7 +53,7 @@ cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s) {
             go(k_atoms<float, false, 64, 64, PH_CELL>, nb(WARPS_CELL), WARPS_CELL * 32, fast);
         }
         mark(0);
-        go(k_atoms<float, false, 64, 64, PH_CLASS>, nb(WARPS_CLASS), WARPS_CLASS * 32, fast);
+        go(k_class<WARPS_CLASS>, nb(WARPS_CLASS), WARPS_CLASS * 32, fast);
     }
     mark(1);
     return go.err;
