@@ -786,15 +786,26 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
         Ctx c;
         c.xyz = A.xyz;
         c.R = A.R;
-        c.pi[0] = A.xyz[3 * i];
-        c.pi[1] = A.xyz[3 * i + 1];
-        c.pi[2] = A.xyz[3 * i + 2];
-        c.Ri = A.R[i];
-        c.h = ghost_h(c.Ri);
+        float hf = 0.f;
+        if constexpr (PH == PH_VOL) {
+            c.pi[0] = A.xyz[3 * i];
+            c.pi[1] = A.xyz[3 * i + 1];
+            c.pi[2] = A.xyz[3 * i + 2];
+            c.Ri = A.R[i];
+            c.h = ghost_h(c.Ri);
+        } else {
+            const AtomD at = load_atom(A.ad + i);
+            c.pi[0] = at.x;
+            c.pi[1] = at.y;
+            c.pi[2] = at.z;
+            c.Ri = at.R;
+            hf = A.gh[i];
+            c.h = (double)hf;
+        }
         c.i = i;
         c.n = A.n;
         c.status = A.status;
-        const R Rr = (R)c.Ri;
+        const R Rr = PH != PH_VOL && sizeof(R) == 4 ? (R)A.Rhl[i].x : (R)c.Ri;
         const FA<R> wi = {Rr * Rr, Rr * Rr};
         CellRec<float, NE, NT>* rec = (CellRec<float, NE, NT>*)A.cells + s;
         auto done = [&]() {   // the outputs of this atom are written: tell the terms kernel
@@ -876,8 +887,9 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                 int j = -1;
                 if (k < nl) {
                     j = DS_IDX(A.nbl[li * NBL_CAP + k] + lofs, A.n, A.status);
-                    const double dx = A.xyz[3 * j] - c.pi[0], dy = A.xyz[3 * j + 1] - c.pi[1], dz = A.xyz[3 * j + 2] - c.pi[2];
-                    const double rr = c.Ri + A.R[j];
+                    const AtomD q = load_atom(A.ad + j);
+                    const double dx = q.x - c.pi[0], dy = q.y - c.pi[1], dz = q.z - c.pi[2];
+                    const double rr = c.Ri + q.R;
                     ok = dx * dx + dy * dy + dz * dz < rr * rr * (1.0 + 1e-9);
                 }
                 unsigned bal = __ballot_sync(FULL, ok);
@@ -912,9 +924,9 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
                     }
                     if (store_lists || A.skin_band) {
                         if (ok) {
-                            const double ddx = A.xyz[3 * j] - c.pi[0], ddy = A.xyz[3 * j + 1] - c.pi[1],
-                                         ddz = A.xyz[3 * j + 2] - c.pi[2];
-                            const double rr64 = c.Ri + A.R[j];
+                            const AtomD q = load_atom(A.ad + j);
+                            const double ddx = q.x - c.pi[0], ddy = q.y - c.pi[1], ddz = q.z - c.pi[2];
+                            const double rr64 = c.Ri + q.R;
                             ok = ddx * ddx + ddy * ddy + ddz * ddz < rr64 * rr64 * (1.0 + 1e-9);
                         }
                     }
@@ -1057,29 +1069,34 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
             rank[r] = el;
             key[r] = ~0u;
             if (el < nc) {
-                double q[3], b, babs;
-                bool ex;
                 tg[r] = S->pg[NG + el];
-                plane64_of(c, tg[r], q, b, babs, ex);
-                const float qx = (float)q[0], qy = (float)q[1], qz = (float)q[2];
+                const AtomD pk = load_atom(A.ad + DS_IDX(tg[r], A.n, A.status));
+                // q and b in FP64, rounded once (an FP64 instruction occupies a sub-partition for 64
+                // cycles: 8 and the 4 conversions are what is left of 18)
+                const double q[3] = {pk.x - c.pi[0], pk.y - c.pi[1], pk.z - c.pi[2]};
+                const double s2 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2];
+                const double b2 = (s2 - pk.R * pk.R) + c.Ri * c.Ri;
+                const float qx = (float)q[0], qy = (float)q[1], qz = (float)q[2], bf = 0.5f * (float)b2;
                 for (int k = 0; k < 3; ++k) tq[r][k] = (R)q[k];
-                tq[r][3] = (R)b;
-                // magnitude proxy of b in float: |b_f| (1 + 2^-22) + 2^-26 babs, rounded up (the float
-                // evaluation loses at most 2 ulp, covered by the larger factors)
-                if (sizeof(R) == 4) tm[r][1] = (R)(fabsf((float)b) * 1.0000003f + (float)babs * 1.5e-8f);
-                else tm[r][1] = (R)(8.0 * babs);
+                tq[r][3] = sizeof(R) == 4 ? (R)bf : (R)(0.5 * b2);
+                const float qq = qx * qx + qy * qy + qz * qz;
+                // magnitude of b: its terms |q|^2, R_k^2, R_i^2 sum to twice babs = |q|^2 + R_i^2 - b; in float
+                // |b_f| (1 + 2^-22) + 2^-26 babs, rounded up (the float evaluation loses a few ulp, covered
+                // by the larger factors)
+                const float babs = (qq + (float)(Rr * Rr) - bf) * 1.00001f;
+                if (sizeof(R) == 4) tm[r][1] = (R)(fabsf(bf) * 1.0000003f + babs * 1.5e-8f);
+                else tm[r][1] = (R)(8.0 * (0.5 * ((s2 + pk.R * pk.R) + c.Ri * c.Ri)));
                 tm[r][0] = (R)((fabsf(qx) + fabsf(qy) + fabsf(qz)) * 1.000001f);
-                const unsigned u = __float_as_uint((float)b * rsqrtf(qx * qx + qy * qy + qz * qz + 1e-30f));
+                const unsigned u = __float_as_uint(bf * rsqrtf(qq + 1e-30f));
                 key[r] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
             }
         }
         if (lane < NG) {
-            double q[3], b;
-            ghost_plane64(lane, c.h, q, b);
-            for (int k = 0; k < 3; ++k) S->pq[lane][k] = (R)q[k];
-            S->pq[lane][3] = (R)b;
-            S->pm[lane][0] = (R)(2.0 * c.h);
-            S->pm[lane][1] = sizeof(R) == 4 ? (R)(fabsf((float)b) * 1.0000004f) : (R)b;
+            const R h2 = (R)(2.f * hf), b = h2 * (R)hf;   // ghost_plane64 (2 h exact in float, 2 h^2 in double)
+            for (int k = 0; k < 3; ++k) S->pq[lane][k] = k == lane >> 1 ? ((lane & 1) ? -h2 : h2) : (R)0;
+            S->pq[lane][3] = b;
+            S->pm[lane][0] = h2;
+            S->pm[lane][1] = sizeof(R) == 4 ? b * (R)1.0000004 : b;
             S->pg[lane] = -1 - lane;
         }
         for (int e = lane; e < NG + nc; e += 32) {

@@ -62,6 +62,8 @@ struct dsasa_ctx {
     // scratch
     double* R = nullptr;
     float2* Rhl = nullptr;
+    AtomD* ad = nullptr;
+    float* gh = nullptr;
     float4* f4 = nullptr;
     int* molid = nullptr;
     int* rank = nullptr;
@@ -134,7 +136,7 @@ template <class T> void dfree(T*& p) {
 }
 
 void free_scratch(dsasa_ctx* c) {
-    dfree(c->R); dfree(c->Rhl); dfree(c->f4); dfree(c->molid); dfree(c->rank); dfree(c->cell); dfree(c->sidx); dfree(c->sf4);
+    dfree(c->R); dfree(c->Rhl); dfree(c->ad); dfree(c->gh); dfree(c->f4); dfree(c->molid); dfree(c->rank); dfree(c->cell); dfree(c->sidx); dfree(c->sf4);
     dfree(c->bbox); dfree(c->grids); dfree(c->counts); dfree(c->cstart); dfree(c->blocksums); dfree(c->bsync); dfree(c->offsets);
     dfree(c->defer); dfree(c->redo); dfree(c->cells); dfree(c->mol_base); dfree(c->mol_reuse); dfree(c->vmol); dfree(c->mol_done);
     dfree(c->nbl); dfree(c->nbn); dfree(c->ref_xyz); dfree(c->ref_rad); dfree(c->vstate);
@@ -167,7 +169,7 @@ dsasa_status ensure(dsasa_ctx* c, int64_t n, int64_t n_mol) {
 #define ALLOC(ptr, count)                                                               \
     e = dev_alloc((void**)&c->ptr, sizeof(*c->ptr) * (size_t)(count));                 \
     if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "cudaMalloc " #ptr); }
-    ALLOC(R, na) ALLOC(Rhl, na) ALLOC(f4, na) ALLOC(molid, na) ALLOC(rank, na) ALLOC(cell, na) ALLOC(sidx, na) ALLOC(sf4, na)
+    ALLOC(R, na) ALLOC(Rhl, na) ALLOC(ad, na) ALLOC(gh, na) ALLOC(f4, na) ALLOC(molid, na) ALLOC(rank, na) ALLOC(cell, na) ALLOC(sidx, na) ALLOC(sf4, na)
     ALLOC(bbox, 8 * nm) ALLOC(grids, nm) ALLOC(counts, nc + 1) ALLOC(cstart, nc + 1) ALLOC(blocksums, (int64_t)scan_scratch_ints((int)nc) + 16)
     ALLOC(offsets, nm + 1) ALLOC(defer, na) ALLOC(redo, na) ALLOC(cells, na * (int64_t)cell_record_bytes()) ALLOC(bsync, BUILD_SYNC_WORDS)
     ALLOC(mol_base, nm) ALLOC(mol_reuse, nm) ALLOC(vmol, 3 * nm + 1) ALLOC(mol_done, nm)
@@ -205,7 +207,7 @@ cudaError_t build_cells(dsasa_ctx* c, const double* coords, const double* radii,
     b.offsets = offsets_dev;
     b.skin = c->cfg.skin;
     b.max_cells = (int)c->cap_cells;
-    b.R = c->R; b.Rhl = c->Rhl; b.f4 = c->f4; b.molid = c->molid; b.rank = c->rank; b.cell = c->cell;
+    b.R = c->R; b.Rhl = c->Rhl; b.ad = c->ad; b.gh = c->gh; b.f4 = c->f4; b.molid = c->molid; b.rank = c->rank; b.cell = c->cell;
     b.bbox = c->bbox; b.grids = c->grids; b.counts = c->counts; b.cstart = c->cstart; b.sidx = c->sidx;
     b.sf4 = c->sf4; b.blocksums = c->blocksums; b.sync = c->bsync; b.zero_word = zero_word; b.status = c->status; b.ncells_out = c->status + 1;
     return launch_build(b, c->stream);
@@ -231,7 +233,7 @@ dsasa_status run(dsasa_ctx* c, const double* coords, const double* radii, double
     if (lists) {
         const int valid = c->lists_n == n && c->lists_probe == probe;
         cudaError_t ev_e = launch_verlet_check(coords, radii, c->ref_xyz, c->ref_rad, (int)n, valid, c->cfg.skin,
-                                               c->vstate, c->stream);
+                                               c->vstate, c->ad, c->stream);
         if (ev_e != cudaSuccess) return cuda_fail(c, ev_e, "Verlet check launch");
     }
     // the build also clears the deferred-atom count of the atom kernels that follow it
@@ -244,6 +246,8 @@ dsasa_status run(dsasa_ctx* c, const double* coords, const double* radii, double
     a.xyz = coords;
     a.R = c->R;
     a.Rhl = c->Rhl;
+    a.ad = c->ad;
+    a.gh = c->gh;
     a.sf4 = c->sf4;
     a.sidx = c->sidx;
     a.molid = c->molid;

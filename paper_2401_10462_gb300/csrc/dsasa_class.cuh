@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(WARPS * 32, MINB_CLASS) k_class(AtomArgs A) {
     const int nc = hd.z, hw = hd.w;
     const bool two = NG + nc > 32 || hw > 32;
     if (two) load(1);
-    const float Ri = (float)A.R[i], w = Ri * Ri;
+    const float Ri = A.Rhl[i].x, w = Ri * Ri;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (h == 1 && !two) break;

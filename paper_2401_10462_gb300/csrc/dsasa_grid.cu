@@ -13,6 +13,7 @@
 // The sorted float4 copy (x, y, z, R) gives coalesced neighbour-tile loads in the atom kernel.
 // Bound: the latency of the dependent launches and of their atomics.
 #include "dsasa_kernels.cuh"
+#include "dsasa_math.cuh"
 
 #include <math.h>
 
@@ -48,6 +49,8 @@ __device__ __forceinline__ float4 prep_atom(const BuildArgs& a, int i, int m) {
     a.R[i] = R;
     const float h = (float)R;
     a.Rhl[i] = make_float2(h, (float)(R - (double)h));
+    a.ad[i] = AtomD{x, y, z, R};
+    a.gh[i] = (float)ghost_h(R);
     a.molid[i] = m;
     const float4 f = make_float4((float)x, (float)y, (float)z, h);
     a.f4[i] = f;
@@ -497,13 +500,18 @@ __device__ bool last_block(unsigned* ticket) {
 // Verlet skin test (see dsasa_kernels.cuh): the largest displacement and any changed radius go
 // to vstate[0..1] (zero between calls); the last block decides and clears them.
 __global__ void __launch_bounds__(CHECK_T) k_verlet_check(const double* xyz, const double* radii, const double* ref_xyz,
-                                                          const double* ref_rad, int n, int valid, float lim2, int* vstate) {
+                                                          const double* ref_rad, int n, int valid, float lim2, int* vstate,
+                                                          AtomD* ad) {
     grid_dep_trigger();
     const int i = blockIdx.x * CHECK_T + threadIdx.x;
     float d2 = 0.f;
     int changed = 0;
     if (valid && i < n) {
-        double dx = xyz[3 * i] - ref_xyz[3 * i], dy = xyz[3 * i + 1] - ref_xyz[3 * i + 1], dz = xyz[3 * i + 2] - ref_xyz[3 * i + 2];
+        const double x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
+        ad[i].x = x;
+        ad[i].y = y;
+        ad[i].z = z;
+        double dx = x - ref_xyz[3 * i], dy = y - ref_xyz[3 * i + 1], dz = z - ref_xyz[3 * i + 2];
         double dd = dx * dx + dy * dy + dz * dz;
         d2 = (float)dd * (1.f + 1e-6f);   // rounded up: the test stays conservative
         if (!(dd == dd)) d2 = INFINITY;
@@ -586,11 +594,11 @@ cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, co
 }
 
 cudaError_t launch_verlet_check(const double* xyz, const double* radii, const double* ref_xyz, const double* ref_rad,
-                                int n, int valid, double skin, int* vstate, cudaStream_t s) {
+                                int n, int valid, double skin, int* vstate, AtomD* ad, cudaStream_t s) {
     // (skin / 2)^2, rounded down in float
     const float lim2 = (float)(0.25 * skin * skin) * (1.f - 1e-6f);
     const int nb = valid && n > 0 ? (n + CHECK_T - 1) / CHECK_T : 1;
-    k_verlet_check<<<nb, CHECK_T, 0, s>>>(xyz, radii, ref_xyz, ref_rad, n, valid, lim2, vstate);
+    k_verlet_check<<<nb, CHECK_T, 0, s>>>(xyz, radii, ref_xyz, ref_rad, n, valid, lim2, vstate, ad);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -72,6 +72,19 @@ __device__ __forceinline__ int ds_checked(int idx, int lim, int* status) {
 #define DS_IDX(idx, lim, status) (idx)
 #endif
 
+// An atom as the atom kernels read it in FP64: position and inflated radius in 32 bytes of device
+// memory (the caller's coordinates may lie in host memory, and a neighbour's come as two 16-byte
+// loads instead of four of 8)
+struct alignas(32) AtomD {
+    double x, y, z, R;
+};
+#ifdef __CUDACC__
+__device__ __forceinline__ AtomD load_atom(const AtomD* p) {
+    const double2 a = ((const double2*)p)[0], b = ((const double2*)p)[1];
+    return {a.x, a.y, b.x, b.y};
+}
+#endif
+
 // cell grid of one molecule: cells of edge `cell` starting at `lo`, cell id = base + local
 struct MolGrid {
     float lo[3];
@@ -102,6 +115,8 @@ struct BuildArgs {
     // outputs / scratch
     double* R;         // n
     float2* Rhl;       // n: R as a float pair (hi, lo), for the float-float area terms
+    AtomD* ad;         // n: position and R
+    float* gh;         // n: half-width of the atom's initial cell (ghost_h, exact in float)
     float4* f4;        // n  (x, y, z, R) float
     int* molid;        // n
     int* rank;         // n
@@ -122,6 +137,8 @@ struct AtomArgs {
     const double* xyz;
     const double* R;
     const float2* Rhl;      // R as (hi, lo) floats
+    const AtomD* ad;        // position and R (of this call's coordinates, also when the lists are reused)
+    const float* gh;        // half-width of the initial cell
     const float4* sf4;
     const int* sidx;
     const int* molid;
@@ -209,10 +226,11 @@ struct SRArgs {
 
 cudaError_t launch_build(const BuildArgs& a, cudaStream_t s);
 // Verlet skin test: vstate[2] = reuse the lists (valid, every atom within skin/2 of its
-// reference position, radii unchanged, no list overflow); vstate[3] overflow, the other words
+// reference position, radii unchanged, no list overflow); the positions go to ad, which a build
+// that is not needed does not write; vstate[3] overflow, the other words
 // scratch (zero between calls; 8 words)
 cudaError_t launch_verlet_check(const double* xyz, const double* radii, const double* ref_xyz, const double* ref_rad,
-                                int n, int valid, double skin, int* vstate, cudaStream_t s);
+                                int n, int valid, double skin, int* vstate, AtomD* ad, cudaStream_t s);
 // the Verlet skin test of a batch of resident molecules: reuse[m] for each molecule (see
 // k_verlet_check_batch); vmol: 3 ints per molecule of scratch, ticket: one more, zero between calls
 cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, const double* ref_xyz,

@@ -25,7 +25,9 @@ constexpr size_t al(size_t x) { return (x + 255) & ~size_t(255); }
 // byte offsets of the regions inside the static scratch array (each 256-byte aligned)
 constexpr size_t OFF_R = 0;
 constexpr size_t OFF_RHL = al(OFF_R + sizeof(double) * kMaxAtoms);
-constexpr size_t OFF_F4 = al(OFF_RHL + sizeof(float2) * kMaxAtoms);
+constexpr size_t OFF_AD = al(OFF_RHL + sizeof(float2) * kMaxAtoms);
+constexpr size_t OFF_GH = al(OFF_AD + sizeof(AtomD) * kMaxAtoms);
+constexpr size_t OFF_F4 = al(OFF_GH + sizeof(float) * kMaxAtoms);
 constexpr size_t OFF_MOLID = al(OFF_F4 + sizeof(float4) * kMaxAtoms);
 constexpr size_t OFF_RANK = al(OFF_MOLID + sizeof(int) * kMaxAtoms);
 constexpr size_t OFF_CELL = al(OFF_RANK + sizeof(int) * kMaxAtoms);
@@ -83,6 +85,8 @@ extern "C" dsasa_status dsasa_compute_noalloc(const double* coords, const double
     b.max_cells = (int)kMaxCells;
     b.R = (double*)(base + OFF_R);
     b.Rhl = (float2*)(base + OFF_RHL);
+    b.ad = (AtomD*)(base + OFF_AD);
+    b.gh = (float*)(base + OFF_GH);
     b.f4 = (float4*)(base + OFF_F4);
     b.molid = (int*)(base + OFF_MOLID);
     b.rank = (int*)(base + OFF_RANK);
@@ -102,6 +106,8 @@ extern "C" dsasa_status dsasa_compute_noalloc(const double* coords, const double
     a.xyz = coords;
     a.R = b.R;
     a.Rhl = b.Rhl;
+    a.ad = b.ad;
+    a.gh = b.gh;
     a.sf4 = b.sf4;
     a.sidx = b.sidx;
     a.molid = b.molid;

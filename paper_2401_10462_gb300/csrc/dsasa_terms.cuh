@@ -139,7 +139,8 @@ __global__ void __launch_bounds__(WARPS_TERMS * 32, TermBlocks<R>::value) k_term
         if constexpr (FFM) q = {rq[h].x, rq[h].y, rq[h].z};
         else {
             const int g = DS_IDX(e < np ? max(rg[h], 0) : 0, A.n, A.status);
-            q = {A.xyz[3 * g] - A.xyz[3 * i], A.xyz[3 * g + 1] - A.xyz[3 * i + 1], A.xyz[3 * g + 2] - A.xyz[3 * i + 2]};
+            const AtomD pk = load_atom(A.ad + g), pi = load_atom(A.ad + i);
+            q = {pk.x - pi.x, pk.y - pi.y, pk.z - pi.z};
         }
         S->pq[e][0] = q.x;
         S->pq[e][1] = q.y;
