@@ -46,16 +46,16 @@ constexpr uint8_t NONE = 0xff;
 // and terms kernels
 constexpr int WARPS = 1, WARPS_CELL = 2, WARPS_CLASS = 2, WARPS_TERMS = 2;
 // resident blocks per SM that each kernel's register budget is sized for (one warp each)
-// (the cell kernels: 64 registers and 32 warps an SM; 20,003-atom globule 176 us, against 186 at
-// 18 blocks of 56 registers, 182 at 14, 194 at 12 and 251 at 21)
-constexpr int MINB = 32, MINB_CELL = 16, MINB_TERMS = 18;
+// (whole calls, us: the cell kernel at 16 / 17 / 18 blocks, 5,000 atoms 130.0 / 135.4 / 135.6 - with 18
+// resident blocks the next kernel's find no room before the last one ends - and 20,000-atom MD
+// steps 1283 / 1307 / 1306; the fused kernel at 16 / 18, 304 atoms 84.6 / 79.3)
+constexpr int MINB = 32, MINB_CELL = 16, MINB_CC = 18, MINB_TERMS = 18;
 
 // kernel phases: the whole computation in one kernel, or three kernels that pass the cell
 // through a global record per atom: the cell construction (gather, sort, clipping), the
 // classification (Steps 2a-2c: which simplices of the cell are in C), and the area terms and
 // gradient.  Each kernel's code then fits the instruction cache.
 enum { PH_ALL = 0, PH_CELL = 1, PH_VOL = 4, PH_CC = 5, PH_CARRY = 6 };
-template <int N> struct IntC { static constexpr int value = N; };
 enum { CELL_OK = 0, CELL_DONE = 1 };   // record flag: CELL_DONE = outputs already written
 
 // Per-warp cell storage.  NE plane entries (0..5 ghosts, then the candidates in sorted
@@ -71,7 +71,7 @@ template <class R, int NE, int NT> struct Smem {
     uint8_t start[NE];    // a vertex slot on the face of this plane
     // boundary edges of the current cut, by number: planes a, b and the kept neighbour's slot,
     // one byte each; the new vertex on the edge that ends at plane b
-    unsigned bedge[NE];
+    unsigned bedge[NE < 96 ? 96 : NE];
     uint8_t bslot[NE], eslot[NE];
     uint8_t ord[NE];      // clipping order (entry ids)
     uint8_t eflag[NE];    // face summary: bit0 edge in C, bit1 interior (closed)
@@ -580,6 +580,209 @@ namespace dsasa {
 
 namespace {
 
+// ------------------------------------------------------------------ clipping
+// The cell during the clipping: slot t = 32 r + lane in the lane's registers.
+constexpr unsigned ALIVE = 0x80000000u;   // TV: a live vertex (else the slot's stack position)
+enum { CUT_DONE = 0, CUT_EMPTY = 1, CUT_FULL = 2 };
+template <class R, int NR> struct ClipState {
+    static constexpr bool LOOSE = sizeof(R) == 4;
+    unsigned TV[NR], TA[NR];             // planes (dead slot: its place in the free stack), neighbours
+    R V[NR][4], Vs[NR], Va[NR][LOOSE ? 1 : 4];
+    int hw = 8, sp = 0;                  // slots used so far, free-stack pointer: 8 - sp vertices are alive
+    bool nothing = false;                // the last cut removed every vertex
+
+    __device__ __forceinline__ void init(int lane) {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            TV[r] = (unsigned)(1024 + 7 - (r * 32 + lane));
+            TA[r] = 0;
+        }
+    }
+    // the coordinates of slot r's vertex from its planes
+    template <class SM> __device__ __forceinline__ void vertex(const SM* S, int r) {
+        const unsigned w = TV[r];
+        const int a = w & 127u, b = (w >> 8) & 127u, m = (w >> 16) & 127u;
+        if constexpr (LOOSE) {
+            new_vertex(*(const float4*)S->pq[a], *(const float2*)S->pm[a], *(const float4*)S->pq[b],
+                       *(const float2*)S->pm[b], *(const float4*)S->pq[m], *(const float2*)S->pm[m], V[r], Vs[r]);
+        } else {
+            const VtxFA<R> q = vertex_fa(S, make_uchar4((uint8_t)a, (uint8_t)b, (uint8_t)m, 0));
+            for (int k = 0; k < 4; ++k) {
+                V[r][k] = q.v[k];
+                Va[r][k] = q.a[k];
+            }
+        }
+    }
+    // the tests of every vertex against plane m: bit r of remv, the lane's vertex r is beyond it;
+    // true if the filter left a test of the warp open
+    template <class SM> __device__ __forceinline__ bool test(const SM* S, int m, unsigned& remv) {
+        bool open = false;
+        remv = 0;
+        if constexpr (LOOSE) {
+            // |q . Dv - b D| errs by at most gamma times the sum of its magnitudes, which is at most
+            // max(|q|_1, |b|) Vs; the floor stands for underflow
+            const float4 M = *(const float4*)S->pq[m];
+            const float2 mm = *(const float2*)S->pm[m];
+            const float qm = fmaxf(mm.x, mm.y) * Gam<R>::gclip;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const float sv = M.x * V[r][0] + M.y * V[r][1] + M.z * V[r][2] - M.w * V[r][3];
+                const float lim = fmaf(qm, Vs[r], Gam<R>::tiny);
+                const bool on = (int)TV[r] < 0;
+                if (on && sv > lim) remv |= 1u << r;
+                if (on && !(fabsf(sv) > lim)) open = true;
+            }
+        } else {
+            const PlaneN<FA<R>> M = fplane(S, m);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                if ((int)TV[r] >= 0) continue;
+                FA<R> sv;
+                sv.v = M.q.x.v * V[r][0] + M.q.y.v * V[r][1] + M.q.z.v * V[r][2] - M.b.v * V[r][3];
+                sv.a = M.q.x.a * Va[r][0] + M.q.y.a * Va[r][1] + M.q.z.a * Va[r][2] + M.b.a * Va[r][3];
+                const int sg = fa_sign(sv, Gam<R>::gclip, Gam<R>::tiny);
+                if (sg > 0) remv |= 1u << r;
+                else if (sg == 0) open = true;
+            }
+        }
+        return __any_sync(FULL, open);
+    }
+    // the cut by plane m of the vertices in remv; CUT_FULL: the cell is as before, a slot is missing
+    template <class SM> __device__ __forceinline__ int cut(SM* S, int m, unsigned remv, int lane) {
+        constexpr int NE = SM::kNE;
+        const unsigned lt = lanemask_lt();
+        unsigned bal[NR];
+        int nrem = 0;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            bal[r] = __ballot_sync(FULL, remv >> r & 1);
+            nrem += __popc(bal[r]);
+        }
+        if (nrem == 0) return CUT_DONE;
+        if (nrem == 8 - sp) {
+            nothing = true;
+            return CUT_EMPTY;
+        }
+        // bit 0: the slot in the low byte of x was removed by this cut (one slot per lane: the shift
+        // takes its low five bits by itself)
+        auto removed = [&](unsigned x) -> unsigned {
+            unsigned w = bal[0];
+#pragma unroll
+            for (int r = 1; r < NR; ++r)
+                if (((x >> 5) & 7u) == (unsigned)r) w = bal[r];
+            return __funnelshift_r(w, 0u, x);
+        };
+        // the removed neighbours of each vertex, and the boundary edges of the removed region:
+        // edge (a -> b) of a removed triangle whose neighbour is kept
+        unsigned nbr[NR];
+        int nb = 0;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const unsigned ta = TA[r];
+            const unsigned n0 = removed(ta), n1 = removed(ta >> 8), n2 = removed(ta >> 16);
+            nbr[r] = (n0 & 1u) | (n1 & 1u) << 1 | (n2 & 1u) << 2;
+            const bool rm = remv >> r & 1;
+            const bool f0 = rm && !(n0 & 1u), f1 = rm && !(n1 & 1u), f2 = rm && !(n2 & 1u);
+            const unsigned b0 = __ballot_sync(FULL, f0), b1 = __ballot_sync(FULL, f1), b2 = __ballot_sync(FULL, f2);
+            const int e = nb + __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt);
+            nb += __popc(b0) + __popc(b1) + __popc(b2);
+            constexpr int EM = NR == 1 ? 127 : NE - 1;   // (one slot per lane: at most 3 x 31 edges)
+            unsigned* be = S->bedge;
+            if (f0) be[e & EM] = __byte_perm(TV[r], ta, 0x3410);
+            if (f1) be[(e + f0) & EM] = __byte_perm(TV[r], ta, 0x3521);
+            if (f2) be[(e + f0 + f1) & EM] = __byte_perm(TV[r], ta, 0x3602);
+        }
+        const int sp2 = sp + nrem - nb, hw2 = max(hw, 8 - sp2);
+        if (hw2 > 32 * NR || nb > NE) return CUT_FULL;
+        __syncwarp();
+        // the new vertices: the owner of boundary edge e's slot takes it
+        unsigned fresh[NR];   // ALIVE, kept neighbour, planes b and a; 0: not new
+        int before = 0;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int t = r * 32 + lane;
+            const bool rm = remv >> r & 1;
+            const int e = rm ? before + __popc(bal[r] & lt) : nrem + sp + 1023 - (int)TV[r];
+            before += __popc(bal[r]);
+            fresh[r] = 0;
+            if ((rm || (int)TV[r] >= 0) && e < nb) {
+                const unsigned w = S->bedge[e];   // (bit 31 set: the removed vertex was alive)
+                S->start[w & 255u] = (uint8_t)t;            // the new triangle on the edge that starts at a
+                S->eslot[(w >> 8) & 255u] = (uint8_t)t;     // ... and ends at b
+                if (e == 0) S->start[m] = (uint8_t)t;
+                fresh[r] = w;
+            } else if (rm) {   // a removed slot left over: onto the free stack
+                TV[r] = (unsigned)(1024 + sp + e - nb);
+            }
+        }
+        sp = sp2;
+        hw = hw2;
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const unsigned w = fresh[r];
+            if (w) {
+                TV[r] = __byte_perm(w, m, 0x3410);
+                TA[r] = pack3((w >> 16) & 127u, S->start[(w >> 8) & 255u], S->eslot[w & 255u]);
+                vertex(S, r);
+            } else if ((int)TV[r] < 0) {
+                // a kept vertex: its edge (b -> a) towards a removed one now borders the new
+                // triangle on the edge that starts at a
+                const unsigned v = TV[r];
+                if (nbr[r] & 1u) TA[r] = __byte_perm(TA[r], S->start[(v >> 8) & 255u], 0x3214);
+                if (nbr[r] & 2u) TA[r] = __byte_perm(TA[r], S->start[(v >> 16) & 127u], 0x3240);
+                if (nbr[r] & 4u) TA[r] = __byte_perm(TA[r], S->start[v & 255u], 0x3410);
+            }
+        }
+        return CUT_DONE;
+    }
+};
+
+// The clipping of a cell by planes kk .. nc - 1 with every slot of the table, tests that the filter
+// leaves open resolved exactly.  In: slots 0 - 31 in tv and ta (kf: alive; a dead slot's tv holds its
+// place in the free stack), sp and hw.  Out: tv and ta of every slot, hw, bad.  Returns whether the
+// cell is empty.  Out of line: rare, and apart from the registers of the loop it is called after.
+template <class SM, class R = typename SM::Real>
+__device__ __noinline__ bool clip_rest(SM* S, const AtomArgs& A, int i, int nc, int kk, int sp, int hw) {
+    constexpr int NR = SM::kNT / 32;
+    const int lane = threadIdx.x & 31;
+    ClipState<R, NR> st;
+    st.init(lane);
+    st.sp = sp;
+    st.hw = hw;
+    {
+        const uchar4 v = S->tv[lane], w = S->ta[lane];
+        st.TV[0] = pack3(v.x, v.y, v.z) | (S->kf[lane] ? ALIVE : 0u);
+        st.TA[0] = pack3(w.x, w.y, w.z);
+        if (S->kf[lane]) st.vertex(S, 0);
+    }
+    __syncwarp();
+    for (; kk < nc; ++kk) {
+        const int m = NG + kk;
+        unsigned remv;
+        if (st.test(S, m, remv)) {
+            remv = 0;
+#pragma unroll
+            for (int r = 0; r < NR; ++r)
+                if ((int)st.TV[r] < 0 && clip_sign(S, A.xyz, A.R, i, A.n, A.status, st.TV[r], m) > 0) remv |= 1u << r;
+        }
+        const int c = st.cut(S, m, remv, lane);
+        if (c == CUT_EMPTY) return true;
+        if (c == CUT_FULL) {
+            if (lane == 0) S->bad = 2;
+            break;
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        S->tv[r * 32 + lane] = unpack3((int)st.TV[r] < 0 ? st.TV[r] : DEADV);
+        S->ta[r * 32 + lane] = unpack3(st.TA[r]);
+    }
+    if (lane == 0) S->hw = st.hw;
+    __syncwarp();
+    return false;
+}
+
 // ------------------------------------------------------------------ carried cells
 // The incremental update of C across MD steps.  On a call that reuses the neighbour lists
 // (every atom within half the skin of its last rebuild), the cell that the previous call
@@ -751,13 +954,14 @@ __device__ __noinline__ int carry_cell(SM* S, const RC* rec, int i, int n, int n
 
 // ------------------------------------------------------------------ the kernel
 __host__ __device__ constexpr int minb(int ph) {
-    return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? MINB_CELL : (ph == PH_VOL ? MINB_TERMS : MINB);
+    if (ph == PH_CC) return MINB_CC;
+    return (ph == PH_CELL || ph == PH_CARRY) ? MINB_CELL : (ph == PH_VOL ? MINB_TERMS : MINB);
 }
 __host__ __device__ constexpr int warps_of(int ph) {
     return (ph == PH_CELL || ph == PH_CC || ph == PH_CARRY) ? WARPS_CELL : (ph == PH_VOL ? WARPS_TERMS : WARPS);
 }
 template <class R, bool GRAD, int NE, int NT, int PHX>
-__global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArgs A) {
+__global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(const __grid_constant__ AtomArgs A) {
     // PH_CARRY: the carried cells of list-reusing calls (the other atoms go to the redo list)
     constexpr bool CARRY = PHX == PH_CARRY;
     constexpr int PH = CARRY ? PH_CELL : PHX;
@@ -1227,178 +1431,65 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(AtomArg
         // Free slots are a stack whose positions live with the slots (in TV): slot t starts at
         // position 7 - t (the slots past the cube's 8, lowest on top), sp is the position above
         // the top, and 8 - sp vertices are alive.
-        // The loop runs with one slot per lane (NR = 1) until a cut needs slot 32, which most
-        // cells never do, and goes on from there with NT / 32: the common loop then holds one
-        // vertex per lane in registers and tests one word of removed bits.
+        // The loop runs with one slot per lane until a cut needs slot 32, which most cells never do,
+        // or a test is left open by the filter, which is rare: it holds one vertex per lane in
+        // registers, tests one word of removed bits and makes no call (with one inside, the
+        // compiler kept the loop's state in local memory: 28 spill operations a cut).  clip_rest
+        // finishes such cells out of line.
         if constexpr (!CARRY) {
-        constexpr unsigned ALIVE = 0x80000000u;   // TV: a live vertex (else the slot's stack position)
-        const unsigned lt = lanemask_lt();
-        int hw = 8, sp = 0;   // slots used so far, free-stack pointer
-#pragma unroll
-        for (int r = 0; r < SPL; ++r) {
-            TV[r] = (unsigned)(1024 + 7 - (r * 32 + lane));
-            TA[r] = 0;
-        }
-        // the coordinates of the vertex on planes a, b (bytes of w) and m
-        auto make_vertex = [&](int r, unsigned w, int m) {
-            const int a = w & 255u, b = (w >> 8) & 255u;
-            if constexpr (LOOSE) {
-                new_vertex(*(const float4*)S->pq[a], *(const float2*)S->pm[a], *(const float4*)S->pq[b],
-                           *(const float2*)S->pm[b], *(const float4*)S->pq[m], *(const float2*)S->pm[m], V[r], Vs[r]);
-            } else {
-                const VtxFA<R> q = vertex_fa(S, make_uchar4((uint8_t)a, (uint8_t)b, (uint8_t)m, 0));
-                for (int k = 0; k < 4; ++k) {
-                    V[r][k] = q.v[k];
-                    Va[r][k] = q.a[k];
-                }
-            }
-        };
+        ClipState<R, 1> st;
+        st.init(lane);
         if (lane < 8) {
             const int sh = 8 * lane;
-            TV[0] = ALIVE | pack3((unsigned)(CUBE_PL0 >> sh) & 255u, (unsigned)(CUBE_PL1 >> sh) & 255u,
-                                  (unsigned)(CUBE_PL2 >> sh) & 255u);
-            TA[0] = pack3((unsigned)(CUBE_ADJ0 >> sh) & 255u, (unsigned)(CUBE_ADJ1 >> sh) & 255u,
-                          (unsigned)(CUBE_ADJ2 >> sh) & 255u);
-            make_vertex(0, TV[0], (TV[0] >> 16) & 127u);
+            st.TV[0] = ALIVE | pack3((unsigned)(CUBE_PL0 >> sh) & 255u, (unsigned)(CUBE_PL1 >> sh) & 255u,
+                                     (unsigned)(CUBE_PL2 >> sh) & 255u);
+            st.TA[0] = pack3((unsigned)(CUBE_ADJ0 >> sh) & 255u, (unsigned)(CUBE_ADJ1 >> sh) & 255u,
+                             (unsigned)(CUBE_ADJ2 >> sh) & 255u);
+            st.vertex(S, 0);
         }
         int kk = 0;
-        // clips by planes kk .. nc - 1 with NR slots per lane; true: a cut needs more slots
-        auto clip = [&](auto nrc) -> bool {
-        constexpr int NR = decltype(nrc)::value;
-        unsigned rsv = 0;          // removal bits of plane kk resolved outside the inner loop; bit 31: valid
-        for (;;) {
-        bool open_tests = false;
         for (; kk < nc; ++kk) {
-            const int m = NG + kk;
-            unsigned remv = 0;
-            if (rsv) {
-                remv = rsv & ~ALIVE;
-                rsv = 0;
-            } else {
-                bool open = false;
-                if constexpr (LOOSE) {
-                    // |q . Dv - b D| errs by at most gamma times the sum of its magnitudes, which
-                    // is at most max(|q|_1, |b|) Vs; the floor stands for underflow
-                    const float4 M = *(const float4*)S->pq[m];
-                    const float2 mm = *(const float2*)S->pm[m];
-                    const float qm = fmaxf(mm.x, mm.y) * Gam<R>::gclip;
-#pragma unroll
-                    for (int r = 0; r < NR; ++r) {
-                        const float sv = M.x * V[r][0] + M.y * V[r][1] + M.z * V[r][2] - M.w * V[r][3];
-                        const float lim = fmaf(qm, Vs[r], Gam<R>::tiny);
-                        const bool on = (int)TV[r] < 0;
-                        if (on && sv > lim) remv |= 1u << r;
-                        if (on && !(fabsf(sv) > lim)) open = true;
-                    }
-                } else {
-                    const PlaneN<FA<R>> M = fplane(S, m);
-#pragma unroll
-                    for (int r = 0; r < NR; ++r) {
-                        if ((int)TV[r] >= 0) continue;
-                        FA<R> sv;
-                        sv.v = M.q.x.v * V[r][0] + M.q.y.v * V[r][1] + M.q.z.v * V[r][2] - M.b.v * V[r][3];
-                        sv.a = M.q.x.a * Va[r][0] + M.q.y.a * Va[r][1] + M.q.z.a * Va[r][2] + M.b.a * Va[r][3];
-                        const int sg = fa_sign(sv, Gam<R>::gclip, Gam<R>::tiny);
-                        if (sg > 0) remv |= 1u << r;
-                        else if (sg == 0) open = true;
-                    }
-                }
-                open_tests = __any_sync(FULL, open);
-                if (open_tests) break;
-            }
-            unsigned bal[NR];
-            int nrem = 0;
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                bal[r] = __ballot_sync(FULL, remv >> r & 1);
-                nrem += __popc(bal[r]);
-            }
-            if (nrem == 0) continue;
-            if (nrem == 8 - sp) { empty = true; break; }
-            auto removed = [&](unsigned t2) -> unsigned {   // bit 0: slot t2 removed by this cut
-                unsigned w = bal[0];
-#pragma unroll
-                for (int r = 1; r < NR; ++r)
-                    if ((t2 >> 5) == (unsigned)r) w = bal[r];
-                return w >> (t2 & 31u);
-            };
-            // the removed neighbours of each vertex, and the boundary edges of the removed region:
-            // edge (a -> b) of a removed triangle whose neighbour is kept
-            unsigned nbr[NR];
-            int nb = 0;
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const unsigned ta = TA[r];
-                nbr[r] = (removed(ta & 255u) & 1u) | (removed((ta >> 8) & 255u) & 1u) << 1 |
-                         (removed(ta >> 16) & 1u) << 2;
-                const unsigned f = (remv >> r & 1) ? (~nbr[r] & 7u) : 0u;
-                const int cnt = __popc(f);
-                const unsigned c0 = __ballot_sync(FULL, cnt & 1), c1 = __ballot_sync(FULL, cnt & 2);
-                int e = nb + __popc(c0 & lt) + 2 * __popc(c1 & lt);
-                nb += __popc(c0) + 2 * __popc(c1);
-                if (f & 1u) S->bedge[e++ & (NE - 1)] = __byte_perm(TV[r], ta, 0x3410);
-                if (f & 2u) S->bedge[e++ & (NE - 1)] = __byte_perm(TV[r], ta, 0x3521);
-                if (f & 4u) S->bedge[e & (NE - 1)] = __byte_perm(TV[r], ta, 0x3602);
-            }
-            const int sp2 = sp + nrem - nb, hw2 = max(hw, 8 - sp2);
-            if (hw2 > 32 * NR && NR < SPL) return true;
-            if (hw2 > NT || nb > NE) {
-                if (lane == 0) S->bad = 2;
-                break;
-            }
-            __syncwarp();
-            // the new vertices: the owner of boundary edge e's slot takes it
-            unsigned fresh[NR];   // ALIVE, kept neighbour, planes b and a; 0: not new
-            int before = 0;
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const int t = r * 32 + lane;
-                const bool rm = remv >> r & 1;
-                const int e = rm ? before + __popc(bal[r] & lt) : nrem + sp + 1023 - (int)TV[r];
-                before += __popc(bal[r]);
-                fresh[r] = 0;
-                if ((rm || (int)TV[r] >= 0) && e < nb) {
-                    const unsigned w = S->bedge[e];   // (bit 31 set: the removed vertex was alive)
-                    S->start[w & 255u] = (uint8_t)t;            // the new triangle on the edge that starts at a
-                    S->eslot[(w >> 8) & 255u] = (uint8_t)t;     // ... and ends at b
-                    if (e == 0) S->start[m] = (uint8_t)t;
-                    fresh[r] = w;
-                } else if (rm) {   // a removed slot left over: onto the free stack
-                    TV[r] = (unsigned)(1024 + sp + e - nb);
-                }
-            }
-            sp = sp2;
-            hw = hw2;
-            __syncwarp();
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const unsigned w = fresh[r];
-                if (w) {
-                    TV[r] = __byte_perm(w, m, 0x3410);
-                    TA[r] = pack3((w >> 16) & 127u, S->start[(w >> 8) & 255u], S->eslot[w & 255u]);
-                    make_vertex(r, w, m);
-                } else if ((int)TV[r] < 0) {
-                    // a kept vertex: its edge (b -> a) towards a removed one now borders the new
-                    // triangle on the edge that starts at a
-                    const unsigned v = TV[r];
-                    if (nbr[r] & 1u) TA[r] = __byte_perm(TA[r], S->start[(v >> 8) & 255u], 0x3214);
-                    if (nbr[r] & 2u) TA[r] = __byte_perm(TA[r], S->start[(v >> 16) & 127u], 0x3240);
-                    if (nbr[r] & 4u) TA[r] = __byte_perm(TA[r], S->start[v & 255u], 0x3410);
-                }
-            }
+            unsigned remv;
+            if (st.test(S, NG + kk, remv)) break;
+            if (st.cut(S, NG + kk, remv, lane) != CUT_DONE) break;
         }
-        if (!open_tests) return false;
-        // the tests of plane kk that the filter left open: tight magnitudes, then exact (out of
-        // the inner loop, which makes no call: with a call inside, the compiler kept the loop's
-        // state in local memory)
-        rsv = ALIVE;
+        empty = st.nothing;
+        int hw = st.hw;
 #pragma unroll
-        for (int r = 0; r < NR; ++r)
-            if ((int)TV[r] < 0 && clip_sign(S, A.xyz, A.R, i, A.n, A.status, TV[r], NG + kk) > 0) rsv |= 1u << r;
+        for (int r = 0; r < SPL; ++r) {
+            TV[r] = r == 0 ? st.TV[0] : 0u;
+            TA[r] = r == 0 ? st.TA[0] : 0u;
         }
-        };
-        if (clip(IntC<1>{})) {
-            if constexpr (SPL > 1) clip(IntC<SPL>{});
+        if (kk < nc && !empty) {
+            // a test left open or no slot free: the cell so far through shared memory, and back
+            S->tv[lane] = unpack3(st.TV[0]);
+            S->ta[lane] = unpack3(st.TA[0]);
+            S->kf[lane] = (uint8_t)((int)st.TV[0] < 0);
+            __syncwarp();
+            empty = clip_rest(S, A, i, nc, kk, st.sp, st.hw);
+            hw = S->hw;
+#pragma unroll
+            for (int r = 0; r < SPL; ++r) {
+                const uchar4 v = S->tv[r * 32 + lane], w = S->ta[r * 32 + lane];
+                TV[r] = pack3(v.x, v.y, v.z);
+                if (TV[r] != DEADV) TV[r] |= ALIVE;
+                TA[r] = pack3(w.x, w.y, w.z);
+            }
+            if constexpr (PH != PH_CELL) {
+                ClipState<R, SPL> all;
+#pragma unroll
+                for (int r = 0; r < SPL; ++r) {
+                    all.TV[r] = TV[r];
+                    if ((int)TV[r] < 0) all.vertex(S, r);
+                    for (int k = 0; k < 4; ++k) V[r][k] = all.V[r][k];
+                    Vs[r] = all.Vs[r];
+                    for (int k = 0; k < (LOOSE ? 1 : 4); ++k) Va[r][k] = all.Va[r][k];
+                }
+            }
+        } else if constexpr (PH != PH_CELL) {
+            for (int k = 0; k < 4; ++k) V[0][k] = st.V[0][k];
+            Vs[0] = st.Vs[0];
+            for (int k = 0; k < (LOOSE ? 1 : 4); ++k) Va[0][k] = st.Va[0][k];
         }
         // the vertices alive, their planes alone (dead slots: NONE)
         nrounds = (hw + 31) >> 5;

@@ -6,20 +6,18 @@
 namespace dsasa {
 namespace {
 
-// Whether the cell construction and the classification run as one kernel: up to half as many
-// atoms as the GPU holds warps of it (2,432 on a GB300).  There an atom's classification
-// overlaps the slowest cells and one launch and the trip of the records through memory are
-// saved; with more atoms the split kernels win, whose smaller instruction streams stay in the
-// cache (fused / split, us per call with the gradient: 2,003 atoms 105 / 112, 2,500 116 / 115,
-// 3,500 136 / 131, 4,800 150.2 / 150.0).
+// Whether the cell construction and the classification run as one kernel: up to 10 atoms a
+// multiprocessor (1,520 on a GB300).  There an atom's classification overlaps the slowest cells and
+// one launch and the trip of the records through memory are saved; with more atoms the split
+// kernels win, whose smaller instruction streams stay in the cache (fused / split, us per call with
+// the gradient: 304 atoms 76 / 81, 700 82 / 90, 1,200 133 / 138, 2,003 107 / 104, 3,000 132 / 119).
 bool cells_fused(int n) {
     static int cap = -1;
     if (cap < 0) {
-        int dev = 0, sms = 0, per = 0;
+        int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_atoms<float, false, 64, 64, PH_CC>, WARPS_CELL * 32, 0);
-        cap = sms * per * WARPS_CELL / 2;
+        cap = 10 * sms;
     }
     return n <= cap;
 }

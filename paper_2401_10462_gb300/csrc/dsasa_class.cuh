@@ -307,7 +307,7 @@ struct alignas(16) ClassSmem {
 
 // (a template, so that only the unit that launches it compiles it)
 template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32, MINB_CLASS) k_class(AtomArgs A) {
+__global__ void __launch_bounds__(WARPS * 32, MINB_CLASS) k_class(const __grid_constant__ AtomArgs A) {
     __shared__ ClassSmem smem_all[WARPS];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     ClassSmem* S = &smem_all[wib];
