@@ -26,6 +26,7 @@ template <> struct TermBlocks<double> { static constexpr int value = 10; };
 template <class R, bool GRAD> struct alignas(16) TermSmem {
     R pq[64][4];                      // plane vector q and its length
     R dih[3 * 64][GRAD ? 4 : 1];      // by 3 t + k: (the gradient and) the angle, last
+    R inv[sizeof(R) == 8 ? 64 : 1];   // 1 / |q| (FP64 form)
     int pg[64];
     uchar4 tv[64], ta[64];            // cell vertices (planes; w: kf), their neighbours (w: tf)
     uint8_t start[64], eflag[64], face[64];
@@ -51,27 +52,29 @@ template <class R> __device__ __forceinline__ R dihedral_o(P3<R> a, R la, P3<R> 
 //          + 2 theta_ia / |u| (w_i R_i (1 - b_u/(u.u)) + w_a R_a b_u/(u.u)) u + (the same for b),
 // and S_iab^(i) = 2 pi R_i^2 - 2 R_i (b_u theta_ia / |u| + b_w theta_ib / |w|) - 2 R_i^2 theta_ix.
 // The lens gradients one owner at a time and Eq. (trianglev) took 9 atan2 and about 40 divisions
-// and square roots a triangle; this takes 3 and 9, one atan2 on each of 3 lanes.
+// and square roots a triangle; this takes 3 and 2, one atan2 on each of 3 lanes (the lengths come from the table of planes).
 struct TriGram {
     P3<double> u, w, n;          // n = u x w
     double uu, ww, uw, bu, bw;   // Gram entries, bisector offsets
+    double nn;                   // |n|^2
     double iu, iw, in;           // 1 / |u|, 1 / |w|, 1 / |n|
     double h;                    // s
 };
-__device__ __forceinline__ TriGram tri_gram(P3<double> u, P3<double> w, double Ri, double Ra, double Rb) {
+__device__ __forceinline__ TriGram tri_gram(P3<double> u, P3<double> w, double lu, double lw, double iu, double iw,
+                                            double Ri, double Ra, double Rb) {
     TriGram g;
     g.u = u;
     g.w = w;
     g.n = cross3(u, w);
-    g.uu = dot3(u, u);
-    g.ww = dot3(w, w);
+    g.uu = lu * lu;
+    g.ww = lw * lw;
     g.uw = dot3(u, w);
     g.bu = 0.5 * (g.uu + (Ri - Ra) * (Ri + Ra));
     g.bw = 0.5 * (g.ww + (Ri - Rb) * (Ri + Rb));
-    g.iu = rsqrt(g.uu);
-    g.iw = rsqrt(g.ww);
-    const double nn = dot3(g.n, g.n);
-    g.in = rsqrt(nn);
+    g.iu = iu;
+    g.iw = iw;
+    g.nn = dot3(g.n, g.n);
+    g.in = rsqrt(g.nn);
     const P3<double> z = cross3(w, g.n) * g.bu + cross3(g.n, u) * g.bw;   // |n|^2 times the foot of x
     const double in2 = g.in * g.in;
     const double s2 = Ri * Ri - dot3(z, z) * in2 * in2;
@@ -145,7 +148,12 @@ __global__ void __launch_bounds__(WARPS_TERMS * 32, TermBlocks<R>::value) k_term
         S->pq[e][0] = q.x;
         S->pq[e][1] = q.y;
         S->pq[e][2] = q.z;
-        S->pq[e][3] = norm3(q);
+        if constexpr (FFM) S->pq[e][3] = norm3(q);
+        else {
+            const R qq = dot3(q, q), iq = rsqrt(qq);
+            S->inv[e] = iq;
+            S->pq[e][3] = qq * iq;
+        }
         S->pg[e] = rg[h];
         S->start[e] = rs[h];
         S->eflag[e] = re[h];
@@ -191,8 +199,23 @@ __global__ void __launch_bounds__(WARPS_TERMS * 32, TermBlocks<R>::value) k_term
         const int a = tv_get(v, k);
         const P3<R> pa = pos(a), pb = pos(tv_get(v, (k + 1) % 3)), pc = pos(tv_get(v, (k + 2) % 3));
         const R la = plen(a);
-        const R th = dihedral_o(pa, la, pb, pc);
         R* d = S->dih[3 * t + k];
+        if constexpr (!FFM) {
+            // the angle and its gradient d/dp_i (dihedral_grad_s for a positive orientation) with one
+            // division and the length from the table
+            const P3<R> mc = cross3(pa, pb), md = cross3(pa, pc);
+            const R v6 = dot3(mc, pc);
+            d[GRAD ? 3 : 0] = atan2(la * fabs(v6), dot3(mc, md));
+            if constexpr (GRAD) {
+                const R mc2 = dot3(mc, mc), md2 = dot3(md, md), f = la / (mc2 * md2), i2 = S->inv[a] * S->inv[a];
+                const R cb = f * md2 * ((R)1 - dot3(pb, pa) * i2), cd = f * mc2 * (dot3(pc, pa) * i2 - (R)1);
+                d[0] = mc.x * cb + md.x * cd;
+                d[1] = mc.y * cb + md.y * cd;
+                d[2] = mc.z * cb + md.z * cd;
+            }
+            continue;
+        }
+        const R th = dihedral_o(pa, la, pb, pc);
         if constexpr (GRAD) {
             // (i, a, b, c) is positively oriented: (a, b, c) is counter-clockwise
             const P3<R> O = {zero, zero, zero};
@@ -250,7 +273,7 @@ __global__ void __launch_bounds__(WARPS_TERMS * 32, TermBlocks<R>::value) k_term
         // R_i h_i (sum(theta) - 2 pi); h_i = (R_i + R_a - d)(R_a - R_i + d) / 2d
         const P3<R> pa = pos(a);
         const int ga = DS_IDX(S->pg[a], A.n, A.status);
-        const R dr = plen(a), inv2d = (R)0.5 / dr;
+        const R dr = plen(a), inv2d = FFM ? (R)0.5 / dr : (R)0.5 * S->inv[FFM ? 0 : a];
         R Raf, dR2;
         if constexpr (FFM) {
             const float2 ra2 = A.Rhl[ga];
@@ -273,7 +296,9 @@ __global__ void __launch_bounds__(WARPS_TERMS * 32, TermBlocks<R>::value) k_term
             // vertex + edge parts of the dihedral derivatives around ia (Eq. inexclu)
             const R kap = -(wif * Rr * ti + waf * Raf * ta);
             // cap derivatives (Eq. edge): -Phi (2 pi / d)(w_i R_i t_a + w_a R_a t_i) u
-            const R cf = -phi * (R)TWO_PI / (dr * dr) * (wif * Rr * ta + waf * Raf * ti);
+            R cf;
+            if constexpr (FFM) cf = -phi * (R)TWO_PI / (dr * dr) * (wif * Rr * ta + waf * Raf * ti);
+            else cf = -phi * (R)TWO_PI * (S->inv[a] * S->inv[a]) * (wif * Rr * ta + waf * Raf * ti);
             gacc.add(kap * gsum.x + cf * pa.x, kap * gsum.y + cf * pa.y, kap * gsum.z + cf * pa.z);
         }
     }
@@ -401,11 +426,11 @@ __global__ void __launch_bounds__(WARPS_TERMS * 32, TermBlocks<R>::value) k_term
             const P3<R> pa = pos(a), pb = pos(b);
             const int ga = DS_IDX(S->pg[a & 63], A.n, A.status), gb = DS_IDX(S->pg[b & 63], A.n, A.status);
             const double Ra = A.R[ga], Rb = A.R[gb];
-            const TriGram g = tri_gram(pa, pb, Ri, Ra, Rb);
-            const double nn = dot3(g.n, g.n);
-            const double sn = g.h * (nn * g.in);   // s |u x w|
+            const double la = plen(a), lb = plen(b);
+            const TriGram g = tri_gram(pa, pb, la, lb, S->inv[a & 63], S->inv[b & 63], Ri, Ra, Rb);
+            const double sn = g.h * (g.nn * g.in);   // s |u x w|
             // this lane's angle: along (i, a), (i, b), (i, x)
-            const double num = sn * (part == 0 ? g.uu * g.iu : (part == 1 ? g.ww * g.iw : Ri));
+            const double num = sn * (part == 0 ? la : (part == 1 ? lb : Ri));
             const double den = part == 0 ? g.uu * g.bw - g.uw * g.bu
                                          : (part == 1 ? g.ww * g.bu - g.uw * g.bw : Ri * Ri * g.uw - g.bu * g.bw);
             const double th = atan2(num, den);
@@ -455,9 +480,22 @@ __global__ void __launch_bounds__(WARPS_TERMS * 32, TermBlocks<R>::value) k_term
         for (int o = 16; o > 0; o >>= 1) cf_sum += __shfl_xor_sync(FULL, cf_sum, o);
         area_acc = ff_to_double(tot) + ((double)cf_sum + (double)vtx_const) * TWO_PI * Ri * Ri;
     } else {
-        area_acc = warp_sum_d(area_acc);
+        // the four sums together: lanes 8 k .. 8 k + 7 end with sum k (6 FP64 additions instead of 20)
+        const bool up = lane & 16, odd = lane & 8;
+        double s0 = up ? gacc.y : area_acc, s1 = up ? gacc.z : gacc.x;
+        const double o0 = up ? area_acc : gacc.y, o1 = up ? gacc.x : gacc.z;
+        s0 += __shfl_xor_sync(FULL, o0, 16);
+        s1 += __shfl_xor_sync(FULL, o1, 16);
+        double t0 = odd ? s1 : s0;
+        const double t1 = odd ? s0 : s1;
+        t0 += __shfl_xor_sync(FULL, t1, 8);
+        for (int o = 4; o > 0; o >>= 1) t0 += __shfl_xor_sync(FULL, t0, o);
+        area_acc = t0;   // (lane 0)
+        gx = __shfl_sync(FULL, t0, 8);
+        gy = __shfl_sync(FULL, t0, 16);
+        gz = __shfl_sync(FULL, t0, 24);
     }
-    if constexpr (GRAD) gacc.reduce(gx, gy, gz);
+    if constexpr (GRAD && FFM) gacc.reduce(gx, gy, gz);
     if (lane == 0) {
         A.areas[i] = iK ? area_acc : 0.0;
         if (GRAD && A.grad) {
