@@ -113,7 +113,9 @@ def nonpolar_energy(coords, radii, gamma=GAMMA, probe: float = api.PROBE, precis
     """E_np = sum_i gamma_i A_i (differentiable in coords); also returns the areas."""
     if lib_ctx is None:
         lib_ctx = _Ctxs.get(coords.device.index or 0, precision)
-    g = gamma if torch.is_tensor(gamma) else torch.tensor(float(gamma), dtype=torch.float64, device=coords.device)
+    # (filled on the device: a tensor made from a host scalar is copied there and waits for the
+    # stream, which left the GPU idle while the call's kernels were launched)
+    g = gamma if torch.is_tensor(gamma) else torch.full((), float(gamma), dtype=torch.float64, device=coords.device)
     return NonpolarEnergy.apply(coords, radii, g, probe, lib_ctx)
 
 
