@@ -1083,7 +1083,10 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(const _
         }
         if (reuse) {
             // the list holds every atom within R_i + R_j + skin at the last rebuild; keep the
-            // ones whose balls overlap B_i now (float64, with a relative slack of 1e-9)
+            // ones whose balls overlap B_i now (float64, with a relative slack of 1e-9; in float where
+            // the distance is further from R_i + R_j than its rounding: an FP64 instruction costs 64
+            // cycles however few lanes need it)
+            const float4 fc = A.f4[i];
             const int nl = A.nbn[li];
             for (int b0 = 0; b0 < nl; b0 += 32) {
                 const int k = b0 + lane;
@@ -1091,10 +1094,16 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(const _
                 int j = -1;
                 if (k < nl) {
                     j = DS_IDX(A.nbl[li * NBL_CAP + k] + lofs, A.n, A.status);
-                    const AtomD q = load_atom(A.ad + j);
-                    const double dx = q.x - c.pi[0], dy = q.y - c.pi[1], dz = q.z - c.pi[2];
-                    const double rr = c.Ri + q.R;
-                    ok = dx * dx + dy * dy + dz * dz < rr * rr * (1.0 + 1e-9);
+                    const float4 f = A.f4[j];
+                    const float fx = f.x - fc.x, fy = f.y - fc.y, fz = f.z - fc.z, fr = f.w + fc.w;
+                    const float d2 = fx * fx + fy * fy + fz * fz;
+                    ok = d2 < (fr - G.fuzz) * (fr - G.fuzz);
+                    if (!ok && !(d2 > (fr + G.fuzz) * (fr + G.fuzz))) {
+                        const AtomD q = load_atom(A.ad + j);
+                        const double dx = q.x - c.pi[0], dy = q.y - c.pi[1], dz = q.z - c.pi[2];
+                        const double rr = c.Ri + q.R;
+                        ok = dx * dx + dy * dy + dz * dz < rr * rr * (1.0 + 1e-9);
+                    }
                 }
                 unsigned bal = __ballot_sync(FULL, ok);
                 int pos = nc + __popc(bal & lanemask_lt());

@@ -233,7 +233,7 @@ dsasa_status run(dsasa_ctx* c, const double* coords, const double* radii, double
     if (lists) {
         const int valid = c->lists_n == n && c->lists_probe == probe;
         cudaError_t ev_e = launch_verlet_check(coords, radii, c->ref_xyz, c->ref_rad, (int)n, valid, c->cfg.skin,
-                                               c->vstate, c->ad, c->stream);
+                                               c->vstate, c->ad, c->f4, c->stream);
         if (ev_e != cudaSuccess) return cuda_fail(c, ev_e, "Verlet check launch");
     }
     // the build also clears the deferred-atom count of the atom kernels that follow it
@@ -248,6 +248,7 @@ dsasa_status run(dsasa_ctx* c, const double* coords, const double* radii, double
     a.Rhl = c->Rhl;
     a.ad = c->ad;
     a.gh = c->gh;
+    a.f4 = c->f4;
     a.sf4 = c->sf4;
     a.sidx = c->sidx;
     a.molid = c->molid;

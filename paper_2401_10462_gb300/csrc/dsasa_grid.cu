@@ -74,7 +74,7 @@ __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
     if (nm <= 0) {
         for (int k = 0; k < 3; ++k) { g.lo[k] = 0.f; g.dims[k] = 0; }
         g.inv_cell = 1.f;
-        g.margin = 0.f;
+        g.margin = g.fuzz = 0.f;
         g.rmax = 0.f;
         g.base = 0;
         return g;
@@ -102,6 +102,7 @@ __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
     }
     for (int k = 0; k < 3; ++k) { g.lo[k] = lo[k]; g.dims[k] = dims[k]; }
     g.inv_cell = 1.0f / cell;
+    g.fuzz = margin;
     g.margin = margin + (float)skin;   // candidates within R_i + R_j + skin (Verlet lists)
     g.rmax = rmax;
     g.base = (dims[0] + 1) * dims[1] * dims[2];
@@ -501,7 +502,7 @@ __device__ bool last_block(unsigned* ticket) {
 // to vstate[0..1] (zero between calls); the last block decides and clears them.
 __global__ void __launch_bounds__(CHECK_T) k_verlet_check(const double* xyz, const double* radii, const double* ref_xyz,
                                                           const double* ref_rad, int n, int valid, float lim2, int* vstate,
-                                                          AtomD* ad) {
+                                                          AtomD* ad, float4* f4) {
     grid_dep_trigger();
     const int i = blockIdx.x * CHECK_T + threadIdx.x;
     float d2 = 0.f;
@@ -511,6 +512,7 @@ __global__ void __launch_bounds__(CHECK_T) k_verlet_check(const double* xyz, con
         ad[i].x = x;
         ad[i].y = y;
         ad[i].z = z;
+        f4[i] = make_float4((float)x, (float)y, (float)z, f4[i].w);
         double dx = x - ref_xyz[3 * i], dy = y - ref_xyz[3 * i + 1], dz = z - ref_xyz[3 * i + 2];
         double dd = dx * dx + dy * dy + dz * dz;
         d2 = (float)dd * (1.f + 1e-6f);   // rounded up: the test stays conservative
@@ -594,11 +596,12 @@ cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, co
 }
 
 cudaError_t launch_verlet_check(const double* xyz, const double* radii, const double* ref_xyz, const double* ref_rad,
-                                int n, int valid, double skin, int* vstate, AtomD* ad, cudaStream_t s) {
+                                int n, int valid, double skin, int* vstate, AtomD* ad, float4* f4,
+                                cudaStream_t s) {
     // (skin / 2)^2, rounded down in float
     const float lim2 = (float)(0.25 * skin * skin) * (1.f - 1e-6f);
     const int nb = valid && n > 0 ? (n + CHECK_T - 1) / CHECK_T : 1;
-    k_verlet_check<<<nb, CHECK_T, 0, s>>>(xyz, radii, ref_xyz, ref_rad, n, valid, lim2, vstate, ad);
+    k_verlet_check<<<nb, CHECK_T, 0, s>>>(xyz, radii, ref_xyz, ref_rad, n, valid, lim2, vstate, ad, f4);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -93,7 +93,8 @@ struct MolGrid {
     int base;         // first global cell of this molecule
     float margin;     // conservative slack of the FP32 neighbour test (A)
     float rmax;       // largest probe-inflated radius of the molecule
-    int pad[2];
+    float fuzz;       // margin without the skin: bound of the FP32 error of a distance minus a sum of radii
+    int pad;
 };
 // the first cell of row (z, y): a row holds dims[0] cells and one more entry for its end
 __host__ __device__ inline int grid_row(const MolGrid& g, int z, int y) {
@@ -139,6 +140,7 @@ struct AtomArgs {
     const float2* Rhl;      // R as (hi, lo) floats
     const AtomD* ad;        // position and R (of this call's coordinates, also when the lists are reused)
     const float* gh;        // half-width of the initial cell
+    const float4* f4;       // (x, y, z, R) in float, by atom (current, like ad)
     const float4* sf4;
     const int* sidx;
     const int* molid;
@@ -226,11 +228,12 @@ struct SRArgs {
 
 cudaError_t launch_build(const BuildArgs& a, cudaStream_t s);
 // Verlet skin test: vstate[2] = reuse the lists (valid, every atom within skin/2 of its
-// reference position, radii unchanged, no list overflow); the positions go to ad, which a build
-// that is not needed does not write; vstate[3] overflow, the other words
+// reference position, radii unchanged, no list overflow); the positions go to ad and f4, which a
+// build that is not needed does not write; vstate[3] overflow, the other words
 // scratch (zero between calls; 8 words)
 cudaError_t launch_verlet_check(const double* xyz, const double* radii, const double* ref_xyz, const double* ref_rad,
-                                int n, int valid, double skin, int* vstate, AtomD* ad, cudaStream_t s);
+                                int n, int valid, double skin, int* vstate, AtomD* ad, float4* f4,
+                                cudaStream_t s);
 // the Verlet skin test of a batch of resident molecules: reuse[m] for each molecule (see
 // k_verlet_check_batch); vmol: 3 ints per molecule of scratch, ticket: one more, zero between calls
 cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, const double* ref_xyz,

@@ -108,6 +108,7 @@ extern "C" dsasa_status dsasa_compute_noalloc(const double* coords, const double
     a.Rhl = b.Rhl;
     a.ad = b.ad;
     a.gh = b.gh;
+    a.f4 = b.f4;
     a.sf4 = b.sf4;
     a.sidx = b.sidx;
     a.molid = b.molid;
