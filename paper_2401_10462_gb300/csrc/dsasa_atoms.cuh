@@ -1117,9 +1117,6 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(const _
             const bool store_lists = slot;
             int nl = 0;
             {
-                int cx = min(max((int)floorf((fi.x - G.lo[0]) * G.inv_cell), 0), G.dims[0] - 1);
-                int cy = min(max((int)floorf((fi.y - G.lo[1]) * G.inv_cell), 0), G.dims[1] - 1);
-                int cz = min(max((int)floorf((fi.z - G.lo[2]) * G.inv_cell), 0), G.dims[2] - 1);
                 // one candidate per lane: the FP32 overlap test with the grid's certified slack,
                 // the Verlet-list entry and the float64 test, the append to the plane table
                 auto gather_one = [&](bool valid, float4 fj, int j) {
@@ -1148,76 +1145,25 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(const _
                     if (ok && pos < KMAX) S->pg[NG + pos] = j;
                     nc += __popc(bal);
                 };
-                // sorted positions [beg, end): the atoms that may overlap B_i
-                auto gather_range = [&](int beg, int end) {
-                    for (int b0 = beg; b0 < end; b0 += 32) {
-                        const int k = b0 + lane;
-                        float4 fj = make_float4(0.f, 0.f, 0.f, 0.f);
-                        int j = -1;
-                        if (k < end) { fj = A.sf4[k]; j = DS_IDX(A.sidx[k], A.n, A.status); }
-                        gather_one(k < end, fj, j);
-                    }
+                // 32 atoms at a time, the next ones on their way
+                NearRows near(G, A.cstart, fi, (int*)S->skey);
+                auto fetch = [&](int f0, float4& f, int& j) {
+                    const int k = near.at(f0);
+                    f = make_float4(0.f, 0.f, 0.f, 0.f);
+                    j = -1;
+                    if (f0 + lane < near.total) { f = A.sf4[k]; j = DS_IDX(A.sidx[k], A.n, A.status); }
                 };
-                if constexpr (PH == PH_CELL) {
-                    // the 9 rows (dz, dy) of 3 cells along x: lane r < 9 looks up row r's range (the
-                    // 18 lookups in one memory round trip); the first 32 atoms of the 3 rows of one
-                    // dz are loaded together (one round trip for the three), longer rows finish by
-                    // rounds.  Measured faster in the split cell kernel (50k globule: 569 -> 548 us)
-                    // and slower in the one-wave kernel, which keeps the row loop
-                    int rbeg = 0, rend = 0;
-                    if (lane < 9) {
-                        const int z = cz + lane / 3 - 1, y = cy + lane % 3 - 1;
-                        if (z >= 0 && z < G.dims[2] && y >= 0 && y < G.dims[1]) {
-                            const int row = grid_row(G, z, y);
-                            const int x0 = max(cx - 1, 0), x1 = min(cx + 1, G.dims[0] - 1);
-                            rbeg = A.cstart[row + x0];
-                            rend = A.cstart[row + x1 + 1];
-                        }
-                    }
+                float4 fj = make_float4(0.f, 0.f, 0.f, 0.f), fn = fj;
+                int j = -1, jn = -1;
+                if (near.total > 0) fetch(0, fj, j);
 #pragma unroll 1
-                    for (int r0 = 0; r0 < 9; r0 += 3) {
-                        float4 rf[3];
-                        int rj[3];
-#pragma unroll
-                        for (int u = 0; u < 3; ++u) {
-                            const int k = __shfl_sync(FULL, rbeg, r0 + u) + lane;
-                            rf[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                            rj[u] = -1;
-                            if (k < __shfl_sync(FULL, rend, r0 + u)) {
-                                rf[u] = A.sf4[k];
-                                rj[u] = DS_IDX(A.sidx[k], A.n, A.status);
-                            }
-                        }
-#pragma unroll 1
-                        for (int u = 0; u < 3; ++u) {
-                            const int e = __shfl_sync(FULL, rend, r0 + u);
-                            int b0 = __shfl_sync(FULL, rbeg, r0 + u);
-                            float4 fj = u == 0 ? rf[0] : (u == 1 ? rf[1] : rf[2]);
-                            int j = u == 0 ? rj[0] : (u == 1 ? rj[1] : rj[2]);
-                            for (;;) {
-                                gather_one(b0 + lane < e, fj, j);
-                                b0 += 32;
-                                if (b0 >= e) break;
-                                const int k = b0 + lane;
-                                fj = make_float4(0.f, 0.f, 0.f, 0.f);
-                                j = -1;
-                                if (k < e) { fj = A.sf4[k]; j = DS_IDX(A.sidx[k], A.n, A.status); }
-                            }
-                        }
-                    }
-                } else {
-                    for (int dz = -1; dz <= 1; ++dz) {
-                        int z = cz + dz;
-                        if (z < 0 || z >= G.dims[2]) continue;
-                        for (int dy = -1; dy <= 1; ++dy) {
-                            int y = cy + dy;
-                            if (y < 0 || y >= G.dims[1]) continue;
-                            int row = grid_row(G, z, y);
-                            int x0 = max(cx - 1, 0), x1 = min(cx + 1, G.dims[0] - 1);
-                            gather_range(A.cstart[row + x0], A.cstart[row + x1 + 1]);
-                        }
-                    }
+                for (int f0 = 0; f0 < near.total; f0 += 32) {
+                    if (f0 + 32 < near.total) fetch(f0 + 32, fn, jn);
+                    gather_one(f0 + lane < near.total, fj, j);
+                    fj = fn;
+                    j = jn;
                 }
+                __syncwarp();
             }
             if (store_lists && lane == 0) {
                 // the list's length and the reference position for the next calls; a list

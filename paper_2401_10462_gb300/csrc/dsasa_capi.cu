@@ -58,7 +58,8 @@ struct dsasa_ctx {
     // capacities
     int64_t cap_atoms = 0;
     int64_t cap_mol = 0;
-    int64_t cap_cells = 0;
+    int64_t cap_cells = 0;     // cubic cells (max_cells, if set)
+    int64_t store_cells = 0;   // what the cell arrays hold
     // scratch
     double* R = nullptr;
     float2* Rhl = nullptr;
@@ -141,7 +142,7 @@ void free_scratch(dsasa_ctx* c) {
     dfree(c->defer); dfree(c->redo); dfree(c->cells); dfree(c->mol_base); dfree(c->mol_reuse); dfree(c->vmol); dfree(c->mol_done);
     dfree(c->nbl); dfree(c->nbn); dfree(c->ref_xyz); dfree(c->ref_rad); dfree(c->vstate);
     c->lists_n = 0;
-    c->cap_atoms = c->cap_mol = c->cap_cells = 0;
+    c->cap_atoms = c->cap_mol = c->cap_cells = c->store_cells = 0;
 }
 void free_host_staging(dsasa_ctx* c) {
     dfree(c->h_xyz); dfree(c->h_rad); dfree(c->h_w); dfree(c->h_area); dfree(c->h_grad);
@@ -166,17 +167,18 @@ dsasa_status ensure(dsasa_ctx* c, int64_t n, int64_t n_mol) {
     if (c->cfg.max_atoms > 0) { na = std::max<int64_t>(n, c->cfg.max_atoms); nm = std::max<int64_t>(nm, 4096); }
     int64_t nc = cells_for(na, nm);
     if (c->cfg.max_cells > 0 && c->cfg.max_cells < nc) nc = std::max<int64_t>(c->cfg.max_cells, 64);
+    const int64_t ns = std::min(cells_for(na, nm), cell_store(nc));   // (without a limit: every molecule's own bound)
 #define ALLOC(ptr, count)                                                               \
     e = dev_alloc((void**)&c->ptr, sizeof(*c->ptr) * (size_t)(count));                 \
     if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "cudaMalloc " #ptr); }
     ALLOC(R, na) ALLOC(Rhl, na) ALLOC(ad, na) ALLOC(gh, na) ALLOC(f4, na) ALLOC(molid, na) ALLOC(rank, na) ALLOC(cell, na) ALLOC(sidx, na) ALLOC(sf4, na)
-    ALLOC(bbox, 8 * nm) ALLOC(grids, nm) ALLOC(counts, nc + 1) ALLOC(cstart, nc + 1) ALLOC(blocksums, (int64_t)scan_scratch_ints((int)nc) + 16)
+    ALLOC(bbox, 8 * nm) ALLOC(grids, nm) ALLOC(counts, ns + 1) ALLOC(cstart, ns + 1) ALLOC(blocksums, (int64_t)scan_scratch_ints((int)ns) + 16)
     ALLOC(offsets, nm + 1) ALLOC(defer, na) ALLOC(redo, na) ALLOC(cells, na * (int64_t)cell_record_bytes()) ALLOC(bsync, BUILD_SYNC_WORDS)
     ALLOC(mol_base, nm) ALLOC(mol_reuse, nm) ALLOC(vmol, 3 * nm + 1) ALLOC(mol_done, nm)
     // what the kernels expect to be zero, and leave zero
     e = cudaMemsetAsync(c->bsync, 0, sizeof(unsigned) * BUILD_SYNC_WORDS, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->bbox, 0, sizeof(unsigned) * 8 * (size_t)nm, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->counts, 0, sizeof(int) * (size_t)(nc + 1), c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(c->counts, 0, sizeof(int) * (size_t)(ns + 1), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->vmol, 0, sizeof(int) * (3 * (size_t)nm + 1), c->stream);
     if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "memset"); }
     if (c->cfg.skin > 0.0) {
@@ -190,6 +192,7 @@ dsasa_status ensure(dsasa_ctx* c, int64_t n, int64_t n_mol) {
     c->cap_atoms = na;
     c->cap_mol = nm;
     c->cap_cells = nc;
+    c->store_cells = ns;
     return DSASA_OK;
 }
 
@@ -206,7 +209,8 @@ cudaError_t build_cells(dsasa_ctx* c, const double* coords, const double* radii,
     b.n_mol = n_mol;
     b.offsets = offsets_dev;
     b.skin = c->cfg.skin;
-    b.max_cells = (int)c->cap_cells;
+    b.max_cells = (int)c->store_cells;
+    b.cube_limit = c->cap_cells < cells_for(c->cap_atoms, c->cap_mol) ? (int)c->cap_cells : 0;
     b.R = c->R; b.Rhl = c->Rhl; b.ad = c->ad; b.gh = c->gh; b.f4 = c->f4; b.molid = c->molid; b.rank = c->rank; b.cell = c->cell;
     b.bbox = c->bbox; b.grids = c->grids; b.counts = c->counts; b.cstart = c->cstart; b.sidx = c->sidx;
     b.sf4 = c->sf4; b.blocksums = c->blocksums; b.sync = c->bsync; b.zero_word = zero_word; b.status = c->status; b.ncells_out = c->status + 1;

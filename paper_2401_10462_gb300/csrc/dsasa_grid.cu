@@ -1,11 +1,11 @@
 // Cell-list build for the neighbour search (input preparation and binning).
 //
-// Atoms are binned per molecule into cubic cells of edge >= 2 R_max + skin + slack, so every
-// pair of overlapping balls |p_i - p_j| < R_i + R_j lies in the same or adjacent cells.  The
-// binning is a counting sort in four kernels that start early behind one another (programmatic
+// Atoms are binned per molecule into cells of edge >= 2 R_max + skin + slack along y and z and a
+// quarter of that along x, so that every pair of overlapping balls |p_i - p_j| < R_i + R_j lies in
+// the same or adjacent rows of cells.  The binning is a counting sort in four kernels that start early behind one another (programmatic
 // dependent launch): input pass, bounding boxes and grids (the last block makes the grids, so
-// nothing waits); counts; starts; scatter.  The neighbour search reads runs of up to three cells
-// that are adjacent along x, so only the cells of one row (fixed y, z) need consecutive starts:
+// nothing waits); counts; starts; scatter.  The neighbour search reads runs of cells that are
+// adjacent along x, so only the cells of one row (fixed y, z) need consecutive starts:
 // a row takes its place in the sorted order with one atomic add and needs no scan over all
 // cells.  (A batch is built in nine kernels, with its grids and a scan over all cells in
 // kernels of their own.)  The order of rows and of the atoms inside a cell is not deterministic, which is
@@ -69,14 +69,14 @@ __device__ __forceinline__ int molecule_of(const long long* offsets, int n_mol, 
 
 // Grid of one molecule from its box (box_words) and atom count: cell size and dimensions; the
 // cell count is returned in base, with one more entry per row of cells for the row's end.
-__device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
+__device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin, int cube_limit) {
     MolGrid g;
     if (nm <= 0) {
         for (int k = 0; k < 3; ++k) { g.lo[k] = 0.f; g.dims[k] = 0; }
         g.inv_cell = 1.f;
         g.margin = g.fuzz = 0.f;
         g.rmax = 0.f;
-        g.base = 0;
+        g.base = g.cubes = 0;
         return g;
     }
     float lo[3], hi[3], amax = 0.f;
@@ -91,15 +91,26 @@ __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
     float cell = 2.0f * rmax + (float)skin + 2.0f * margin + 1e-3f;
     double cap = 8.0 * (double)nm + 64.0;
     int dims[3];
-    for (int it = 0; it < 64; ++it) {
+    const auto fit = [&](float& edge, float xf, int ends) {   // the edge grows until the cells fit `cap`
         double prod = 1.0;
-        for (int k = 0; k < 3; ++k) {
-            dims[k] = (int)fminf((hi[k] - lo[k]) / cell, 1e6f) + 1;
-            prod *= dims[k] + (k == 0);
+        for (int it = 0; it < 64; ++it) {
+            prod = 1.0;
+            for (int k = 0; k < 3; ++k) {
+                dims[k] = (int)fminf((hi[k] - lo[k]) / edge * (k == 0 ? xf : 1.f), 1e6f) + 1;
+                prod *= dims[k] + (k == 0 ? ends : 0);
+            }
+            if (prod <= cap) break;
+            edge *= (float)fmax(1.01, cbrt(prod / cap) * 1.01);
         }
-        if (prod <= cap) break;
-        cell *= (float)fmax(1.01, cbrt(prod / cap) * 1.01);
+        return prod;
+    };
+    g.cubes = 0;
+    if (cube_limit > 0) {   // (only where the caller set a limit of his own)
+        float edge = cell;
+        g.cubes = (int)fit(edge, 1.f, 0);
+        cap = fmin(cap, (double)cell_store(g.cubes));
     }
+    fit(cell, (float)GRID_XF, 1);
     for (int k = 0; k < 3; ++k) { g.lo[k] = lo[k]; g.dims[k] = dims[k]; }
     g.inv_cell = 1.0f / cell;
     g.fuzz = margin;
@@ -110,11 +121,14 @@ __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin) {
 }
 
 __device__ __forceinline__ int cell_of(const MolGrid& g, float4 f) {
-    int cx = min(max((int)floorf((f.x - g.lo[0]) * g.inv_cell), 0), g.dims[0] - 1);
+    int cx = min(max((int)floorf((f.x - g.lo[0]) * (g.inv_cell * GRID_XF)), 0), g.dims[0] - 1);
     int cy = min(max((int)floorf((f.y - g.lo[1]) * g.inv_cell), 0), g.dims[1] - 1);
     int cz = min(max((int)floorf((f.z - g.lo[2]) * g.inv_cell), 0), g.dims[2] - 1);
     return grid_row(g, cz, cy) + cx;
 }
+
+// a user's limit is exceeded by so many cubic cells
+__device__ __forceinline__ bool refused(const BuildArgs& a, int cubes) { return a.cube_limit > 0 && cubes > a.cube_limit; }
 
 constexpr int PREP_T = 256;
 
@@ -186,8 +200,8 @@ __global__ void __launch_bounds__(PREP_T) k_prep(BuildArgs a) {
         bx[k] = __ldcg(a.bbox + k);
         a.bbox[k] = 0;
     }
-    MolGrid g = make_grid(bx, a.n, a.skin);
-    const int cells = g.base;
+    MolGrid g = make_grid(bx, a.n, a.skin, a.cube_limit);
+    const int cells = refused(a, g.cubes) ? a.max_cells + 1 : g.base;
     g.base = 0;
     a.sync[BUILD_ROWS] = (unsigned)(g.dims[1] * g.dims[2]);
     a.sync[BUILD_CURSOR] = 0u;
@@ -215,7 +229,7 @@ __global__ void k_grid_local(BuildArgs a) {
     grid_dep_wait();
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= a.n_mol) return;
-    a.grids[m] = make_grid(a.bbox + 8 * m, a.offsets[m + 1] - a.offsets[m], a.skin);
+    a.grids[m] = make_grid(a.bbox + 8 * m, a.offsets[m + 1] - a.offsets[m], a.skin, a.cube_limit);
     for (int k = 0; k < 8; ++k) a.bbox[8 * m + k] = 0;
 }
 
@@ -223,9 +237,14 @@ __global__ void k_grid_local(BuildArgs a) {
 __global__ void __launch_bounds__(PREP_T) k_grid_scan(BuildArgs a) {
     grid_dep_trigger();
     grid_dep_wait();
-    int cells = 0;
+    int cells = 0, cubes = 0;
     for (int m0 = 0; m0 < a.n_mol; m0 += PREP_T) {
         const int m = m0 + threadIdx.x;
+        if (a.cube_limit > 0) {
+            int e, tot;
+            block_excl_scan(m < a.n_mol ? a.grids[m].cubes : 0, e, tot);
+            cubes += tot;
+        }
         const int v = m < a.n_mol ? a.grids[m].base : 0;
         int e, tot;
         block_excl_scan(v, e, tot);
@@ -238,6 +257,7 @@ __global__ void __launch_bounds__(PREP_T) k_grid_scan(BuildArgs a) {
         cells += tot;
     }
     if (threadIdx.x == 0) {
+        if (refused(a, cubes)) cells = a.max_cells + 1;
         *a.ncells_out = cells;
         if (cells > a.max_cells) atomicOr(a.status, ST_GRID_OVF);
     }
@@ -381,8 +401,8 @@ __global__ void __launch_bounds__(kSmallT) k_build_small(BuildArgs a) {
     }
     __syncthreads();
     if (tid == 0) {
-        MolGrid gg = make_grid(bb, a.n, a.skin);
-        const int ncells = gg.base;
+        MolGrid gg = make_grid(bb, a.n, a.skin, a.cube_limit);
+        const int ncells = refused(a, gg.cubes) ? a.max_cells + 1 : gg.base;
         gg.base = 0;
         if (ncells > a.max_cells) {   // an empty grid keeps every index in range
             for (int k = 0; k < 3; ++k) gg.dims[k] = 0;

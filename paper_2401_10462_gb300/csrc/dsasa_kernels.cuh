@@ -85,21 +85,85 @@ __device__ __forceinline__ AtomD load_atom(const AtomD* p) {
 }
 #endif
 
-// cell grid of one molecule: cells of edge `cell` starting at `lo`, cell id = base + local
+// cell grid of one molecule, starting at `lo`: along y and z cells reach as far as any overlap (and
+// the skin), so an atom's neighbours lie in its own row of cells and the eight around it; along x
+// they are GRID_XF times shorter, so that a row's run can be cut close to the atom's reach
+constexpr int GRID_XF = 4;
 struct MolGrid {
     float lo[3];
-    float inv_cell;
+    float inv_cell;   // 1 / edge along y and z (GRID_XF times that along x)
     int dims[3];
     int base;         // first global cell of this molecule
     float margin;     // conservative slack of the FP32 neighbour test (A)
     float rmax;       // largest probe-inflated radius of the molecule
     float fuzz;       // margin without the skin: bound of the FP32 error of a distance minus a sum of radii
-    int pad;
+    int cubes;        // cubic cells of the same edge in its box: what a user's max_cells bounds
 };
 // the first cell of row (z, y): a row holds dims[0] cells and one more entry for its end
 __host__ __device__ inline int grid_row(const MolGrid& g, int z, int y) {
     return g.base + (z * g.dims[1] + y) * (g.dims[0] + 1);
 }
+
+#ifdef __CUDACC__
+// The atoms that may lie within f.w + rmax + margin of atom f = (x, y, z, R) of the grid, as one index
+// space 0 .. total - 1 over the runs of the nine rows of cells around it; called by a whole warp (buf:
+// 32 ints of its shared memory).  Nine lanes look the runs up in one memory round trip, each cut to
+// what the sphere can reach in its row: about 120 atoms of a globule in 4 full rounds of 32.  (Whole
+// cells of the reach along x gave 200, row by row at 23 of 32 lanes, and three times the
+// instructions; cells of half the reach in 25 rows gave 80, but their runs of four atoms spread
+// every load over eight lines and more: slower than the nine whole rows.)
+struct NearRows {
+    int off, len, total, rows;
+    int* buf;
+    unsigned le;
+    __device__ __forceinline__ NearRows(const MolGrid& G, const int* cstart, float4 f, int* b) : off(0), len(0), rows(0), buf(b) {
+        const int lane = threadIdx.x & 31;
+        const unsigned full = 0xffffffffu;
+        int beg = 0;
+        if (lane < 9) {
+            const int z = min(max((int)floorf((f.z - G.lo[2]) * G.inv_cell), 0), G.dims[2] - 1) + lane / 3 - 1;
+            const int y = min(max((int)floorf((f.y - G.lo[1]) * G.inv_cell), 0), G.dims[1] - 1) + lane % 3 - 1;
+            if (z >= 0 && z < G.dims[2] && y >= 0 && y < G.dims[1]) {
+                const float slack = 1e-3f + 2.f * G.fuzz;   // rounding of an atom's place in the grid
+                const float cell = __frcp_rn(G.inv_cell), r = f.w + G.rmax + G.margin + slack;
+                const float y0 = G.lo[1] + y * cell, z0 = G.lo[2] + z * cell;
+                const float dy = fmaxf(fmaxf(y0 - f.y, f.y - (y0 + cell)) - slack, 0.f);
+                const float dz = fmaxf(fmaxf(z0 - f.z, f.z - (z0 + cell)) - slack, 0.f);
+                const float w2 = r * r - (dy * dy + dz * dz);
+                if (w2 > 0.f) {
+                    const float w = w2 * rsqrtf(w2) * 1.00001f + slack, ix = G.inv_cell * GRID_XF, x = f.x - G.lo[0];
+                    const int x0 = max((int)floorf((x - w) * ix), 0), x1 = min((int)floorf((x + w) * ix), G.dims[0] - 1);
+                    if (x0 <= x1) {
+                        const int row = grid_row(G, z, y);
+                        beg = cstart[row + x0];
+                        len = cstart[row + x1 + 1] - beg;
+                    }
+                }
+            }
+        }
+        const unsigned ne = __ballot_sync(full, len > 0);
+        off = len;
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) {
+            const int p = __shfl_up_sync(full, off, o);
+            if (lane >= o) off += p;
+        }
+        total = __shfl_sync(full, off, 8);
+        off -= len;
+        asm("mov.u32 %0, %%lanemask_le;" : "=r"(le));
+        if (len > 0) buf[__popc(ne & (le >> 1))] = beg - off;
+        __syncwarp();
+    }
+    // the lane's sorted position of indices f0 .. f0 + 31 (f0 = 0, 32, ... in turn; past total: any)
+    __device__ __forceinline__ int at(int f0) {
+        const int p = off - f0;
+        const unsigned m = __reduce_or_sync(0xffffffffu, len > 0 && (unsigned)p < 32u ? 1u << p : 0u);
+        const int r = rows + __popc(m & le) - 1;
+        rows += __popc(m);
+        return buf[r] + f0 + (int)(threadIdx.x & 31);
+    }
+};
+#endif
 
 struct BuildArgs {
     const double* xyz;
@@ -112,7 +176,8 @@ struct BuildArgs {
     const int* skip;   // non-NULL and *skip != 0: the previous cell list is reused (nothing to do)
     int* zero_word;    // non-NULL: zero_word[0..1] set to 0 by the build's first kernel (the next atom
                        // kernels' deferred count, and a spare word)
-    int max_cells;
+    int max_cells;     // cells (and row ends) that counts and cstart hold
+    int cube_limit;    // > 0: more cubic cells than this are refused (cell_store makes room for what they become)
     // outputs / scratch
     double* R;         // n
     float2* Rhl;       // n: R as a float pair (hi, lo), for the float-float area terms
@@ -246,6 +311,8 @@ cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s);
 cudaError_t launch_atoms_f32(const AtomArgs& a, bool grad, cudaStream_t s);
 cudaError_t launch_atoms_f64(const AtomArgs& a, bool grad, cudaStream_t s);
 size_t scan_scratch_ints(int max_cells);
+// entries that `cubes` cubic cells can become: a quarter as long along x, and an end for each row
+__host__ __device__ inline int64_t cell_store(int64_t cubes) { return (GRID_XF + 1) * cubes; }
 size_t cell_record_bytes();
 
 }  // namespace dsasa

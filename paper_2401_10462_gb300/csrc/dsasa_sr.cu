@@ -10,9 +10,9 @@
 // exact float64 test |p_i - p_j|^2 < (R_i + R_j)^2.
 //
 // One warp per atom.  Bound: instruction issue.
-//   * The candidates of the 27 cells that pass the float test are packed before the float64
-//     test, whose instructions cost 64 cycles each however few lanes are active (9 rows of
-//     cells took 9 of them before, 1 or 2 do now).
+//   * The candidates that pass the float test are packed before the float64 test, whose
+//     instructions cost 64 cycles each however few lanes are active (9 rows of cells took 9 of
+//     them before, 1 or 2 do now).
 //   * d2 <= R_j^2 is x.q - (|q|^2 - R_j^2) / 2 >= |x|^2 / 2: three multiply-adds and a maximum
 //     per pair instead of nine operations.  Only a point whose largest value comes within the
 //     rounding bound of |x|^2 / 2 is decided by the operations above.
@@ -96,48 +96,32 @@ __global__ void __launch_bounds__(SR_WARPS * 32) k_shrake_rupley(SRArgs A) {
         }
         nn += __popc(bal);
     };
-    {
-        const int cx = min(max((int)floorf((fi.x - G.lo[0]) * G.inv_cell), 0), G.dims[0] - 1);
-        const int cy = min(max((int)floorf((fi.y - G.lo[1]) * G.inv_cell), 0), G.dims[1] - 1);
-        const int cz = min(max((int)floorf((fi.z - G.lo[2]) * G.inv_cell), 0), G.dims[2] - 1);
-        int rbeg = 0, rend = 0;   // lane r < 9: the run of atoms in row r of three cells
-        if (lane < 9) {
-            const int z = cz + lane / 3 - 1, y = cy + lane % 3 - 1;
-            if (z >= 0 && z < G.dims[2] && y >= 0 && y < G.dims[1]) {
-                const int row = grid_row(G, z, y);
-                rbeg = A.cstart[row + max(cx - 1, 0)];
-                rend = A.cstart[row + min(cx + 1, G.dims[0] - 1) + 1];
-            }
+    NearRows near(G, A.cstart, fi, (int*)S->key);
+    for (int f0 = 0; f0 < near.total; f0 += 32) {
+        const int k = near.at(f0);
+        bool ok = false;
+        int j = -1;
+        if (f0 + lane < near.total) {
+            const float4 fj = A.sf4[k];
+            j = A.sidx[k];
+            const float dx = fj.x - fi.x, dy = fj.y - fi.y, dz = fj.z - fi.z;
+            const float rr = fi.w + fj.w + G.margin;
+            ok = j != i && dx * dx + dy * dy + dz * dz < rr * rr;
         }
-        for (int r = 0; r < 9; ++r) {
-            const int end = __shfl_sync(full, rend, r);
-            for (int b0 = __shfl_sync(full, rbeg, r); b0 < end; b0 += 32) {
-                const int k = b0 + lane;
-                bool ok = false;
-                int j = -1;
-                if (k < end) {
-                    const float4 fj = A.sf4[k];
-                    j = A.sidx[k];
-                    const float dx = fj.x - fi.x, dy = fj.y - fi.y, dz = fj.z - fi.z;
-                    const float rr = fi.w + fj.w + G.margin;
-                    ok = j != i && dx * dx + dy * dy + dz * dz < rr * rr;
-                }
-                const unsigned bal = __ballot_sync(full, ok);
-                if (ok) S->cand[nc + __popc(bal & lt)] = j;
-                nc += __popc(bal);
-                if (nc >= 32) {
-                    __syncwarp();
-                    exact(32);
-                    const int rest = lane < nc - 32 ? S->cand[32 + lane] : 0;
-                    __syncwarp();
-                    if (lane < nc - 32) S->cand[lane] = rest;
-                    nc -= 32;
-                }
-            }
+        const unsigned bal = __ballot_sync(full, ok);
+        if (ok) S->cand[nc + __popc(bal & lt)] = j;
+        nc += __popc(bal);
+        if (nc >= 32) {
+            __syncwarp();
+            exact(32);
+            const int rest = lane < nc - 32 ? S->cand[32 + lane] : 0;
+            __syncwarp();
+            if (lane < nc - 32) S->cand[lane] = rest;
+            nc -= 32;
         }
-        __syncwarp();
-        if (nc > 0) exact(nc);
     }
+    __syncwarp();
+    if (nc > 0) exact(nc);
     __syncwarp();
     if (__any_sync(full, ovf) || nn > SR_KN) {
         if (lane == 0) {
