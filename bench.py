@@ -133,7 +133,7 @@ class ClockSampler:
 def kernel_sha() -> str:
     import hashlib
     h = hashlib.sha256()
-    for f in ("dsasa_atoms.cuh", "dsasa_math.cuh", "dsasa_kernels.cuh"):
+    for f in ("dsasa_atoms.cuh", "dsasa_class.cuh", "dsasa_terms.cuh", "dsasa_math.cuh", "dsasa_kernels.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2401_10462_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -242,8 +242,8 @@ def roofline_block(wm, n, ph, pk, dpk, counters):
                  "frac": ach / pk["issue_ginst_s"],
                  "source": "smsp__inst_executed.sum of one ncu launch (profiles/traffic.json) / live duration; "
                            "peak = warp instructions/s of the FP32 FMA microbenchmark"}
-    names = {"cell": "k_atoms<float,0,64,64,PH_CC or PH_CELL> (restricted power cell; with all atoms in one wave "
-                     "also the classification)", "terms": "k_atoms<float,1,64,64,PH_TERMS>"}
+    names = {"cell": "k_atoms<float,0,64,64,PH_CC or PH_CELL> (restricted power cell; PH_CC, up to 20 atoms an SM: "
+                     "also the classification)", "terms": "k_terms<float,1>"}
     out = {"bound": "alu", "kernel": names.get(dom, dom), "achieved": achieved, "peak": pk["fp32_tflops"],
            "unit": "TFLOP/s", "frac": achieved / pk["fp32_tflops"], "traffic": counters.get("bytes_per_launch"),
            "kernel_ms": dom_ms, "peak_source": "FP32 FMA roof measured in this run (of measured)",

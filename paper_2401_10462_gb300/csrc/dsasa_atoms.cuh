@@ -48,8 +48,9 @@ constexpr int WARPS = 1, WARPS_CELL = 2, WARPS_CLASS = 2, WARPS_TERMS = 2;
 // resident blocks per SM that each kernel's register budget is sized for (one warp each)
 // (whole calls, us: the cell kernel at 16 / 17 / 18 blocks, 5,000 atoms 130.0 / 135.4 / 135.6 - with 18
 // resident blocks the next kernel's find no room before the last one ends - and 20,000-atom MD
-// steps 1283 / 1307 / 1306; the fused kernel at 16 / 18, 304 atoms 84.6 / 79.3)
-constexpr int MINB = 32, MINB_CELL = 16, MINB_CC = 18, MINB_TERMS = 18;
+// steps 1283 / 1307 / 1306; the fused kernel serves 20 atoms an SM: 10 blocks leave it the registers
+// it wants - 304 atoms: its phase 51 -> 44 us)
+constexpr int MINB = 32, MINB_CELL = 16, MINB_CC = 10, MINB_TERMS = 18;
 
 // kernel phases: the whole computation in one kernel, or three kernels that pass the cell
 // through a global record per atom: the cell construction (gather, sort, clipping), the
@@ -953,6 +954,13 @@ __device__ __noinline__ int carry_cell(SM* S, const RC* rec, int i, int n, int n
 }
 
 // ------------------------------------------------------------------ the kernel
+// What bounds it: neither memory (0.6 KB an atom each way) nor arithmetic, but the chain of dependent
+// instructions of a cut and, with the SM full, instruction issue: about 5,100 warp instructions an
+// atom, half of them in 13 cuts and 28 tests.  A lone warp issues one in 7 cycles (2.2 fixed latency,
+// 1.7 global and local loads, 0.9 shared memory, 0.7 branches).  Hence the cell in registers, the
+// few FP64 instructions and the call-free loop below.  PH_CELL: 5,000 atoms 54 us (one wave: as long as
+// its slowest atoms, 100k cycles against 51k on average), 20k 146, 50k RNA 212, 1M shell 6.15 ms; with
+// the cell in shared memory and 27 whole cells in the gather 20k took 256 us and 1M 10.5 ms.
 __host__ __device__ constexpr int minb(int ph) {
     if (ph == PH_CC) return MINB_CC;
     return (ph == PH_CELL || ph == PH_CARRY) ? MINB_CELL : (ph == PH_VOL ? MINB_TERMS : MINB);
@@ -1291,13 +1299,19 @@ __global__ void __launch_bounds__(warps_of(PHX) * 32, minb(PHX)) k_atoms(const _
 #pragma unroll
             for (int r = 0; r < SPL; ++r)
                 if (r * 32 + lane < nc && S->bedge[rank[r]] != (unsigned)(r * 32 + lane)) tie = true;
-            if (__any_sync(FULL, tie)) {
+            if (__any_sync(FULL, tie)) {   // the lower atom first among equals (compared one by one from
+                                           // scratch this cost 15 - 30k cycles, a call's slowest atoms)
 #pragma unroll
                 for (int r = 0; r < SPL; ++r) {
-                    rank[r] = 0;
-                    if (r * 32 + lane < nc)
-                        for (int j = 0; j < nc; ++j)
-                            rank[r] += S->skey[j] < key[r] || (S->skey[j] == key[r] && S->pg[NG + j] < tg[r]);
+                    if (r * 32 >= nc) break;
+                    for (int j = 0; j < nc; j += 4) {
+                        const uint4 k = k4[j >> 2];
+                        unsigned eq = (k.x == key[r]) | (k.y == key[r]) << 1 | (k.z == key[r]) << 2 | (k.w == key[r]) << 3;
+                        for (; eq; eq &= eq - 1) {
+                            const int q = j + __ffs(eq) - 1;
+                            rank[r] += q < nc && S->pg[NG + q] < tg[r];
+                        }
+                    }
                 }
             }
         }
@@ -2062,9 +2076,10 @@ namespace dsasa {
 // (measured: 3 % faster on a 5k-atom molecule in the mixed form).
 struct AtomLaunch {
     cudaStream_t s;
+    int carveout;
     cudaError_t err = cudaSuccess;
     template <class K> void operator()(K kernel, int grid, int block, const AtomArgs& args) {
-        const cudaError_t e = launch_dependent(kernel, grid, block, s, true, args);
+        const cudaError_t e = launch_dependent_smem(kernel, grid, block, 0, s, true, carveout, args);
         if (err == cudaSuccess) err = e;
         note_launches(1);
     }
@@ -2090,7 +2105,7 @@ cudaError_t launch_atoms_t(const AtomArgs& a, bool grad, cudaStream_t s) {
     auto mark = [&](int k) {
         if (a.ev) cudaEventRecord(a.ev[k], s);
     };
-    AtomLaunch go{s};
+    AtomLaunch go{s, a.cells && cells_fused(a.n) ? CARVEOUT_SMALL : CARVEOUT_DEFAULT};
     if (a.cells) {
         const int grid = (a.n + WARPS_TERMS - 1) / WARPS_TERMS;
         const cudaError_t e = launch_cells(a, s);

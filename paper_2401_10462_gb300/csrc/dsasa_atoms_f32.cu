@@ -4,25 +4,23 @@
 #include "dsasa_atoms.cuh"
 
 namespace dsasa {
-namespace {
 
-// Whether the cell construction and the classification run as one kernel: up to 10 atoms a
-// multiprocessor (1,520 on a GB300).  There an atom's classification overlaps the slowest cells and
-// one launch and the trip of the records through memory are saved; with more atoms the split
-// kernels win, whose smaller instruction streams stay in the cache (fused / split, us per call with
-// the gradient: 304 atoms 76 / 81, 700 82 / 90, 1,200 133 / 138, 2,003 107 / 104, 3,000 132 / 119).
+// Whether the cell construction and the classification run as one kernel: up to 20 atoms a
+// multiprocessor (3,040 on a GB300), all resident at once.  There an atom's classification overlaps the
+// slowest cells and one launch and the trip of the records through memory are saved; with more atoms the
+// split kernels win, whose smaller instruction streams stay in the cache and which hold 32 warps (fused /
+// split, us per call with the gradient: 304 atoms 66 / 80, 700 66 / 88, 1,200 110 / 131, 2,003 87 / 101,
+// 3,000 96 / 116, 4,200 125 / 124).
 bool cells_fused(int n) {
     static int cap = -1;
     if (cap < 0) {
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cap = 10 * sms;
+        cap = 20 * sms;
     }
     return n <= cap;
 }
-
-}  // namespace
 
 // The cell records of every atom, classified (Steps 1 and 2).
 cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s) {
@@ -34,8 +32,9 @@ cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s) {
         if (a.ev) cudaEventRecord(a.ev[k], s);
     };
     auto nb = [&](int w) { return (a.n + w - 1) / w; };
-    AtomLaunch go{s};
-    if (!a.carry && cells_fused(a.n)) {
+    const bool small = cells_fused(a.n);
+    AtomLaunch go{s, small ? CARVEOUT_SMALL : CARVEOUT_DEFAULT};
+    if (!a.carry && small) {
         go(k_atoms<float, false, 64, 64, PH_CC>, nb(WARPS_CELL), WARPS_CELL * 32, fast);
         mark(0);
     } else {

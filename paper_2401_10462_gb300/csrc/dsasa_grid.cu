@@ -635,7 +635,7 @@ cudaError_t launch_build(const BuildArgs& a, cudaStream_t s) {
         // idempotent, and needed once per context: above 48 KB a kernel has to ask
         cudaError_t e = cudaFuncSetAttribute(k_build_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        e = launch_dependent_smem(k_build_small, 1, kSmallT, smem, s, early, a);
+        e = launch_dependent_smem(k_build_small, 1, kSmallT, smem, s, early, CARVEOUT_DEFAULT, a);
         note_launches(1);
         return e;
     }

@@ -17,24 +17,32 @@ namespace dsasa {
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 #endif
+// How much of an SM's memory is shared memory rather than L1 cache, in percent (default: as the runtime
+// decides for each kernel's occupancy).  A kernel cannot start beside one that runs with another split,
+// so early launches need the same split along the chain.  Molecules small enough for the fused cell
+// kernel leave most of an SM idle and gain from the overlap; larger ones need each kernel's own split
+// (one split for all, 20k energy + forces: 372 - 400 us against 365, RNA areas 440 - 486 against 424).
+constexpr int CARVEOUT_DEFAULT = -1, CARVEOUT_SMALL = 44;
 template <class... K, class... A>
 cudaError_t launch_dependent_smem(void (*kernel)(K...), int grid, int block, size_t smem, cudaStream_t s, bool early,
-                                  A&&... args) {
+                                  int carveout, A&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[1].val.sharedMemCarveout = (unsigned)carveout;
+    cfg.numAttrs = carveout < 0 ? 1 : 2;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 template <class... K, class... A>
 cudaError_t launch_dependent(void (*kernel)(K...), int grid, int block, cudaStream_t s, bool early, A&&... args) {
-    return launch_dependent_smem(kernel, grid, block, 0, s, early, std::forward<A>(args)...);
+    return launch_dependent_smem(kernel, grid, block, 0, s, early, CARVEOUT_DEFAULT, std::forward<A>(args)...);
 }
 
 // host: adds k to the library-wide count of kernel launches (dsasa_kernel_launches)
@@ -308,6 +316,7 @@ cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, co
 cudaError_t launch_sr(const SRArgs& a, cudaStream_t s);
 // the classified cell records of every atom (a.cells), for the terms of either precision
 cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s);
+bool cells_fused(int n);   // (dsasa_atoms_f32.cu)
 cudaError_t launch_atoms_f32(const AtomArgs& a, bool grad, cudaStream_t s);
 cudaError_t launch_atoms_f64(const AtomArgs& a, bool grad, cudaStream_t s);
 size_t scan_scratch_ints(int max_cells);

@@ -50,10 +50,10 @@ def _check(a, g, ra, rg):
 
 
 @pytest.mark.parametrize("axis", [0, 1, 2])
-@pytest.mark.parametrize("n,seed", [(2047, 1), (2049, 2), (5001, 3)])
+@pytest.mark.parametrize("n,seed", [(2047, 1), (2049, 2), (3040, 4), (3041, 5), (5001, 3)])
 def test_elongated_along_each_axis(api, torch_cuda, orc, gen, axis, n, seed):
     """A long molecule along x (long runs of cells), y and z (many rows), on both sides of the one-block
-    build's size, far from the origin."""
+    build's size and of the fused kernel's, far from the origin."""
     m = gen.rna(n, seed)
     x = np.roll(m.coords, axis - 2, axis=1) + np.array([300.0, -200.0, 100.0])
     a, g = _run(api, torch_cuda, x, m.radii)
