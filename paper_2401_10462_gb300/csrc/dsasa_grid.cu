@@ -68,7 +68,10 @@ __device__ __forceinline__ int molecule_of(const long long* offsets, int n_mol, 
 }
 
 // Grid of one molecule from its box (box_words) and atom count: cell size and dimensions; the
-// cell count is returned in base, with one more entry per row of cells for the row's end.
+// cell count is returned in base, with one more entry per row of cells for the row's end (-1: no
+// edge makes a grid of the box).  No axis may be cut off at its limit of cells: the neighbour search
+// relies on an atom lying within its cell.
+constexpr float AXIS_CELLS = 1e6f;
 __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin, int cube_limit) {
     MolGrid g;
     if (nm <= 0) {
@@ -91,32 +94,38 @@ __device__ MolGrid make_grid(const unsigned* bb, long long nm, double skin, int 
     float cell = 2.0f * rmax + (float)skin + 2.0f * margin + 1e-3f;
     double cap = 8.0 * (double)nm + 64.0;
     int dims[3];
-    const auto fit = [&](float& edge, float xf, int ends) {   // the edge grows until the cells fit `cap`
-        double prod = 1.0;
+    double prod = 1.0;
+    // the edge grows until the cells fit `cap` and every axis its limit (`axis` times AXIS_CELLS)
+    const auto fit = [&](float& edge, float xf, int ends, float axis) {
         for (int it = 0; it < 64; ++it) {
+            float longest = 0.f;
             prod = 1.0;
             for (int k = 0; k < 3; ++k) {
-                dims[k] = (int)fminf((hi[k] - lo[k]) / edge * (k == 0 ? xf : 1.f), 1e6f) + 1;
+                const float d = (hi[k] - lo[k]) / edge * (k == 0 ? xf : 1.f);
+                longest = fmaxf(longest, d);
+                dims[k] = (int)fminf(d, AXIS_CELLS) + 1;
                 prod *= dims[k] + (k == 0 ? ends : 0);
             }
-            if (prod <= cap) break;
-            edge *= (float)fmax(1.01, cbrt(prod / cap) * 1.01);
+            longest /= axis * AXIS_CELLS;
+            if (prod <= cap && longest <= 1.f) return true;
+            edge *= (float)fmax(1.01, fmax(cbrt(prod / cap), (double)longest) * 1.01);
         }
-        return prod;
+        return false;
     };
     g.cubes = 0;
     if (cube_limit > 0) {   // (only where the caller set a limit of his own)
         float edge = cell;
-        g.cubes = (int)fit(edge, 1.f, 0);
+        fit(edge, 1.f, 0, INFINITY);
+        g.cubes = (int)prod;
         cap = fmin(cap, (double)cell_store(g.cubes));
     }
-    fit(cell, (float)GRID_XF, 1);
+    const bool fits = fit(cell, (float)GRID_XF, 1, 1.f);
     for (int k = 0; k < 3; ++k) { g.lo[k] = lo[k]; g.dims[k] = dims[k]; }
     g.inv_cell = 1.0f / cell;
     g.fuzz = margin;
     g.margin = margin + (float)skin;   // candidates within R_i + R_j + skin (Verlet lists)
     g.rmax = rmax;
-    g.base = (dims[0] + 1) * dims[1] * dims[2];
+    g.base = fits ? (dims[0] + 1) * dims[1] * dims[2] : -1;
     return g;
 }
 
@@ -129,6 +138,10 @@ __device__ __forceinline__ int cell_of(const MolGrid& g, float4 f) {
 
 // a user's limit is exceeded by so many cubic cells
 __device__ __forceinline__ bool refused(const BuildArgs& a, int cubes) { return a.cube_limit > 0 && cubes > a.cube_limit; }
+// the cells of one molecule's grid from make_grid, or more than there may be
+__device__ __forceinline__ int cells_or_refused(const BuildArgs& a, const MolGrid& g) {
+    return refused(a, g.cubes) || g.base < 0 ? a.max_cells + 1 : g.base;
+}
 
 constexpr int PREP_T = 256;
 
@@ -201,7 +214,7 @@ __global__ void __launch_bounds__(PREP_T) k_prep(BuildArgs a) {
         a.bbox[k] = 0;
     }
     MolGrid g = make_grid(bx, a.n, a.skin, a.cube_limit);
-    const int cells = refused(a, g.cubes) ? a.max_cells + 1 : g.base;
+    const int cells = cells_or_refused(a, g);
     g.base = 0;
     a.sync[BUILD_ROWS] = (unsigned)(g.dims[1] * g.dims[2]);
     a.sync[BUILD_CURSOR] = 0u;
@@ -238,6 +251,7 @@ __global__ void __launch_bounds__(PREP_T) k_grid_scan(BuildArgs a) {
     grid_dep_trigger();
     grid_dep_wait();
     int cells = 0, cubes = 0;
+    bool none = false;   // some molecule has no grid
     for (int m0 = 0; m0 < a.n_mol; m0 += PREP_T) {
         const int m = m0 + threadIdx.x;
         if (a.cube_limit > 0) {
@@ -245,11 +259,12 @@ __global__ void __launch_bounds__(PREP_T) k_grid_scan(BuildArgs a) {
             block_excl_scan(m < a.n_mol ? a.grids[m].cubes : 0, e, tot);
             cubes += tot;
         }
-        const int v = m < a.n_mol ? a.grids[m].base : 0;
+        const int own = m < a.n_mol ? a.grids[m].base : 0, v = max(own, 0);
+        none |= __syncthreads_or(own < 0) != 0;
         int e, tot;
         block_excl_scan(v, e, tot);
         if (m < a.n_mol) {
-            const bool fits = cells + e + v <= a.max_cells;   // (reported below; an empty grid keeps every index in range)
+            const bool fits = own >= 0 && cells + e + v <= a.max_cells;   // (reported below; an empty grid keeps every index in range)
             a.grids[m].base = fits ? cells + e : 0;
             if (!fits)
                 for (int k = 0; k < 3; ++k) a.grids[m].dims[k] = 0;
@@ -257,7 +272,7 @@ __global__ void __launch_bounds__(PREP_T) k_grid_scan(BuildArgs a) {
         cells += tot;
     }
     if (threadIdx.x == 0) {
-        if (refused(a, cubes)) cells = a.max_cells + 1;
+        if (refused(a, cubes) || none) cells = a.max_cells + 1;
         *a.ncells_out = cells;
         if (cells > a.max_cells) atomicOr(a.status, ST_GRID_OVF);
     }
@@ -402,7 +417,7 @@ __global__ void __launch_bounds__(kSmallT) k_build_small(BuildArgs a) {
     __syncthreads();
     if (tid == 0) {
         MolGrid gg = make_grid(bb, a.n, a.skin, a.cube_limit);
-        const int ncells = refused(a, gg.cubes) ? a.max_cells + 1 : gg.base;
+        const int ncells = cells_or_refused(a, gg);
         gg.base = 0;
         if (ncells > a.max_cells) {   // an empty grid keeps every index in range
             for (int k = 0; k < 3; ++k) gg.dims[k] = 0;
