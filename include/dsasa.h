@@ -273,6 +273,10 @@ int64_t dsasa_kernel_launches(void);
  * DSASA_ERR_OOM and leaves its context usable).  count <= 0 clears it.  Thread-safe. */
 void dsasa_debug_fail_allocations(int count);
 
+/* Test hook (no paper counterpart): leaves the context's cell counts as two calls that overlapped
+ * on it could, before the context's next call.  Enqueues on the context's stream. */
+dsasa_status dsasa_debug_disturb_counts(dsasa_ctx* ctx);
+
 /* Diagnostic export of the dual complex C as seen by each atom's local cell.  For every atom
  * i and every simplex of C that contains i, one record of 5 int32 is written to `records`
  * (device, capacity `max_records`): {i, v0, v1, v2, v3} with the simplex's atom indices in

@@ -64,6 +64,7 @@ _lib.dsasa_kernel_times.argtypes = [_vp, ctypes.POINTER(ctypes.c_double), ctypes
 _lib.dsasa_export_complex.argtypes = [_vp, _vp, _vp, ctypes.c_double, _i64, _vp, _i64, ctypes.POINTER(ctypes.c_int64)]
 _lib.dsasa_last_error.argtypes = [_vp]
 _lib.dsasa_debug_fail_allocations.argtypes = [ctypes.c_int]
+_lib.dsasa_debug_disturb_counts.argtypes = [_vp]
 _lib.dsasa_kernel_launches.argtypes = []
 _lib.dsasa_kernel_launches.restype = ctypes.c_int64
 _lib.dsasa_last_error.restype = ctypes.c_char_p
@@ -84,7 +85,7 @@ EXPORTED = ("dsasa_default_config", "dsasa_create", "dsasa_set_stream", "dsasa_s
             "dsasa_compute_volume_vjp", "dsasa_arena_create", "dsasa_arena_invalidate", "dsasa_arena_destroy",
             "dsasa_compute_batch_resident", "dsasa_batch_reused",
             "dsasa_compute_sr", "dsasa_sr_tests", "dsasa_lists_reused", "dsasa_cells_carried", "dsasa_kernel_launches",
-            "dsasa_debug_fail_allocations")
+            "dsasa_debug_fail_allocations", "dsasa_debug_disturb_counts")
 
 
 class DSASAError(RuntimeError):

@@ -92,7 +92,7 @@ struct dsasa_ctx {
     int* nbn = nullptr;
     double* ref_xyz = nullptr;
     double* ref_rad = nullptr;
-    int* vstate = nullptr;        // [0] max displacement^2 (float bits), [1] radii changed, [2] reuse, [3] overflow, [4] ticket
+    int* vstate = nullptr;        // [2] reuse, [3] overflow, from VSTATE_TEST on the skin test's scratch
     int64_t lists_n = 0;          // the lists hold this many atoms of the last single-molecule call
     double lists_probe = -1.0;
     int* status = nullptr;      // [0] status bits, [1] total cells, [2] deferred count, [3] redo count
@@ -175,15 +175,14 @@ dsasa_status ensure(dsasa_ctx* c, int64_t n, int64_t n_mol) {
     ALLOC(bbox, 8 * nm) ALLOC(grids, nm) ALLOC(counts, ns + 1) ALLOC(cstart, ns + 1) ALLOC(blocksums, (int64_t)scan_scratch_ints((int)ns) + 16)
     ALLOC(offsets, nm + 1) ALLOC(defer, na) ALLOC(redo, na) ALLOC(cells, na * (int64_t)cell_record_bytes()) ALLOC(bsync, BUILD_SYNC_WORDS)
     ALLOC(mol_base, nm) ALLOC(mol_reuse, nm) ALLOC(vmol, 3 * nm + 1) ALLOC(mol_done, nm)
-    // what the kernels expect to be zero, and leave zero
+    // what the kernels expect to be zero, and clear in every call
     e = cudaMemsetAsync(c->bsync, 0, sizeof(unsigned) * BUILD_SYNC_WORDS, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->bbox, 0, sizeof(unsigned) * 8 * (size_t)nm, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->counts, 0, sizeof(int) * (size_t)(ns + 1), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->vmol, 0, sizeof(int) * (3 * (size_t)nm + 1), c->stream);
     if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "memset"); }
     if (c->cfg.skin > 0.0) {
-        ALLOC(nbl, na * NBL_CAP) ALLOC(nbn, na) ALLOC(ref_xyz, 3 * na) ALLOC(ref_rad, na) ALLOC(vstate, 8)
-        e = cudaMemsetAsync(c->vstate, 0, 8 * sizeof(int), c->stream);
+        ALLOC(nbl, na * NBL_CAP) ALLOC(nbn, na) ALLOC(ref_xyz, 3 * na) ALLOC(ref_rad, na) ALLOC(vstate, VSTATE_WORDS)
+        e = cudaMemsetAsync(c->vstate, 0, VSTATE_WORDS * sizeof(int), c->stream);
         if (e != cudaSuccess) { free_scratch(c); return cuda_fail(c, e, "memset"); }
     }
 #undef ALLOC
@@ -199,9 +198,11 @@ dsasa_status ensure(dsasa_ctx* c, int64_t n, int64_t n_mol) {
 // the cell list of the inputs in the context's scratch (enqueued on its stream)
 cudaError_t build_cells(dsasa_ctx* c, const double* coords, const double* radii, double probe, int64_t n, int n_mol,
                         const long long* offsets_dev, const int* skip = nullptr,
-                        int* zero_word = nullptr) {
+                        int* zero_word = nullptr, int* test_words = nullptr, int test_n = 0) {
     BuildArgs b{};
     b.skip = skip;
+    b.test_words = test_words;
+    b.test_n = test_n;
     b.xyz = coords;
     b.radii = radii;
     b.probe = probe;
@@ -241,8 +242,10 @@ dsasa_status run(dsasa_ctx* c, const double* coords, const double* radii, double
         if (ev_e != cudaSuccess) return cuda_fail(c, ev_e, "Verlet check launch");
     }
     // the build also clears the deferred-atom count of the atom kernels that follow it
+    // and the scratch of the skin test before it
+    int* const test = lists ? c->vstate + VSTATE_TEST : (bx.arena ? c->vmol : nullptr);
     cudaError_t e = build_cells(c, coords, radii, probe, n, n_mol, offsets_dev, lists ? c->vstate + 2 : nullptr,
-                                c->status + 2);
+                                c->status + 2, test, lists ? VSTATE_TEST_N : 1 + 3 * n_mol);
     if (e != cudaSuccess) return cuda_fail(c, e, "cell-list launch");
     if (ev) cudaEventRecord(ev[1], c->stream);
     AtomArgs a{};
@@ -600,8 +603,7 @@ dsasa_status dsasa_compute_batch_resident(dsasa_ctx* c, dsasa_arena* arena, int 
                             c->stream);
         if (e == cudaSuccess)
             e = launch_verlet_check_batch(coords, radii, arena->ref_xyz, arena->ref_rad, arena->nbn, c->offsets,
-                                          c->mol_base, (int)n, n_mol, c->cfg.skin, c->vmol,
-                                          (unsigned*)c->vmol + 3 * c->cap_mol, c->mol_reuse, c->stream);
+                                          c->mol_base, (int)n, n_mol, c->cfg.skin, c->vmol, c->mol_reuse, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "resident list check");
         bx.arena = arena;
     }
@@ -745,6 +747,14 @@ dsasa_status dsasa_export_complex(dsasa_ctx* c, const double* coords, const doub
 const char* dsasa_last_error(const dsasa_ctx* c) { return c ? c->err : "null context"; }
 
 int64_t dsasa_kernel_launches(void) { return g_launches.load(std::memory_order_relaxed); }
+
+dsasa_status dsasa_debug_disturb_counts(dsasa_ctx* c) {
+    if (!c) return DSASA_ERR_ARG;
+    cudaError_t e = cudaSetDevice(c->device);
+    if (e == cudaSuccess && c->counts)
+        e = cudaMemsetAsync(c->counts, 1, sizeof(int) * (size_t)(c->store_cells + 1), c->stream);
+    return e == cudaSuccess ? DSASA_OK : cuda_fail(c, e, "memset");
+}
 
 void dsasa_debug_fail_allocations(int count) { g_fail_allocs.store(count > 0 ? count : 0); }
 

@@ -145,6 +145,20 @@ __device__ __forceinline__ int cells_or_refused(const BuildArgs& a, const MolGri
 
 constexpr int PREP_T = 256;
 
+// the words that must be zero later in this call (thread t of nt): the counts of the cells that the
+// grids can have (8 per atom and 64 per molecule) ...
+__device__ __forceinline__ void clear_counts(const BuildArgs& a, int t, int nt) {
+    const int words = min(8 * a.n + 64 * a.n_mol, a.max_cells);
+    for (int k = t; k < words / 4; k += nt) ((int4*)a.counts)[k] = make_int4(0, 0, 0, 0);
+    if (t < words % 4) a.counts[words - 1 - t] = 0;
+}
+// ... and, for the next calls, the skin test's scratch, and the deferred counts of the atom kernels
+__device__ __forceinline__ void clear_words(const BuildArgs& a, int t, int nt) {
+    if (a.test_words)
+        for (int k = t; k < a.test_n; k += nt) a.test_words[k] = 0;
+    if (t < 2 && a.zero_word) a.zero_word[t] = 0;
+}
+
 // exclusive sum of v over the block's threads (in thread order) and the total
 __device__ void block_excl_scan(int v, int& ev, int& tv) {
     __shared__ int sv[PREP_T / 32];
@@ -166,17 +180,17 @@ __device__ void block_excl_scan(int v, int& ev, int& tv) {
     __syncthreads();
 }
 
-// Input pass and bounding boxes.  GRIDS: the block that finishes last makes the grid, and clears
-// the box and the ticket for the next call.
+// Input pass and bounding boxes.  GRIDS: the block that finishes last makes the grid.
 template <bool GRIDS>
 __global__ void __launch_bounds__(PREP_T) k_prep(BuildArgs a) {
     grid_dep_trigger();
     grid_dep_wait();
-    if (GRIDS && blockIdx.x == 0 && threadIdx.x == 0 && a.zero_word) { a.zero_word[0] = 0; a.zero_word[1] = 0; }
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (GRIDS && blockIdx.x == 0) clear_words(a, tid, PREP_T);
     if (a.skip && *a.skip) return;
+    clear_counts(a, blockIdx.x * PREP_T + tid, gridDim.x * PREP_T);
     __shared__ unsigned bb[7];
     __shared__ bool last;
-    const int tid = threadIdx.x, lane = tid & 31;
     if (tid < 7) bb[tid] = 0;
     __syncthreads();
     const int i0 = blockIdx.x * PREP_T, i = i0 + tid;
@@ -209,16 +223,12 @@ __global__ void __launch_bounds__(PREP_T) k_prep(BuildArgs a) {
     if (!last || tid != 0) return;
     __threadfence();
     unsigned bx[7];
-    for (int k = 0; k < 7; ++k) {
-        bx[k] = __ldcg(a.bbox + k);
-        a.bbox[k] = 0;
-    }
+    for (int k = 0; k < 7; ++k) bx[k] = __ldcg(a.bbox + k);
     MolGrid g = make_grid(bx, a.n, a.skin, a.cube_limit);
     const int cells = cells_or_refused(a, g);
     g.base = 0;
     a.sync[BUILD_ROWS] = (unsigned)(g.dims[1] * g.dims[2]);
     a.sync[BUILD_CURSOR] = 0u;
-    a.sync[BUILD_TICKET] = 0u;
     *a.ncells_out = cells;
     if (cells > a.max_cells) {   // an empty grid keeps every index in range
         for (int k = 0; k < 3; ++k) g.dims[k] = 0;
@@ -227,11 +237,11 @@ __global__ void __launch_bounds__(PREP_T) k_prep(BuildArgs a) {
     a.grids[0] = g;
 }
 
-// batches: the boxes and the atom kernels' counts cleared
+// batches: the boxes and the words of clear_words cleared
 __global__ void k_bbox_init(BuildArgs a) {
     grid_dep_trigger();
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m == 0 && a.zero_word) { a.zero_word[0] = 0; a.zero_word[1] = 0; }
+    clear_words(a, m, gridDim.x * blockDim.x);
     if (m >= a.n_mol) return;
     for (int k = 0; k < 8; ++k) a.bbox[8 * m + k] = 0;
 }
@@ -243,7 +253,6 @@ __global__ void k_grid_local(BuildArgs a) {
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= a.n_mol) return;
     a.grids[m] = make_grid(a.bbox + 8 * m, a.offsets[m + 1] - a.offsets[m], a.skin, a.cube_limit);
-    for (int k = 0; k < 8; ++k) a.bbox[8 * m + k] = 0;
 }
 
 // batches: the first cell of each molecule (one block)
@@ -278,12 +287,17 @@ __global__ void __launch_bounds__(PREP_T) k_grid_scan(BuildArgs a) {
     }
 }
 
-// each atom's cell and its rank there (the counts are zero when this starts)
+// each atom's cell and its rank there; the single-molecule build's box and ticket are zero again
+// afterwards
 __global__ void k_count(BuildArgs a) {
     grid_dep_trigger();
     grid_dep_wait();
     if (a.skip && *a.skip) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x < 8) a.bbox[threadIdx.x] = 0;
+        if (threadIdx.x == 8) a.sync[BUILD_TICKET] = 0u;
+    }
     if (i >= a.n || *a.ncells_out > a.max_cells) return;
     const MolGrid g = a.grids[a.molid[i]];
     const int c = cell_of(g, a.f4[i]);
@@ -291,8 +305,7 @@ __global__ void k_count(BuildArgs a) {
     a.rank[i] = atomicAdd(&a.counts[c], 1);
 }
 
-// one molecule: the starts of every row's cells, one warp per row; the counts are zero again
-// afterwards
+// one molecule: the starts of every row's cells, one warp per row
 __global__ void __launch_bounds__(256) k_rows(BuildArgs a) {
     grid_dep_trigger();
     grid_dep_wait();
@@ -317,14 +330,12 @@ __global__ void __launch_bounds__(256) k_rows(BuildArgs a) {
                 if (lane >= o) y += p;
             }
             if (x <= d0) a.cstart[c0 + x] = pos + y - v;
-            if (x < d0) a.counts[c0 + x] = 0;
             pos += __shfl_sync(0xffffffffu, y, 31);
         }
     }
 }
 
-// batches: exclusive scan of the counts of the cells in use into cstart (three kernels; the counts
-// are zero again afterwards)
+// batches: exclusive scan of the counts of the cells in use into cstart (three kernels)
 constexpr int SCAN_V = 16, SCAN_TILE = PREP_T * SCAN_V;
 __global__ void __launch_bounds__(PREP_T) k_scan_reduce(BuildArgs a, int* bsum) {
     grid_dep_trigger();
@@ -362,10 +373,7 @@ __global__ void __launch_bounds__(PREP_T) k_scan_down(BuildArgs a, const int* bs
     block_excl_scan(s, e, tot);
     int pre = e + bsum[blockIdx.x];
     for (int k = 0; k < SCAN_V; ++k) {
-        if (base + k < used) {
-            a.cstart[base + k] = pre;
-            a.counts[base + k] = 0;
-        }
+        if (base + k < used) a.cstart[base + k] = pre;
         pre += v[k];
     }
 }
@@ -389,7 +397,7 @@ constexpr int kSmallT = 1024, kSmallAtoms = 2 * kSmallT, kSmallCells = 8 * kSmal
 __global__ void __launch_bounds__(kSmallT) k_build_small(BuildArgs a) {
     grid_dep_trigger();
     grid_dep_wait();
-    if (threadIdx.x == 0 && a.zero_word) { a.zero_word[0] = 0; a.zero_word[1] = 0; }
+    clear_words(a, threadIdx.x, kSmallT);
     if (a.skip && *a.skip) return;
     __shared__ unsigned bb[7];
     __shared__ MolGrid g;
@@ -519,22 +527,19 @@ namespace {
 constexpr int CHECK_T = 256;
 
 // whether this block is the last of the grid to come here (every thread's writes before it are
-// visible to the last block after it); the ticket is zero again for the next call
+// visible to the last block after it)
 __device__ bool last_block(unsigned* ticket) {
     __shared__ bool last;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) {
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-        if (last) *ticket = 0;
-    }
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     __syncthreads();
     if (last) __threadfence();
     return last;
 }
 
-// Verlet skin test (see dsasa_kernels.cuh): the largest displacement and any changed radius go
-// to vstate[0..1] (zero between calls); the last block decides and clears them.
+// Verlet skin test (see dsasa_kernels.cuh): the largest displacement, any changed radius and the
+// ticket are the words from VSTATE_TEST on; the last block decides.
 __global__ void __launch_bounds__(CHECK_T) k_verlet_check(const double* xyz, const double* radii, const double* ref_xyz,
                                                           const double* ref_rad, int n, int valid, float lim2, int* vstate,
                                                           AtomD* ad, float4* f4) {
@@ -556,30 +561,30 @@ __global__ void __launch_bounds__(CHECK_T) k_verlet_check(const double* xyz, con
     }
     const unsigned d2max = __reduce_max_sync(0xffffffffu, __float_as_uint(d2));   // d2 >= 0: bits order as values
     changed = __reduce_or_sync(0xffffffffu, changed);
+    int* word = vstate + VSTATE_TEST;
     if ((threadIdx.x & 31) == 0) {
-        if (d2max) atomicMax((unsigned*)&vstate[0], d2max);
-        if (changed) atomicOr(&vstate[1], 1);
+        if (d2max) atomicMax((unsigned*)&word[0], d2max);
+        if (changed) atomicOr(&word[1], 1);
     }
-    if (!last_block((unsigned*)vstate + 4) || threadIdx.x != 0) return;
-    const float dm = __uint_as_float((unsigned)__ldcg(vstate));
-    const int reuse = valid && __ldcg(vstate + 1) == 0 && vstate[3] == 0 && dm <= lim2;
-    vstate[0] = 0;
-    vstate[1] = 0;
+    if (!last_block((unsigned*)word + 2) || threadIdx.x != 0) return;
+    const float dm = __uint_as_float((unsigned)__ldcg(word));
+    const int reuse = valid && __ldcg(word + 1) == 0 && vstate[3] == 0 && dm <= lim2;
     vstate[2] = reuse;
     if (!reuse) vstate[3] = 0;   // the lists are rebuilt by this call
 }
 
 // The same test for a batch of resident molecules, per molecule m (atoms [off[m], off[m+1]),
-// lists at arena slot base[m] + local index; base[m] < 0: no lists): vmol[3m] the largest
-// squared displacement since the lists were built (float bits, rounded up), vmol[3m + 1] a
-// radius changed, vmol[3m + 2] some atom has no valid list (negative length).  vmol and the
-// ticket are zero between calls.
+// lists at arena slot base[m] + local index; base[m] < 0: no lists): words[0] is the ticket; of
+// words 1 + 3m .. 3 + 3m the first is the largest squared displacement since the lists were built
+// (float bits, rounded up), the second says that a radius changed, the third that some atom has no
+// valid list (negative length).
 __global__ void __launch_bounds__(CHECK_T) k_verlet_check_batch(const double* xyz, const double* radii,
                                                                 const double* ref_xyz, const double* ref_rad,
                                                                 const int* nbn, const long long* off,
                                                                 const long long* base, int n, int n_mol, float lim2,
-                                                                int* vmol, unsigned* ticket, int* reuse) {
+                                                                int* words, int* reuse) {
     grid_dep_trigger();
+    int* vmol = words + 1;
     const int i = blockIdx.x * CHECK_T + threadIdx.x;
     int m = -1;
     unsigned d2b = 0;
@@ -609,11 +614,10 @@ __global__ void __launch_bounds__(CHECK_T) k_verlet_check_batch(const double* xy
         if (changed) atomicOr(&vmol[3 * m + 1], 1);
         if (none) atomicOr(&vmol[3 * m + 2], 1);
     }
-    if (!last_block(ticket)) return;
+    if (!last_block((unsigned*)words)) return;
     for (int k = threadIdx.x; k < n_mol; k += CHECK_T) {
         reuse[k] = base[k] >= 0 && __ldcg(vmol + 3 * k + 1) == 0 && __ldcg(vmol + 3 * k + 2) == 0 &&
                    __uint_as_float((unsigned)__ldcg(vmol + 3 * k)) <= lim2;
-        vmol[3 * k] = vmol[3 * k + 1] = vmol[3 * k + 2] = 0;
     }
 }
 
@@ -622,10 +626,10 @@ __global__ void __launch_bounds__(CHECK_T) k_verlet_check_batch(const double* xy
 cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, const double* ref_xyz,
                                       const double* ref_rad, const int* nbn, const long long* off,
                                       const long long* base, int n, int n_mol, double skin, int* vmol,
-                                      unsigned* ticket, int* reuse, cudaStream_t s) {
+                                      int* reuse, cudaStream_t s) {
     const float lim2 = (float)(0.25 * skin * skin) * (1.f - 1e-6f);
     const int nb = n > 0 ? (n + CHECK_T - 1) / CHECK_T : 1;
-    k_verlet_check_batch<<<nb, CHECK_T, 0, s>>>(xyz, radii, ref_xyz, ref_rad, nbn, off, base, n, n_mol, lim2, vmol, ticket, reuse);
+    k_verlet_check_batch<<<nb, CHECK_T, 0, s>>>(xyz, radii, ref_xyz, ref_rad, nbn, off, base, n, n_mol, lim2, vmol, reuse);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -48,8 +48,8 @@ cudaError_t launch_dependent(void (*kernel)(K...), int grid, int block, cudaStre
 // host: adds k to the library-wide count of kernel launches (dsasa_kernel_launches)
 void note_launches(int k);
 
-// words of the single-molecule build's exchange area: the ticket of the input pass (zero between
-// calls), the rows of the grid, and the cursor of the sorted order
+// words of the single-molecule build's exchange area: the ticket of the input pass (zero before a
+// build), the rows of the grid, and the cursor of the sorted order
 enum { BUILD_TICKET = 0, BUILD_ROWS = 1, BUILD_CURSOR = 2, BUILD_SYNC_WORDS = 4 };
 
 // device status bits (ORed by kernels, read by dsasa_status_sync)
@@ -184,6 +184,12 @@ struct BuildArgs {
     const int* skip;   // non-NULL and *skip != 0: the previous cell list is reused (nothing to do)
     int* zero_word;    // non-NULL: zero_word[0..1] set to 0 by the build's first kernel (the next atom
                        // kernels' deferred count, and a spare word)
+    // The words that kernels count up start every call at zero whatever came before: a call that
+    // overlapped another on the same scratch (which no caller may do) spoils itself, not the later
+    // ones.  The counts of the cells are cleared before they are used; the box and the ticket of the
+    // input pass and the skin test's words by a kernel of the same call after it.
+    int* test_words;   // the skin test's scratch (test_n words), set to 0 by the build's first kernel
+    int test_n;
     int max_cells;     // cells (and row ends) that counts and cstart hold
     int cube_limit;    // > 0: more cubic cells than this are refused (cell_store makes room for what they become)
     // outputs / scratch
@@ -195,9 +201,9 @@ struct BuildArgs {
     int* molid;        // n
     int* rank;         // n
     int* cell;         // n
-    unsigned* bbox;    // n_mol * 8, zero between calls (box words, pad)
+    unsigned* bbox;    // n_mol * 8 (box words, pad); molecule 0's are zero before a build
     MolGrid* grids;    // n_mol
-    int* counts;       // max_cells + 1, zero between calls
+    int* counts;       // max_cells + 1, 16-byte aligned
     int* cstart;       // max_cells + 1
     int* sidx;         // n
     float4* sf4;       // n
@@ -302,17 +308,18 @@ struct SRArgs {
 cudaError_t launch_build(const BuildArgs& a, cudaStream_t s);
 // Verlet skin test: vstate[2] = reuse the lists (valid, every atom within skin/2 of its
 // reference position, radii unchanged, no list overflow); the positions go to ad and f4, which a
-// build that is not needed does not write; vstate[3] overflow, the other words
-// scratch (zero between calls; 8 words)
+// build that is not needed does not write; vstate[3] overflow; VSTATE_TEST .. + VSTATE_TEST_N - 1
+// scratch, which starts at zero (BuildArgs.test_words of the build that follows)
+enum { VSTATE_TEST = 4, VSTATE_TEST_N = 3, VSTATE_WORDS = 8 };
 cudaError_t launch_verlet_check(const double* xyz, const double* radii, const double* ref_xyz, const double* ref_rad,
                                 int n, int valid, double skin, int* vstate, AtomD* ad, float4* f4,
                                 cudaStream_t s);
 // the Verlet skin test of a batch of resident molecules: reuse[m] for each molecule (see
-// k_verlet_check_batch); vmol: 3 ints per molecule of scratch, ticket: one more, zero between calls
+// k_verlet_check_batch); vmol: 1 + 3 n_mol ints of scratch, which start at zero
 cudaError_t launch_verlet_check_batch(const double* xyz, const double* radii, const double* ref_xyz,
                                       const double* ref_rad, const int* nbn, const long long* off,
                                       const long long* base, int n, int n_mol, double skin, int* vmol,
-                                      unsigned* ticket, int* reuse, cudaStream_t s);
+                                      int* reuse, cudaStream_t s);
 cudaError_t launch_sr(const SRArgs& a, cudaStream_t s);
 // the classified cell records of every atom (a.cells), for the terms of either precision
 cudaError_t launch_cells(const AtomArgs& a, cudaStream_t s);

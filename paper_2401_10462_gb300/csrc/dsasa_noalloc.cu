@@ -66,14 +66,9 @@ extern "C" dsasa_status dsasa_compute_noalloc(const double* coords, const double
         base = (unsigned char*)p;
     }
     int* status = (int*)(base + OFF_STATUS);
-    // the array keeps the previous call's contents: clear what must start at zero (the status
-    // words and, although the cell-list build leaves them zero, its boxes, counts and ticket:
-    // a call that overlapped this one must not spoil the later ones)
-    static_assert(OFF_SYNC == OFF_STATUS + 256 && OFF_GRID == OFF_BBOX + 256, "cleared together");
-    if (cudaMemsetAsync(status, 0, 256 + sizeof(unsigned) * BUILD_SYNC_WORDS, s) != cudaSuccess ||
-        cudaMemsetAsync(base + OFF_BBOX, 0, 256, s) != cudaSuccess ||
-        cudaMemsetAsync(base + OFF_COUNTS, 0, sizeof(int) * (size_t)(8 * n + 129), s) != cudaSuccess)
-        return DSASA_ERR_CUDA;
+    // the array keeps the previous call's contents: the status words start at zero (the build clears
+    // the rest)
+    if (cudaMemsetAsync(status, 0, sizeof(int) * 4, s) != cudaSuccess) return DSASA_ERR_CUDA;
     BuildArgs b{};
     b.xyz = coords;
     b.radii = radii;
