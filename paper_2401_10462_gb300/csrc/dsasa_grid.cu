@@ -144,6 +144,15 @@ __device__ __forceinline__ int cells_or_refused(const BuildArgs& a, const MolGri
 }
 
 constexpr int PREP_T = 256;
+constexpr int SCAN_V = 16, SCAN_TILE = PREP_T * SCAN_V;   // cells that a thread / a block of a scan takes
+__host__ __device__ constexpr int tiles_of(int cells) { return cells / SCAN_TILE + (cells % SCAN_TILE != 0); }
+
+// Rows of more than LONG_ROW cells (a fibre along x) are not scanned by one warp each but in tiles
+// by whole blocks, whose sums the counting pass gathers.  A warp takes about 0.2 us for 32 cells, so
+// 7 us for the longest row that it gets.  Whole calls on 130,000 atoms in one row, with one warp a
+// row / with tiles: 280,000 cells 2893 / 646 us, a million cells 9297 / 625 us; 5,000 atoms in a row of
+// 11,000 cells 110 / 61 us.
+constexpr int LONG_ROW = 1024;
 
 // the words that must be zero later in this call (thread t of nt): the counts of the cells that the
 // grids can have (8 per atom and 64 per molecule) ...
@@ -151,6 +160,7 @@ __device__ __forceinline__ void clear_counts(const BuildArgs& a, int t, int nt) 
     const int words = min(8 * a.n + 64 * a.n_mol, a.max_cells);
     for (int k = t; k < words / 4; k += nt) ((int4*)a.counts)[k] = make_int4(0, 0, 0, 0);
     if (t < words % 4) a.counts[words - 1 - t] = 0;
+    for (int k = t; k < tiles_of(words); k += nt) a.blocksums[k] = 0;
 }
 // ... and, for the next calls, the skin test's scratch, and the deferred counts of the atom kernels
 __device__ __forceinline__ void clear_words(const BuildArgs& a, int t, int nt) {
@@ -303,18 +313,52 @@ __global__ void k_count(BuildArgs a) {
     const int c = cell_of(g, a.f4[i]);
     a.cell[i] = c;
     a.rank[i] = atomicAdd(&a.counts[c], 1);
+    if (!a.offsets && g.dims[0] > LONG_ROW) {
+        // one molecule with long rows: the sums of the tiles (atoms next to one another often share one)
+        const int lanes = a.n - (i & ~31);
+        const unsigned same = __match_any_sync(lanes >= 32 ? 0xffffffffu : (1u << lanes) - 1u, c / SCAN_TILE);
+        if ((threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(&a.blocksums[c / SCAN_TILE], __popc(same));
+    }
 }
 
-// one molecule: the starts of every row's cells, one warp per row
-__global__ void __launch_bounds__(256) k_rows(BuildArgs a) {
+// the starts of a tile's cells, `before` atoms lying in the tiles before it
+__device__ __forceinline__ void scan_tile(const BuildArgs& a, int tile, int used, int before) {
+    const int base = tile * SCAN_TILE + threadIdx.x * SCAN_V;
+    int v[SCAN_V], s = 0, e, tot;
+    for (int k = 0; k < SCAN_V; ++k) {
+        v[k] = (base + k < used) ? a.counts[base + k] : 0;
+        s += v[k];
+    }
+    block_excl_scan(s, e, tot);
+    int pre = before + e;
+    for (int k = 0; k < SCAN_V; ++k) {
+        if (base + k < used) a.cstart[base + k] = pre;
+        pre += v[k];
+    }
+}
+
+// one molecule: the starts of every row's cells, one warp per row (long rows: one block per tile)
+__global__ void __launch_bounds__(PREP_T) k_rows(BuildArgs a) {
     grid_dep_trigger();
     grid_dep_wait();
     if (a.skip && *a.skip) return;
-    if (*a.ncells_out > a.max_cells) return;
+    const int used = *a.ncells_out;
+    if (used > a.max_cells) return;
+    const int d0 = a.grids[0].dims[0];
+    if (d0 > LONG_ROW) {
+        // (a cell's end is the next one's start, as for a row's last cell the entry after it, which is empty)
+        for (int tile = blockIdx.x; tile < tiles_of(used); tile += gridDim.x) {
+            int s = 0, e, before;
+            for (int k = threadIdx.x; k < tile; k += PREP_T) s += a.blocksums[k];
+            block_excl_scan(s, e, before);
+            scan_tile(a, tile, used, before);
+        }
+        return;
+    }
     const int rows = (int)a.sync[BUILD_ROWS];
     const int lane = threadIdx.x & 31;
-    for (int r = (blockIdx.x * 256 + threadIdx.x) >> 5; r < rows; r += gridDim.x * 8) {
-        const int d0 = a.grids[0].dims[0], c0 = r * (d0 + 1);
+    for (int r = (blockIdx.x * PREP_T + threadIdx.x) >> 5; r < rows; r += gridDim.x * (PREP_T / 32)) {
+        const int c0 = r * (d0 + 1);
         int tot = 0;
         for (int x = lane; x < d0; x += 32) tot += a.counts[c0 + x];
         tot = __reduce_add_sync(0xffffffffu, tot);
@@ -336,12 +380,11 @@ __global__ void __launch_bounds__(256) k_rows(BuildArgs a) {
 }
 
 // batches: exclusive scan of the counts of the cells in use into cstart (three kernels)
-constexpr int SCAN_V = 16, SCAN_TILE = PREP_T * SCAN_V;
 __global__ void __launch_bounds__(PREP_T) k_scan_reduce(BuildArgs a, int* bsum) {
     grid_dep_trigger();
     grid_dep_wait();
     const int used = min(*a.ncells_out, a.max_cells), base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
-    if (blockIdx.x * SCAN_TILE >= used) return;
+    if (blockIdx.x >= tiles_of(used)) return;
     int s = 0, e, tot;
     for (int k = 0; k < SCAN_V; ++k) s += (base + k < used) ? a.counts[base + k] : 0;
     block_excl_scan(s, e, tot);
@@ -350,7 +393,7 @@ __global__ void __launch_bounds__(PREP_T) k_scan_reduce(BuildArgs a, int* bsum) 
 __global__ void __launch_bounds__(PREP_T) k_scan_top(BuildArgs a, int* bsum) {
     grid_dep_trigger();
     grid_dep_wait();
-    const int nb = (min(*a.ncells_out, a.max_cells) + SCAN_TILE - 1) / SCAN_TILE;
+    const int nb = tiles_of(min(*a.ncells_out, a.max_cells));
     int carry = 0;
     for (int b0 = 0; b0 < nb; b0 += PREP_T) {
         const int b = b0 + threadIdx.x;
@@ -363,19 +406,8 @@ __global__ void __launch_bounds__(PREP_T) k_scan_top(BuildArgs a, int* bsum) {
 __global__ void __launch_bounds__(PREP_T) k_scan_down(BuildArgs a, const int* bsum) {
     grid_dep_trigger();
     grid_dep_wait();
-    const int used = min(*a.ncells_out, a.max_cells), base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_V;
-    if (blockIdx.x * SCAN_TILE >= used) return;
-    int v[SCAN_V], s = 0, e, tot;
-    for (int k = 0; k < SCAN_V; ++k) {
-        v[k] = (base + k < used) ? a.counts[base + k] : 0;
-        s += v[k];
-    }
-    block_excl_scan(s, e, tot);
-    int pre = e + bsum[blockIdx.x];
-    for (int k = 0; k < SCAN_V; ++k) {
-        if (base + k < used) a.cstart[base + k] = pre;
-        pre += v[k];
-    }
+    const int used = min(*a.ncells_out, a.max_cells);
+    if (blockIdx.x < tiles_of(used)) scan_tile(a, blockIdx.x, used, bsum[blockIdx.x]);
 }
 
 __global__ void k_scatter(BuildArgs a) {
@@ -520,7 +552,7 @@ cudaError_t launch_build_batch(const BuildArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-size_t scan_scratch_ints(int max_cells) { return (size_t)(max_cells + SCAN_TILE - 1) / SCAN_TILE + 1; }
+size_t scan_scratch_ints(int max_cells) { return (size_t)tiles_of(max_cells) + 1; }
 
 namespace {
 

@@ -207,7 +207,7 @@ struct BuildArgs {
     int* cstart;       // max_cells + 1
     int* sidx;         // n
     float4* sf4;       // n
-    int* blocksums;    // scan scratch (batches)
+    int* blocksums;    // scan_scratch_ints(max_cells): atoms in each run of SCAN_TILE cells (batches; long rows)
     unsigned* sync;    // BUILD_SYNC_WORDS
     int* status;
     int* ncells_out;   // device int: total cells used

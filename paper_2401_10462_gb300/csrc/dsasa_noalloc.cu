@@ -37,7 +37,8 @@ constexpr size_t OFF_BBOX = al(OFF_SF4 + sizeof(float4) * kMaxAtoms);
 constexpr size_t OFF_GRID = al(OFF_BBOX + sizeof(unsigned) * 8);
 constexpr size_t OFF_COUNTS = al(OFF_GRID + sizeof(MolGrid));
 constexpr size_t OFF_CSTART = al(OFF_COUNTS + sizeof(int) * (kMaxCells + 1));
-constexpr size_t OFF_DEFER = al(OFF_CSTART + sizeof(int) * (kMaxCells + 1));
+constexpr size_t OFF_SUMS = al(OFF_CSTART + sizeof(int) * (kMaxCells + 1));
+constexpr size_t OFF_DEFER = al(OFF_SUMS + sizeof(int) * 128);
 constexpr size_t OFF_STATUS = al(OFF_DEFER + sizeof(int) * kMaxAtoms);
 constexpr size_t OFF_SYNC = al(OFF_STATUS + sizeof(int) * 4);
 constexpr size_t kScratchBytes = al(OFF_SYNC + sizeof(unsigned) * BUILD_SYNC_WORDS);
@@ -52,6 +53,7 @@ extern "C" dsasa_status dsasa_compute_noalloc(const double* coords, const double
     if (n == 0) return DSASA_OK;
     if (!coords || !radii || !areas_out) return DSASA_ERR_ARG;
     if (n > kMaxAtoms) return DSASA_ERR_CAPACITY;   // more atoms than the static scratch holds
+    if ((long long)scan_scratch_ints((int)kMaxCells) > 128) return DSASA_ERR_CAPACITY;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     // The host-side name of the array is only a stand-in; its device address belongs to the
     // CUDA context that is current now (it changes after a device reset or under another
@@ -92,6 +94,7 @@ extern "C" dsasa_status dsasa_compute_noalloc(const double* coords, const double
     b.grids = (MolGrid*)(base + OFF_GRID);
     b.counts = (int*)(base + OFF_COUNTS);
     b.cstart = (int*)(base + OFF_CSTART);
+    b.blocksums = (int*)(base + OFF_SUMS);
     b.sync = (unsigned*)(base + OFF_SYNC);
     b.zero_word = status + 2;   // the deferred count of the atom kernels (and a spare word)
     b.status = status;
