@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 
 import numpy as np
 
@@ -139,6 +140,9 @@ class Context:
             raise DSASAError(st, "dsasa_create failed")
         self._h = h
         self._stream = stream
+        self._lock = threading.Lock()   # held by each call: two threads' calls come one after the other
+        self._bound = None              # stream handle that the library enqueues on
+        self._last = None               # stream of the last call that was not captured
 
     @staticmethod
     def _stream_handle(stream):
@@ -150,8 +154,28 @@ class Context:
         return stream.cuda_stream
 
     def _sync_stream(self):
-        if self._stream is None:
-            _lib.dsasa_set_stream(self._h, _vp(self._stream_handle(None)))
+        """A context without a stream of its own follows torch's current stream.  Its calls share one
+        scratch, so a call on another stream than the one before waits for that one's work.  (Not
+        ordered: calls captured in a graph, whose replays the caller orders, and calls on a stream that
+        torch does not own, which may no longer exist at the next call.)"""
+        if self._stream is not None:
+            return
+        import torch
+        cur = torch.cuda.current_stream()
+        handle = cur.cuda_stream
+        if handle == self._bound:
+            return
+        _lib.dsasa_set_stream(self._h, _vp(handle))
+        if torch.cuda.is_current_stream_capturing():
+            self._bound = None
+            return
+        last, self._last, self._bound = self._last, cur, handle
+        torch_owns = last is not None and (last.cuda_stream == 0 or last.stream_id & 1)   # (others: even ids)
+        if torch_owns and last.cuda_stream != handle:
+            with torch.cuda.stream(last):
+                capturing = torch.cuda.is_current_stream_capturing()
+            if not capturing:
+                cur.wait_stream(last)
 
     def _raise(self, st):
         if st != DSASA_OK:
@@ -171,9 +195,10 @@ class Context:
             _check_tensor(grad_out, "grad_out", n, 3)
         if weights is not None:
             _check_tensor(weights, "weights", n)
-        self._sync_stream()
-        self._raise(_lib.dsasa_compute_vjp(self._h, _ptr(coords), _ptr(radii), float(probe), n, _ptr(weights),
-                                           _ptr(areas_out), _ptr(grad_out)))
+        with self._lock:
+            self._sync_stream()
+            self._raise(_lib.dsasa_compute_vjp(self._h, _ptr(coords), _ptr(radii), float(probe), n, _ptr(weights),
+                                               _ptr(areas_out), _ptr(grad_out)))
 
     def compute_volume(self, coords, radii, areas_out, volumes_out, grad_out=None, vol_grad_out=None,
                        probe: float = PROBE):
@@ -188,9 +213,10 @@ class Context:
             _check_tensor(grad_out, "grad_out", n, 3)
         if vol_grad_out is not None:
             _check_tensor(vol_grad_out, "vol_grad_out", n, 3)
-        self._sync_stream()
-        self._raise(_lib.dsasa_compute_volume(self._h, _ptr(coords), _ptr(radii), float(probe), n, _ptr(areas_out),
-                                              _ptr(grad_out), _ptr(volumes_out), _ptr(vol_grad_out)))
+        with self._lock:
+            self._sync_stream()
+            self._raise(_lib.dsasa_compute_volume(self._h, _ptr(coords), _ptr(radii), float(probe), n, _ptr(areas_out),
+                                                  _ptr(grad_out), _ptr(volumes_out), _ptr(vol_grad_out)))
 
     def compute_volume_vjp(self, coords, radii, weights, areas_out, volumes_out, vol_grad_out,
                            probe: float = PROBE):
@@ -204,9 +230,11 @@ class Context:
         _check_tensor(vol_grad_out, "vol_grad_out", n, 3)
         if weights is not None:
             _check_tensor(weights, "weights", n)
-        self._sync_stream()
-        self._raise(_lib.dsasa_compute_volume_vjp(self._h, _ptr(coords), _ptr(radii), float(probe), n, _ptr(weights),
-                                                  _ptr(areas_out), _ptr(volumes_out), _ptr(vol_grad_out)))
+        with self._lock:
+            self._sync_stream()
+            self._raise(_lib.dsasa_compute_volume_vjp(self._h, _ptr(coords), _ptr(radii), float(probe), n,
+                                                      _ptr(weights), _ptr(areas_out), _ptr(volumes_out),
+                                                      _ptr(vol_grad_out)))
 
     def compute_sr(self, coords, radii, unit_points, areas_out, exposed_out=None, probe: float = PROBE):
         """dsasa_compute_sr: Shrake-Rupley areas on the m float32 unit vectors unit_points
@@ -220,9 +248,10 @@ class Context:
             raise ValueError("unit_points must be a contiguous float32 CUDA tensor (m, 3)")
         if exposed_out is not None and (exposed_out.dtype != torch.int32 or exposed_out.numel() != n):
             raise ValueError("exposed_out must be int32 with n entries")
-        self._sync_stream()
-        self._raise(_lib.dsasa_compute_sr(self._h, _ptr(coords), _ptr(radii), float(probe), n, _ptr(unit_points),
-                                          int(unit_points.shape[0]), _ptr(areas_out), _ptr(exposed_out)))
+        with self._lock:
+            self._sync_stream()
+            self._raise(_lib.dsasa_compute_sr(self._h, _ptr(coords), _ptr(radii), float(probe), n, _ptr(unit_points),
+                                              int(unit_points.shape[0]), _ptr(areas_out), _ptr(exposed_out)))
 
     def lists_reused(self) -> bool:
         """Whether the last call reused the Verlet lists (contexts with skin > 0)."""
@@ -249,10 +278,11 @@ class Context:
         _check_tensor(coords, "coords", n, 3)
         _check_tensor(radii, "radii", n)
         _check_tensor(areas_out, "areas_out", n)
-        self._sync_stream()
-        self._raise(_lib.dsasa_compute_batch(self._h, len(off) - 1, off.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)),
-                                             _ptr(coords), _ptr(radii), float(probe), _ptr(weights), _ptr(areas_out),
-                                             _ptr(grad_out)))
+        with self._lock:
+            self._sync_stream()
+            self._raise(_lib.dsasa_compute_batch(
+                self._h, len(off) - 1, off.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), _ptr(coords), _ptr(radii),
+                float(probe), _ptr(weights), _ptr(areas_out), _ptr(grad_out)))
 
     def compute_batch_resident(self, offsets, coords, radii, areas_out, grad_out=None, arena=None,
                                arena_base=None, mol_ready=None, weights=None, probe: float = PROBE):
@@ -267,12 +297,13 @@ class Context:
             base = np.ascontiguousarray(arena_base, dtype=np.int64)
             if base.shape != (n_mol,):
                 raise ValueError("arena_base needs one entry per molecule")
-        self._sync_stream()
         p64 = ctypes.POINTER(ctypes.c_int64)
-        self._raise(_lib.dsasa_compute_batch_resident(
-            self._h, arena._h if arena is not None else None, n_mol, off.ctypes.data_as(p64),
-            base.ctypes.data_as(p64) if base is not None else None, _ptr(coords), _ptr(radii), float(probe),
-            _ptr(weights), _ptr(areas_out), _ptr(grad_out), _ptr(mol_ready)))
+        with self._lock:
+            self._sync_stream()
+            self._raise(_lib.dsasa_compute_batch_resident(
+                self._h, arena._h if arena is not None else None, n_mol, off.ctypes.data_as(p64),
+                base.ctypes.data_as(p64) if base is not None else None, _ptr(coords), _ptr(radii), float(probe),
+                _ptr(weights), _ptr(areas_out), _ptr(grad_out), _ptr(mol_ready)))
 
     def batch_reused(self, n_mol: int) -> np.ndarray:
         """Per molecule of the last resident batch: whether its lists were reused."""
@@ -297,9 +328,10 @@ class Context:
                 if arr is not None and (arr.dtype != np.float64 or arr.shape != shape or not arr.flags.c_contiguous
                                         or not arr.flags.writeable):
                     raise ValueError(f"out arrays must be writeable C-contiguous float64 of shape {shape}")
-        self._sync_stream()
         dp = lambda x: None if x is None else x.ctypes.data   # the address (cheaper than data_as)
-        self._raise(_lib.dsasa_compute_host(self._h, dp(xyz), dp(r), float(probe), n, dp(w), dp(a), dp(g)))
+        with self._lock:
+            self._sync_stream()
+            self._raise(_lib.dsasa_compute_host(self._h, dp(xyz), dp(r), float(probe), n, dp(w), dp(a), dp(g)))
         return a, g
 
     def status_sync(self):
@@ -335,10 +367,11 @@ class Context:
         cap = max_records or 64 * n + 64
         rec = torch.empty((cap, 5), dtype=torch.int32, device=coords.device)
         cnt = ctypes.c_int64(0)
-        self._sync_stream()
-        st = _lib.dsasa_export_complex(self._h, _ptr(coords), _ptr(radii), float(probe), n, _ptr(rec), cap,
-                                       ctypes.byref(cnt))
-        self._raise(st)
+        with self._lock:
+            self._sync_stream()
+            st = _lib.dsasa_export_complex(self._h, _ptr(coords), _ptr(radii), float(probe), n, _ptr(rec), cap,
+                                           ctypes.byref(cnt))
+            self._raise(st)
         return rec[: cnt.value]
 
     def close(self):
