@@ -768,7 +768,11 @@ __device__ __noinline__ bool clip_rest(SM* S, const AtomArgs& A, int i, int nc, 
                 if ((int)st.TV[r] < 0 && clip_sign(S, A.xyz, A.R, i, A.n, A.status, st.TV[r], m) > 0) remv |= 1u << r;
         }
         const int c = st.cut(S, m, remv, lane);
-        if (c == CUT_EMPTY) return true;
+        if (c == CUT_EMPTY) {   // (no slot may look alive to the caller)
+#pragma unroll
+            for (int r = 0; r < NR; ++r) st.TV[r] = 0;
+            break;
+        }
         if (c == CUT_FULL) {
             if (lane == 0) S->bad = 2;
             break;
@@ -781,7 +785,7 @@ __device__ __noinline__ bool clip_rest(SM* S, const AtomArgs& A, int i, int nc, 
     }
     if (lane == 0) S->hw = st.hw;
     __syncwarp();
-    return false;
+    return st.nothing;
 }
 
 // ------------------------------------------------------------------ carried cells
