@@ -278,11 +278,15 @@ template <class N> DS_HD N pred_edge_beyond(const PlaneN<N>& A, const PlaneN<N>&
 
 // ------------------------------------------------------------------ plane construction
 // Ghost planes bound the initial cell: a cube of half-width h around p_i, h >= R_i * 1.0625
-// with at most 24 significant bits so that 2h and 2h^2 are exact doubles (and 2h an exact
-// float).  Ghost g in 0..5: +x, -x, +y, -y, +z, -z.
+// with at most 24 significant bits so that 2h and 2h^2 are exact doubles (and h and 2h exact
+// floats: the filters' planes and the exact predicates' are the same cube).  Ghost g in 0..5: +x,
+// -x, +y, -y, +z, -z.
 DS_HD double ghost_h(double Ri) {
     double h = Ri * 1.0625 + 0.0625;
-    return ceil(h * 1048576.0) / 1048576.0;   // multiple of 2^-20 (< 2^4): <= 24 bits
+    h = ceil(h * 1048576.0) / 1048576.0;   // multiple of 2^-20: <= 24 bits below 2^4
+    float f = (float)h;                    // from 2^4 on: the next float
+    if ((double)f < h) f = nextafterf(f, INFINITY);
+    return f <= 3.4028234e38f ? (double)f : h;   // (beyond the floats nothing is exact)
 }
 DS_HD void ghost_plane64(int g, double h, double q[3], double& b) {
     q[0] = q[1] = q[2] = 0.0;
