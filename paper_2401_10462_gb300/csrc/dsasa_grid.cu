@@ -50,7 +50,7 @@ __device__ __forceinline__ float4 prep_atom(const BuildArgs& a, int i, int m) {
     const float h = (float)R;
     a.Rhl[i] = make_float2(h, (float)(R - (double)h));
     a.ad[i] = AtomD{x, y, z, R};
-    a.gh[i] = (float)ghost_h(R);
+    a.gh[i] = ghost_hf(R);
     a.molid[i] = m;
     const float4 f = make_float4((float)x, (float)y, (float)z, h);
     a.f4[i] = f;

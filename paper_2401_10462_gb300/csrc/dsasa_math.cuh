@@ -281,13 +281,16 @@ template <class N> DS_HD N pred_edge_beyond(const PlaneN<N>& A, const PlaneN<N>&
 // with at most 24 significant bits so that 2h and 2h^2 are exact doubles (and h and 2h exact
 // floats: the filters' planes and the exact predicates' are the same cube).  Ghost g in 0..5: +x,
 // -x, +y, -y, +z, -z.
-DS_HD double ghost_h(double Ri) {
-    double h = Ri * 1.0625 + 0.0625;
-    h = ceil(h * 1048576.0) / 1048576.0;   // multiple of 2^-20: <= 24 bits below 2^4
-    float f = (float)h;                    // from 2^4 on: the next float
-    if ((double)f < h) f = nextafterf(f, INFINITY);
-    return f <= 3.4028234e38f ? (double)f : h;   // (beyond the floats nothing is exact)
+DS_HD float ghost_hf(double Ri) {
+    const double h = ceil((Ri * 1.0625 + 0.0625) * 1048576.0) / 1048576.0;   // multiple of 2^-20: <= 24 bits below 2^4
+#if defined(__CUDA_ARCH__)
+    return __double2float_ru(h);   // from 2^4 on: the next float
+#else
+    const float f = (float)h;
+    return (double)f < h ? nextafterf(f, INFINITY) : f;
+#endif
 }
+DS_HD double ghost_h(double Ri) { return (double)ghost_hf(Ri); }
 DS_HD void ghost_plane64(int g, double h, double q[3], double& b) {
     q[0] = q[1] = q[2] = 0.0;
     q[g >> 1] = (g & 1) ? -2.0 * h : 2.0 * h;
