@@ -312,7 +312,7 @@ __device__ __noinline__ int resolve_exact(const Ctx& c, int kind, int g0, int g1
     XP v = eval_kind(kind, P, wi);
     if (v.ovf) {
         atomicOr(c.status, ST_UNRESOLVED);
-        return v.n ? (v.c[v.n - 1] > 0 ? 1 : -1) : 0;
+        return v.n ? (v.c[v.n - 1] > 0 ? 2 : -2) : 0;   // (not +-1: a guess)
     }
     int s = xp_sign(v);
     if (s == 0 && kind == PK_CLIP) {
@@ -740,15 +740,35 @@ template <class R, int NR> struct ClipState {
     }
 };
 
+// The structure of a cell is checked where a sign was a guess: only an expansion past its capacity or a
+// tie that no perturbation breaks can make signs that contradict one another, and leave a cell whose
+// faces do not close (bad: 3, else 0).  (In the classification, for every cell, it cost 2.4 % of a
+// 1,000,000-atom call; here, out of line, 0.9 %.)
+template <class SM> __device__ __noinline__ void check_cell(SM* S) {
+    const int lane = threadIdx.x & 31, hw = S->hw;
+    bool agree = true;
+    for (int t = lane; t < hw; t += 32) {
+        const uchar4 v = S->tv[t], a = S->ta[t];
+        if (v.x == NONE) continue;
+        for (int k = 0; k < 3; ++k) {
+            const int t2 = tv_get(a, k);
+            if (t2 >= hw) agree = false;
+            else {
+                const uchar4 w = S->tv[t2], b = S->ta[t2];
+                agree = agree && edge_agrees(pack3(v.x, v.y, v.z), pack3(w.x, w.y, w.z), pack3(b.x, b.y, b.z), t, k);
+            }
+        }
+    }
+    agree = __all_sync(FULL, agree);
+    if (lane == 0) S->bad = agree ? 0 : 3;
+    __syncwarp();
+}
+
 // The clipping of a cell by planes kk .. nc - 1 with every slot of the table, tests that the filter
 // leaves open resolved exactly.  In: slots 0 - 31 in tv and ta (kf: alive; a dead slot's tv holds its
 // place in the free stack), sp and hw.  Out: tv and ta of every slot, hw, bad (2: no slot free, 3: the
-// cell is inconsistent).  Returns whether the cell is empty.  Out of line: rare, and apart from the
-// registers of the loop it is called after.
-// The structure of a cell is checked where a test was resolved: the filters' signs are certified, so
-// only an expansion past its capacity or a tie that no perturbation breaks can make signs that
-// contradict one another, and leave a cell whose faces do not close.  (In the classification, for
-// every cell, the check cost 2.4 % of a 1,000,000-atom call.)
+// cell is inconsistent; 1 in between: a sign was a guess).  Returns whether the cell is empty.  Out
+// of line: rare, and apart from the registers of the loop it is called after.
 template <class SM, class R = typename SM::Real>
 __device__ __noinline__ bool clip_rest(SM* S, const AtomArgs& A, int i, int nc, int kk, int sp, int hw) {
     constexpr int NR = SM::kNT / 32;
@@ -764,22 +784,27 @@ __device__ __noinline__ bool clip_rest(SM* S, const AtomArgs& A, int i, int nc, 
         if (S->kf[lane]) st.vertex(S, 0);
     }
     __syncwarp();
-    bool resolved = false;
     for (; kk < nc; ++kk) {
         const int m = NG + kk;
         unsigned remv;
         if (st.test(S, m, remv)) {
-            resolved = true;
             remv = 0;
 #pragma unroll
-            for (int r = 0; r < NR; ++r)
-                if ((int)st.TV[r] < 0 && clip_sign(S, A.xyz, A.R, i, A.n, A.status, st.TV[r], m) > 0) remv |= 1u << r;
+            for (int r = 0; r < NR; ++r) {
+                if ((int)st.TV[r] >= 0) continue;
+                const int sg = clip_sign(S, A.xyz, A.R, i, A.n, A.status, st.TV[r], m);
+                if (sg > 0) remv |= 1u << r;
+                if (sg != 1 && sg != -1) S->bad = 1;
+            }
         }
         const int c = st.cut(S, m, remv, lane);
+        if (c != CUT_DONE) __syncwarp();
         if (c == CUT_EMPTY) {   // (no slot may look alive to the caller)
 #pragma unroll
-            for (int r = 0; r < NR; ++r) st.TV[r] = 0;
-            break;
+            for (int r = 0; r < NR; ++r) S->tv[r * 32 + lane] = make_uchar4(NONE, NONE, NONE, 0);
+            if (lane == 0) S->hw = S->bad = 0;
+            __syncwarp();
+            return true;
         }
         if (c == CUT_FULL) {
             if (lane == 0) S->bad = 2;
@@ -793,25 +818,8 @@ __device__ __noinline__ bool clip_rest(SM* S, const AtomArgs& A, int i, int nc, 
     }
     if (lane == 0) S->hw = st.hw;
     __syncwarp();
-    if (resolved && S->bad == 0) {
-        bool agree = true;
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            if ((int)st.TV[r] >= 0) continue;
-            for (int k = 0; k < 3; ++k) {
-                const unsigned t2 = (st.TA[r] >> (8 * k)) & 255u;
-                if (t2 >= 32u * NR) {
-                    agree = false;
-                    break;
-                }
-                const uchar4 v = S->tv[t2], w = S->ta[t2];
-                agree = agree && edge_agrees(st.TV[r], pack3(v.x, v.y, v.z), pack3(w.x, w.y, w.z), r * 32 + lane, k);
-            }
-        }
-        if (!__all_sync(FULL, agree) && lane == 0) S->bad = 3;
-        __syncwarp();
-    }
-    return st.nothing;
+    if (S->bad == 1) check_cell(S);
+    return false;
 }
 
 // ------------------------------------------------------------------ carried cells
