@@ -247,7 +247,8 @@ __global__ void __launch_bounds__(PREP_T) k_prep(BuildArgs a) {
     a.grids[0] = g;
 }
 
-// batches: the boxes and the words of clear_words cleared
+// batches: the boxes and the words of clear_words cleared (this call's boxes may lie where another
+// batch, with other molecules, or a single molecule left its own)
 __global__ void k_bbox_init(BuildArgs a) {
     grid_dep_trigger();
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -421,8 +422,10 @@ __global__ void k_scatter(BuildArgs a) {
     a.sf4[pos] = a.f4[i];
 }
 
-// The whole build for one molecule of at most kSmallAtoms atoms in one block (below that size
-// the launches of the four kernels cost more than their width gains).  Same grid, same cells;
+// The whole build for one molecule of at most kSmallAtoms atoms in one block: below that size
+// the launches of the four kernels cost more than their width gains (whole calls, areas + gradient:
+// 2,048 atoms in one block 88 us, 2,049 with the four kernels 93).  The line is where a thread
+// would take a third atom and the counts more than 66 KB of shared memory.  Same grid, same cells;
 // counts in shared memory, starts by one scan over all cells (which also ends every row where
 // the next one starts).
 constexpr int kSmallT = 1024, kSmallAtoms = 2 * kSmallT, kSmallCells = 8 * kSmallAtoms + 64;

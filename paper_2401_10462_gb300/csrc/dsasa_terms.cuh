@@ -13,7 +13,7 @@
 // The lengths |q| of the plane vectors are taken once per plane, not once per term.
 // Mixed form: 20k globule 137 -> 98 us, 5k 42 -> 33.5, 1M shell 5.5 -> 4.1 ms; its loop over the rounds
 // and 18 blocks also fix how its float terms round (without the loop, at 14 - 16 blocks: 84 - 87 us at 20k,
-// areas other by 2e-7).  FP64 form: 5k 717 -> 172 us.
+// areas other by 2e-7).  FP64 form: 5k 717 -> 181 us.
 #pragma once
 #include "dsasa_kernels.cuh"
 #include "dsasa_math.cuh"
