@@ -133,7 +133,7 @@ class ClockSampler:
 def kernel_sha() -> str:
     import hashlib
     h = hashlib.sha256()
-    for f in ("dsasa_atoms.cuh", "dsasa_class.cuh", "dsasa_terms.cuh", "dsasa_math.cuh", "dsasa_kernels.cuh"):
+    for f in ("dsasa_atoms.cuh", "dsasa_cell.cuh", "dsasa_class.cuh", "dsasa_terms.cuh", "dsasa_math.cuh", "dsasa_kernels.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2401_10462_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

@@ -104,7 +104,9 @@ typedef struct {
                          * simplices of the complex are the same as a fresh build's, the areas
                          * and gradient equal up to the rounding of the terms.  0: off; 1
                          * (default): for molecules of more than 36 atoms per
-                         * multiprocessor (5,472 on a GB300), where it pays; 2: always. */
+                         * multiprocessor (5,472 on a GB300); 2: always.  A step of 20,000
+                         * atoms takes 0.348 ms with carried cells, 0.333 ms with lists
+                         * alone and 0.348 ms without lists: 0 is the faster choice there. */
 } dsasa_config;
 
 /* Fills cfg with defaults: MIXED, skin 0, grow on demand, default cell cap, carry 1 (auto). */
